@@ -241,6 +241,18 @@ __device__ __forceinline__ void named_bar_sync(int id, int threads)
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
 
+// True in one lane of a converged warp.  The single threads that issue bulk copies, tensor-map loads and tcgen05
+// instructions are chosen with elect.sync rather than `lane == 0`: the compiler then knows that one thread is active and
+// keeps the operands in uniform registers, where for a lane comparison it emits a loop over the active threads around each
+// such instruction (measured, back-to-back 128 x 16 x 16 MMAs from one thread: 57-91 clocks each after `lane == 0`, 9 after
+// elect.sync; 128 x 256 x 16: 128, the tensor pipe itself).
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.u32 %0, 1, 0, q;\n\t}" : "=r"(p));
+    return p != 0;
+}
+
 // (a & b) | c in one instruction
 __device__ __forceinline__ uint32_t lop3_and_or(uint32_t a, uint32_t b, uint32_t c)
 {

@@ -147,7 +147,7 @@ splitk_kernel(const SplitKArgs a, const __grid_constant__ CUtensorMap x_map)
     const uint32_t bar_empty = smem_base + 64;            // stages x 8 B
     const uint32_t bar_recv = smem_base + 128;
     const uint32_t ring = smem_base + kRingOffset;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // warp: uniform
     const int S = a.S;
     const int p = blockIdx.x / S, rank = blockIdx.x - p * S;   // cluster = the S CTAs of panel p
     const int g0 = rank * a.G / S, g1 = (rank + 1) * a.G / S;  // this CTA's groups
@@ -184,7 +184,7 @@ splitk_kernel(const SplitKArgs a, const __grid_constant__ CUtensorMap x_map)
 
     if (warp == kConsumerWarps) {
         // ------------------------------------------------------------------ producer (one thread)
-        if (lane == 0) {
+        if (elect_one()) {
             const uint64_t policy = l2_policy_evict_first();
             tma_prefetch_descriptor(&x_map);
             const uint32_t meta_bytes = kItemWBytes + SUB * (kItemSBytes + kItemZBytes);

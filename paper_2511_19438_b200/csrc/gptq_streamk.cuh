@@ -165,7 +165,7 @@ streamk_kernel(const StreamKArgs a, const __grid_constant__ CUtensorMap x_map)
     const uint32_t bar_full = smem_base;                  // stages x 8 B
     const uint32_t bar_empty = smem_base + 64;            // stages x 8 B
     const uint32_t ring = smem_base + kRingOffset;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const int C = gridDim.x, c = blockIdx.x;
     const long long T = a.items;
     const int t0 = sk_range_begin(T, C, c), t1 = sk_range_begin(T, C, c + 1);
@@ -186,7 +186,7 @@ streamk_kernel(const StreamKArgs a, const __grid_constant__ CUtensorMap x_map)
 
     if (warp == kConsumerWarps) {
         // ------------------------------------------------------------------ producer (one thread)
-        if (lane != 0) return;
+        if (!elect_one()) return;
         const uint64_t policy = l2_policy_evict_first();
         tma_prefetch_descriptor(&x_map);
         const uint32_t meta_bytes = kItemWBytes + kItemSBytes + kItemZBytes;

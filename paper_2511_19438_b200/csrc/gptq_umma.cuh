@@ -228,7 +228,7 @@ umma_kernel(const UmmaArgs a, const __grid_constant__ CUtensorMap w_map, const _
     const uint32_t bar_full = base, bar_afull = base + 128, bar_done = base + 320;
     const uint32_t bar_dfull = base + 256, tmem_slot = base + 264, bar_recv = base + 272;
     const uint32_t ring = base + 1024;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const int NS = a.stages;
     const int panels = a.N / kPanel;
     const int S = a.S;
@@ -270,7 +270,7 @@ umma_kernel(const UmmaArgs a, const __grid_constant__ CUtensorMap w_map, const _
 
     if (warp == 0) {
         // ---------------------------------------------------------------- TMA producer (one thread)
-        if (lane == 0) {
+        if (elect_one()) {
             tma_prefetch_descriptor(&w_map);
             tma_prefetch_descriptor(&x_map);
             constexpr uint32_t kXBytes = BPS * kXTile;
@@ -316,7 +316,7 @@ umma_kernel(const UmmaArgs a, const __grid_constant__ CUtensorMap w_map, const _
         }
     } else if (warp <= ISS) {
         // ---------------------------------------------------------------- MMA issue (one thread per issuing warp)
-        if (lane == 0) {
+        if (elect_one()) {
             constexpr uint32_t idesc = umma_idesc_f16(128, TOK) | (BF ? kUmmaIdescBf16 : 0u);
             // Every instruction this thread issues costs it 60-110 cycles (a tcgen05.mma about 60, a commit
             // about 80, a barrier wait about 100 even when the barrier is ready), so the loop is kept to one wait

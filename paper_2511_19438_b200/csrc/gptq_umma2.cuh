@@ -80,7 +80,7 @@ umma2_kernel(const UmmaArgs a, const __grid_constant__ CUtensorMap w_map, const 
     const uint32_t bar_full = base, bar_afull = base + 128, bar_done = base + 320;
     const uint32_t bar_dfull = base + 256, tmem_slot = base + 264;
     const uint32_t ring = base + 1024;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const int NS = a.stages;
     const int ptiles = a.N / kPanel / 2;
     const int pair = blockIdx.x >> 1, rank = blockIdx.x & 1;             // cluster = CTAs 2 pair, 2 pair + 1
@@ -116,7 +116,7 @@ umma2_kernel(const UmmaArgs a, const __grid_constant__ CUtensorMap w_map, const 
     const int G = a.G;
     if (warp == 0) {
         // ---------------------------------------------------------------- TMA producer (one thread per CTA)
-        if (lane == 0) {
+        if (elect_one()) {
             tma_prefetch_descriptor(&w_map);
             tma_prefetch_descriptor(&x_map);
             constexpr uint32_t kWBytes = 2 * kUmmaWBlockBytes, kXBytes = 2 * kXTile;
@@ -146,7 +146,7 @@ umma2_kernel(const UmmaArgs a, const __grid_constant__ CUtensorMap w_map, const 
         }
     } else if (warp == 1) {
         // ---------------------------------------------------------------- MMA issue (one thread of the leader CTA)
-        if (lane == 0 && rank == 0) {
+        if (rank == 0 && elect_one()) {
             constexpr uint32_t idesc = umma_idesc_f16(256, kUmma2Tok);
             int s = 0, sa = 0;
             uint32_t pha = 0;

@@ -246,7 +246,10 @@ def kernel_of(spec, M, sm_count):
     for (K, N) in spec["shapes"].values():
         if spec.get("w8", False):
             K = 2 * K
-        st, pl = B.gptq_plan(M, N, K, wl.GROUP_SIZE, 1 if spec["act_order"] else 0, sm_count)
+        act = 1 if spec["act_order"] else 0
+        st, pl = B.gptq_plan_decode(M, N, K, wl.GROUP_SIZE, act, sm_count)
+        if st != B.GPTQ_OK or spec.get("bf16", False):
+            st, pl = B.gptq_plan(M, N, K, wl.GROUP_SIZE, act, sm_count)
         assert st == B.GPTQ_OK
         names[B.plan_kernel_name(pl)] = names.get(B.plan_kernel_name(pl), 0) + K * N
     return max(names, key=names.get)

@@ -148,7 +148,7 @@ int gptq_set_workspace(void *ptr, size_t bytes);
  * y fp16[M,N] = x fp16[M,K] . dequant(W).  qweight/qzeros/scales are the REPACKED buffers from
  * gptq_repack; with act_order != 0, g_idx is gptq_repack's perm_out (16-byte aligned like every other pointer, else
  * GPTQ_ERR_ALIGN; without act-order it may be NULL).
- * fp32 accumulation, one round-to-nearest-even conversion to fp16.  Any M >= 1.  Up to 16 rows the
+ * fp32 accumulation, one round-to-nearest-even conversion to fp16 (an infinite x may give NaN).  Any M >= 1.  Up to 16 rows the
  * weights enter the MMA as exact integers q - z and the scale multiplies fp32 group sums; above
  * that each scaled weight is rounded to fp16 once before the MMA.
  * The kernels begin fetching weights before earlier work on the stream has finished
@@ -383,7 +383,8 @@ typedef struct {
                              bfloat16 flag (false for gptq_gemm, true for gptq_gemm_bf16) */
     int kernel;       /* 1 = cluster split-K mma.sync kernel (gptq_gemm, M <= 16),
                          2 = tcgen05 kernel (gptq_gemm, M >= 17),
-                         3 = stream-K mma.sync kernel (gptq_gemm_noalloc) */
+                         3 = stream-K mma.sync kernel (gptq_gemm_noalloc),
+                         4 = streaming tcgen05 decode kernel (gptq_gemm, M <= 4, see gptq_plan_decode) */
     int m_tile;       /* tokens per CTA tile */
     int m_chunks;     /* launches along M */
     int stages;       /* pipeline depth */
@@ -398,8 +399,13 @@ typedef struct {
     int tail_cluster_size; /* cluster size of that second launch (1 when there is none) */
 } gptq_plan_t;
 
-/* How gptq_gemm would launch this problem on a GPU with sm_count SMs. */
+/* How the tile kernels (kernel 1 and 2) would launch this problem on a GPU with sm_count SMs: what gptq_gemm does, unless
+ * gptq_plan_decode takes the problem. */
 int gptq_plan(int M, int N, int K, int group_size, int act_order, int sm_count, gptq_plan_t *out);
+/* The same for the streaming decode kernel (kernel 4), which takes fp16 problems of up to 4 token rows that fill the SMs;
+ * GPTQ_ERR_UNSUPPORTED for a problem that it leaves to the tile kernels.  `ctas` = clusters x cluster_size, each cluster
+ * working through several panels; `stages` = depth of the weight ring in steps. */
+int gptq_plan_decode(int M, int N, int K, int group_size, int act_order, int sm_count, gptq_plan_t *out);
 /* The same for gptq_gemm_noalloc (stream-K kernel; workspace_bytes is its need of the built-in scratch). */
 int gptq_plan_noalloc(int M, int N, int K, int group_size, int act_order, int sm_count, gptq_plan_t *out);
 

@@ -97,6 +97,7 @@ _SIGNATURES = {
     "gptq_trace_reset": (_i, [_vp]),
     "gptq_trace_read": (_i, [_vp, _i, _vp]),
     "gptq_plan": (_i, [_i, _i, _i, _i, _i, _i, ctypes.POINTER(gptq_plan_t)]),
+    "gptq_plan_decode": (_i, [_i, _i, _i, _i, _i, _i, ctypes.POINTER(gptq_plan_t)]),
     "gptq_plan_noalloc": (_i, [_i, _i, _i, _i, _i, _i, ctypes.POINTER(gptq_plan_t)]),
     "gptq_plan_cta_range": (_i, [_i, _i, _i, ctypes.POINTER(_i), ctypes.POINTER(_i)]),
     "gptq_plan_panel_owners": (_i, [_i, _i, _i, _i, ctypes.POINTER(_i), ctypes.POINTER(_i)]),
@@ -343,6 +344,12 @@ def gptq_plan(M, N, K, group_size, act_order, sm_count):
     out = gptq_plan_t()
     st = _lib.gptq_plan(M, N, K, group_size, int(act_order), sm_count, ctypes.byref(out))
     return st, out
+
+
+def gptq_plan_decode(M, N, K, group_size, act_order, sm_count):
+    plan = gptq_plan_t()
+    st = _lib.gptq_plan_decode(M, N, K, group_size, int(act_order), sm_count, ctypes.byref(plan))
+    return st, plan
 
 
 def gptq_plan_noalloc(M, N, K, group_size, act_order, sm_count):

@@ -5,6 +5,7 @@
 #include "gptq_streamk.cuh"
 #include "gptq_splitk.cuh"
 #include "gptq_umma.cuh"
+#include "gptq_decode.cuh"
 #include "gptq_umma2.cuh"
 #include "gptq_w8.cuh"
 #include "gptq_wn.cuh"
@@ -315,6 +316,32 @@ int gptq_plan(int M, int N, int K, int group_size, int act_order, int sm_count, 
     return GPTQ_OK;
 }
 
+int gptq_plan_decode(int M, int N, int K, int group_size, int act_order, int sm_count, gptq_plan_t *out)
+{
+    if (!out) return GPTQ_ERR_NULL;
+    int st = check_shape(M, N, K, group_size);
+    if (st) return st;
+    st = check_fast_path(N, K, group_size);
+    if (st) return st;
+    if (sm_count < 1) return GPTQ_ERR_SHAPE;
+    const DecodePlan pl = plan_decode(M, N, K, group_size, 0, 0, sm_count);
+    if (!pl.use) return GPTQ_ERR_UNSUPPORTED;
+    out->kernel = 4;
+    out->m_tile = pl.nx;
+    out->m_chunks = 1;
+    out->stages = pl.w_slots;
+    out->ctas = pl.ctas;
+    out->items = (N / kPanel) * (K / kGroup);
+    out->split_panels = pl.S > 1 ? N / kPanel : 0;
+    out->smem_bytes = pl.smem_bytes;
+    out->workspace_bytes = gemm_workspace_need(M, K, act_order);
+    out->cluster_size = pl.S;
+    out->tail_ctas = 0;
+    out->tail_cluster_size = 1;
+    set_kernel_name(out, "decode_kernel<%d,%d>", pl.nx, pl.sub);
+    return GPTQ_OK;
+}
+
 int gptq_plan_noalloc(int M, int N, int K, int group_size, int act_order, int sm_count, gptq_plan_t *out)
 {
     if (!out) return GPTQ_ERR_NULL;
@@ -418,6 +445,9 @@ static int gemm_dispatch(const void *x, const void *qweight, const void *qzeros,
         xin = x_perm;
     }
     const size_t ldy = fuse ? (size_t)N / 2 : (size_t)N;
+    if (const DecodePlan dp = plan_decode(M, N, K, group_size, fuse, bf16, sms); dp.use)
+        return launch_decode(xin, qweight, qzeros, scales, (__half *)y, M, N, K, dp, fuse, (const __half *)bias,
+                             (const __half *)residual, out_index, s);
     if (M >= kUmmaMinTokens) {
         if (!fuse && !extras && !bf16 && g_use_cta_pairs.load() && umma2_applicable(M, N) && group_size == kGroup) {
             const Umma2Plan p2 = plan_umma2(M, N, K);

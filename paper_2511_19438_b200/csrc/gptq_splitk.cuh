@@ -67,6 +67,8 @@ __device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t par
 // bounded like mbar_wait, but observing arrivals and stores from other CTAs of the cluster
 __device__ __noinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity)
 {
+    for (int it = 0; it < kWaitTries; ++it)
+        if (mbar_try_wait_cluster(bar, parity)) return true;
     const uint64_t start = global_timer_ns();
     for (;;) {
         for (int it = 0; it < 256; ++it)
@@ -428,6 +430,16 @@ SplitKPlan plan_splitk(int m_rows, int N, int K, int group_size, int sm_count)
     return pl;
 }
 
+// The owners' column slices of a run (128 columns, or 64 with the gate/up epilogue): byte q of *slice_lo = first column of
+// owner q < S, *slice_max = the widest slice.
+inline void split_columns(int fuse, int S, unsigned long long *slice_lo, int *slice_max)
+{
+    const int run = fuse ? 64 : kPanel;
+    *slice_lo = 0;
+    for (int q = 0; q < 8; ++q) *slice_lo |= (unsigned long long)(q < S ? q * run / S : run) << (8 * q);
+    *slice_max = (run + S - 1) / S;
+}
+
 template <int MT, int SUB, bool BF>
 static int launch_splitk_mt(const SplitKArgs &args, const CUtensorMap &x_map, const SplitKPlan &plan, cudaStream_t s)
 {
@@ -477,12 +489,7 @@ int launch_splitk(const __half *x, const void *qweight, const void *qzeros, cons
     args.residual = residual;
     args.trace_slot = next_trace_slot();
     args.out_index = out_index;
-    {
-        const int run = fuse ? 64 : kPanel;
-        args.slice_lo = 0;
-        for (int q = 0; q < 8; ++q) args.slice_lo |= (unsigned long long)(q < plan.S ? q * run / plan.S : run) << (8 * q);
-        args.slice_max = (run + plan.S - 1) / plan.S;
-    }
+    split_columns(fuse, plan.S, &args.slice_lo, &args.slice_max);
     args.trailer = reinterpret_cast<const TiledTrailer *>((const uint8_t *)qzeros + tiled_zero_bytes(N, K, kGroup / plan.sub));
     // x as a 2-D tensor [M rows, K halves]; a box is one K64 tile of all token rows of the CTA tile
     CUtensorMap x_map;

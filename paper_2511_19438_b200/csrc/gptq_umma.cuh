@@ -203,6 +203,7 @@ umma_kernel(const UmmaArgs a, const __grid_constant__ CUtensorMap w_map, const _
             GPTQ_TRACE_SET(a.trace_slot, kernel_and_ctas, (2ull << 32) | gridDim.x);
         }
     }
+    auto wait = [](uint32_t bar, uint32_t parity) { return TOK <= 128 ? mbar_wait_once(bar, parity) : mbar_wait(bar, parity); };
     constexpr int kStage = umma_slot_bytes(TOK, NP);
     // ring slot = BPS K64 blocks: [x tile of each block][W blocks of each panel]
     constexpr int BPS = umma_blocks_per_slot(TOK);
@@ -304,7 +305,7 @@ umma_kernel(const UmmaArgs a, const __grid_constant__ CUtensorMap w_map, const _
                 const uint32_t bar = bar_full + 8 * s, st = ring + s * kStage;
                 if (i >= NS) {
                     const int c = (i - NS) * BPS + BPS - 1;
-                    if (!mbar_wait(bar_done + 8 * (c & (kUmmaDoneRing - 1)), (uint32_t)((c / kUmmaDoneRing) & 1))) break;
+                    if (!wait(bar_done + 8 * (c & (kUmmaDoneRing - 1)), (uint32_t)((c / kUmmaDoneRing) & 1))) break;
                     mbar_arrive_expect_tx(bar, kXBytes + kWBytes);
                     issue_w(i, s);
                 } else {
@@ -334,7 +335,7 @@ umma_kernel(const UmmaArgs a, const __grid_constant__ CUtensorMap w_map, const _
                 const uint64_t bdesc = umma_desc_k_major_sw128(ring + s * kStage + (b % BPS) * kXTile);
 #pragma unroll
                 for (int j = 0; j < NP; ++j) {
-                    ok = mbar_wait(bar_afull + 8 * (j * NA + sa), pha);
+                    ok = wait(bar_afull + 8 * (j * NA + sa), pha);
                     if (!ok) return;
                     tc_fence_after_sync();
                     if (b == b_begin) GPTQ_TRACE_MIN(a.trace_slot, first_data);   // (nothing in a normal build)
@@ -419,8 +420,8 @@ umma_kernel(const UmmaArgs a, const __grid_constant__ CUtensorMap w_map, const _
                 // A set skips the other sets' slots, so its parity wait on a slot is only unambiguous once the slot's
                 // previous refill is known to have landed: the MMAs of that refill's last block have completed.
                 const int c = (b / BPS - NS) * BPS + BPS - 1;
-                if (c > 0) ok = __all_sync(0xffffffffu, mbar_wait(bar_done + 8 * (c & (kUmmaDoneRing - 1)), (uint32_t)((c / kUmmaDoneRing) & 1)));
-                ok = ok && __all_sync(0xffffffffu, mbar_wait(bar_full + 8 * s, ph));   // warp-uniform
+                if (c > 0) ok = __all_sync(0xffffffffu, wait(bar_done + 8 * (c & (kUmmaDoneRing - 1)), (uint32_t)((c / kUmmaDoneRing) & 1)));
+                ok = ok && __all_sync(0xffffffffu, wait(bar_full + 8 * s, ph));   // warp-uniform
                 if (!ok) break;
             }
             if ((b & 1) == 0) {
@@ -475,7 +476,7 @@ umma_kernel(const UmmaArgs a, const __grid_constant__ CUtensorMap w_map, const _
                     o[3] = hmul2_u32(hsub2_u32(lop3_and_or(w, HI, MAGIC_HI), zhi_b[jj]), s2_b[jj]);
                 }
             if (b >= NA) {     // the stage's previous block b - NA must have been multiplied
-                ok = __all_sync(0xffffffffu, mbar_wait(bar_done + 8 * ((b - NA) & (kUmmaDoneRing - 1)), (uint32_t)(((b - NA) / kUmmaDoneRing) & 1)));
+                ok = __all_sync(0xffffffffu, wait(bar_done + 8 * ((b - NA) & (kUmmaDoneRing - 1)), (uint32_t)(((b - NA) / kUmmaDoneRing) & 1)));
                 if (!ok) break;
                 tc_fence_after_sync();
             }
@@ -493,7 +494,7 @@ umma_kernel(const UmmaArgs a, const __grid_constant__ CUtensorMap w_map, const _
         }
         // ---- epilogue: lane n of the accumulator holds y[m0 .. m0+TOK, 128 p + n]
         pdl_wait();
-        ok = __all_sync(0xffffffffu, ok && mbar_wait(bar_dfull, 0));
+        ok = __all_sync(0xffffffffu, ok && wait(bar_dfull, 0));
         if (ok) tc_fence_after_sync();
         ok = ok && layout_ok;
         // 32 tokens (from c0) of this lane's column: the sum of the issuers' accumulators (an issuer without blocks,

@@ -1428,3 +1428,33 @@ def test_low_bit_repack_argument_checks():
     assert call(k=K + 128 + 8) == B.GPTQ_ERR_SHAPE
     assert call() == B.GPTQ_OK
     torch.cuda.synchronize()
+
+
+# ------------------------------------------------------------------------------- the streaming decode kernel
+@pytest.mark.parametrize("K,N,gs,act,zm1", [
+    (4096, 4096, 128, False, False),      # one panel per cluster
+    (4096, 12288, 128, False, True),      # three panels per cluster, both zero conventions
+    (4224, 12288, 128, True, False),      # K groups that four CTAs share unevenly (9, 8, 8, 8): lone last items
+    (4096, 22016, 64, False, False),      # clusters of three (unequal column slices), two groups per item
+    (3328, 22016, 32, False, True),       # four groups per item
+    (13824, 5120, 128, False, False),     # the widest K range per CTA
+])
+@pytest.mark.parametrize("M", [1, 2, 3, 4])
+def test_decode_kernel(K, N, gs, act, zm1, M, ws):
+    """Every token tile and group size of the streaming decode kernel, with the plain, bias + residual and gate/up epilogues.
+    The operands are exact (nibbles as e4m3, x as four e5m2 pieces) and the sums fp32, so the tight bound of the mma.sync
+    kernel holds: half an ulp of the fp16 result plus 1e-4 sqrt(K / 4096)."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    if sms == 148 and M <= 2:
+        assert B.gptq_plan_decode(M, N, K, gs, int(act), sms)[0] == B.GPTQ_OK, "the planner no longer takes this shape: choose another"
+    L = wl.make_linear(K, N, seed=wl.seed_for("decode", K, N, gs), group_size=gs, act_order=act, zeros_minus_one=zm1)
+    x_np = wl.make_x(M, K, wl.seed_for("decode-x", M, K))
+    x_np[0, :8] = np.float16([6e-8, -6e-8, 3e-5, 0, 100.5, -0.1, 2.0 ** -14, 1.0])      # subnormals and a large value
+    y, _ = run_gemm(L, x_np, ws)
+    y64 = oracle.gemm_f64(x_np, L.qweight, L.qzeros, L.scales, L.g_idx, gs, zeros_minus_one=zm1)
+    assert_close(y, y64, K, M)
+    if not zm1:
+        check_bias_residual(L, M, ws, True, True)
+    if N == 22016:
+        check_silu_mul(L, x_np, ws)
+    assert B.gptq_check_status() == B.GPTQ_OK

@@ -230,7 +230,7 @@ def launches_per_gemm(spec, M, name, sm_count):
     from paper_2511_19438_b200 import binding as B
     K, N = spec["shapes"][name]
     if spec.get("w8", False):       # the 4-bit kernels on the stacked planes (2 K rows), always behind the x gather
-        st, pl = B.gptq_plan(M, N, 2 * K, wl.GROUP_SIZE, 0, sm_count)
+        st, pl = B.gptq_plan(M, N, 2 * K if M <= 16 else K, wl.GROUP_SIZE, 0, sm_count)     # from 17 rows on: both planes at once
         assert st == B.GPTQ_OK
         return 2 + (1 if pl.tail_ctas > 0 else 0)
     st, pl = B.gptq_plan(M, N, K, wl.GROUP_SIZE, 1 if spec["act_order"] else 0, sm_count)
@@ -244,7 +244,7 @@ def kernel_of(spec, M, sm_count):
     from paper_2511_19438_b200 import binding as B
     names = {}
     for (K, N) in spec["shapes"].values():
-        if spec.get("w8", False):
+        if spec.get("w8", False) and M <= 16:
             K = 2 * K
         act = 1 if spec["act_order"] else 0
         st, pl = B.gptq_plan_decode(M, N, K, wl.GROUP_SIZE, act, sm_count)

@@ -247,7 +247,8 @@ int gptq_dequant_f32_bits(int bits, const void *qweight, const void *qzeros, con
  * that convention, z = 256, is refused with GPTQ_ERR_UNSUPPORTED).
  * An 8-bit weight is two nibbles, (q - z) s = (hi - zh) (16 s) + (lo - zl) s: gptq_repack_w8 stores the layer as a 4-bit
  * layer of 2 K rows (rows 0..K-1 the high nibbles with scales 16 s, rows K..2K-1 the low nibbles) in the usual tiled
- * layout, and gptq_gemm_w8 gathers x into [x | x] in that layer's row order and runs the 4-bit kernels on 2 K rows.  One
+ * layout.  gptq_gemm_w8 gathers x into that layer's row order; up to 16 token rows it runs the 4-bit kernels on the 2 K
+ * rows (x taken twice), above that the tcgen05 kernel joins the two nibbles of a weight before the MMA.  One
  * byte per weight is streamed, as the format requires; scales and zero points take twice their canonical bytes.
  * Requirements: as gptq_repack (group_size 32, 64 or a multiple of 128; K % 128 == 0; N % 128 == 0), scales < 4096. */
 
@@ -273,7 +274,7 @@ int gptq_dequant_f32_w8(const void *qweight, const void *qzeros, const void *sca
  * aligned).  Needs the registered workspace: gptq_workspace_bytes(M, N, 2 * K, group_size, 1) bytes, for the gathered
  * activations.  K and group_size are the checkpoint's.  Stream semantics, kernels by M, accuracy bar and error codes as
  * for gptq_gemm with act_order = 1; up to 16 token rows the integers are exact and the scales join in fp32, above that
- * each plane's scaled weight is rounded to fp16 once. */
+ * each scaled weight is rounded to fp16 once. */
 int gptq_gemm_w8(const void *x, const void *qweight, const void *qzeros, const void *scales, const int32_t *perm,
                  void *y, int M, int N, int K, int group_size, void *stream);
 

@@ -456,7 +456,7 @@ static int gemm_dispatch(const void *x, const void *qweight, const void *qzeros,
         // tcgen05 kernel: 32- to 256-token tiles
         const UmmaPlan pl = plan_umma(M, N, K, sms);
         return launch_umma(xin, qweight, qzeros, scales, (__half *)y, M, N, K, group_size, pl, fuse, (const __half *)bias,
-                           (const __half *)residual, out_index, bf16, s);
+                           (const __half *)residual, out_index, bf16, 0, s);
     }
     for (int m0 = 0; m0 < M; m0 += kStreamKMaxRows) {
         const int rows = (M - m0) < kStreamKMaxRows ? (M - m0) : kStreamKMaxRows;
@@ -590,6 +590,13 @@ int gptq_gemm_w8(const void *x, const void *qweight, const void *qzeros, const v
         ws = g_workspace[dev];
     }
     if (ws.ptr == nullptr || ws.bytes < gemm_workspace_need(M, 2 * K, 1)) return GPTQ_ERR_WORKSPACE;
+    if (M >= kUmmaMinTokens) {
+        // the tcgen05 kernel joins the planes itself: x once, in the row order of either plane
+        st = launch_gather_x((const __half *)x, perm, (__half *)ws.ptr, M, K, (cudaStream_t)stream);
+        if (st) return st;
+        return launch_umma((const __half *)ws.ptr, qweight, qzeros, scales, (__half *)y, M, N, K, tiled,
+                           plan_umma(M, N, K, sms, true), 0, nullptr, nullptr, nullptr, 0, 1, (cudaStream_t)stream);
+    }
     st = launch_w8_gather_x((const __half *)x, perm, (__half *)ws.ptr, M, K, (cudaStream_t)stream);
     if (st) return st;
     // the stacked layer, its activations already in its row order

@@ -174,11 +174,12 @@ struct UmmaArgs {
 // K64 blocks per ring slot of the single-CTA kernel: a whole K group (two blocks: fewer, larger copies for the
 // producer thread) except for 128-token tiles, where two CTAs share an SM and group-sized slots would leave each
 // a ring of only two
-__host__ __device__ constexpr int umma_blocks_per_slot(int TOK) { return TOK == 128 ? 1 : 2; }
+// With 8-bit weights a block is 4 KB of each plane: slots of one block, so that 256-token tiles keep five of them.
+__host__ __device__ constexpr int umma_blocks_per_slot(int TOK, bool W8 = false) { return TOK == 128 || W8 ? 1 : 2; }
 // one ring slot: x tile(s) and packed weights of each panel (scales and zeros do not pass through shared memory)
-__host__ __device__ constexpr int umma_slot_bytes(int TOK, int NP)
+__host__ __device__ constexpr int umma_slot_bytes(int TOK, int NP, bool W8 = false)
 {
-    return (umma_blocks_per_slot(TOK) * (TOK * 128 + NP * kUmmaWBlockBytes) + 1023) & ~1023;
+    return (umma_blocks_per_slot(TOK, W8) * (TOK * 128 + NP * (W8 ? 2 : 1) * kUmmaWBlockBytes) + 1023) & ~1023;
 }
 __host__ __device__ constexpr int umma_tmem_cols(int TOK, int NA, int NP, int ISS)
 {
@@ -188,7 +189,11 @@ __host__ __device__ constexpr int umma_tmem_cols(int TOK, int NA, int NP, int IS
     return c;
 }
 
-template <int TOK, int NA, int NP, int SETS, int SUB, bool BF = false>
+// W8: 8-bit weights, stored as two stacked 4-bit planes (K rows of high nibbles, then K of low ones; a.K and a.G count the K
+// real rows).  The dequant warps join the nibbles to fp16 integers 1024 + q8 - one MMA row per weight, where the stacked
+// layer run as a 4-bit one takes two.  (4096 x 22016, gather included: 44 instead of 55 us at M = 64, 99 instead of 152 at
+// M = 300, 211 instead of 343 at M = 1024.)
+template <int TOK, int NA, int NP, int SETS, int SUB, bool BF = false, bool W8 = false>
 __global__ void __launch_bounds__(umma_threads(TOK, NP, SETS), (NP > 1 || TOK > 128) ? 1 : TOK <= 32 ? 3 : 2)
 umma_kernel(const UmmaArgs a, const __grid_constant__ CUtensorMap w_map, const __grid_constant__ CUtensorMap x_map)
 {
@@ -204,9 +209,10 @@ umma_kernel(const UmmaArgs a, const __grid_constant__ CUtensorMap w_map, const _
         }
     }
     auto wait = [](uint32_t bar, uint32_t parity) { return TOK <= 128 ? mbar_wait_once(bar, parity) : mbar_wait(bar, parity); };
-    constexpr int kStage = umma_slot_bytes(TOK, NP);
+    constexpr int kStage = umma_slot_bytes(TOK, NP, W8);
     // ring slot = BPS K64 blocks: [x tile of each block][W blocks of each panel]
-    constexpr int BPS = umma_blocks_per_slot(TOK);
+    constexpr int BPS = umma_blocks_per_slot(TOK, W8);
+    constexpr int PL = W8 ? 2 : 1;                          // nibble planes
     constexpr int kXTile = TOK * 128;
     constexpr int kOffW = BPS * kXTile;
     constexpr int ISS = umma_issuers(TOK, SETS);
@@ -276,7 +282,7 @@ umma_kernel(const UmmaArgs a, const __grid_constant__ CUtensorMap w_map, const _
             tma_prefetch_descriptor(&x_map);
             constexpr uint32_t kXBytes = BPS * kXTile;
             const int NR = NB / BPS;                         // ring refills of this CTA
-            constexpr uint32_t kWBytes = NP * BPS * kUmmaWBlockBytes;
+            constexpr uint32_t kWBytes = NP * BPS * PL * kUmmaWBlockBytes;
             // the packed weights of refill i (scales and zeros are read by the dequant warps themselves)
             auto issue_w = [&](int i, int s) {
                 const uint32_t st = ring + s * kStage, bar = bar_full + 8 * s;
@@ -284,7 +290,10 @@ umma_kernel(const UmmaArgs a, const __grid_constant__ CUtensorMap w_map, const _
 #pragma unroll
                 for (int j = 0; j < NP; ++j)
                     // packed weights viewed as rows of 64 bytes; block b of panel p starts at row (2 G p + b) * 64
-                    tma_load_2d(st + kOffW + j * BPS * kUmmaWBlockBytes, &w_map, 0, (2 * a.G * (p0 + j) + b_first + b) * 64, bar);
+#pragma unroll
+                    for (int pl = 0; pl < PL; ++pl)
+                        tma_load_2d(st + kOffW + (j * PL + pl) * BPS * kUmmaWBlockBytes, &w_map, 0,
+                                    (2 * a.G * (PL * (p0 + j) + pl) + b_first + b) * 64, bar);
             };
             const int n_pre = NR < NS ? NR : NS;
             GPTQ_TRACE_MIN(a.trace_slot, first_weight_issue);
@@ -380,13 +389,15 @@ umma_kernel(const UmmaArgs a, const __grid_constant__ CUtensorMap w_map, const _
         // the column's 8 bytes (two words: rows +0..7 and +32..39) in each of the four 16-byte chunks
         uint32_t w_rd[4];
 #pragma unroll
-        for (int t4 = 0; t4 < 4; ++t4) w_rd[t4] = kOffW + j * BPS * kUmmaWBlockBytes + (u * 8 + g) * 64 + ((uint32_t)(t4 ^ (g >> 1)) << 4) + 8 * h;
+        for (int t4 = 0; t4 < 4; ++t4) w_rd[t4] = kOffW + j * PL * BPS * kUmmaWBlockBytes + (u * 8 + g) * 64 + ((uint32_t)(t4 ^ (g >> 1)) << 4) + 8 * h;
         // The column's scale and zero point of a group come straight from global memory (2 bytes and a nibble per
         // lane: 64 + 16 bytes per warp), fetched one group ahead into registers, which spares the producer thread two
         // copies per group.  In the tiled layout the pair (column, column + 8) is adjacent.
         // A 128-row item holds SUB quantisation groups (128 / group_size), each with its own scales and zeros.
-        const uint8_t *s_gl = a.scales + ((size_t)p * a.G + g0) * (SUB * kItemSBytes) + (16 * u + 2 * g + h) * 2;
-        const uint8_t *z_gl = a.qzeros + ((size_t)p * a.G + g0) * (SUB * kItemZBytes) + 8 * u + g;
+        // (8-bit: the scale of the low plane; zero points of both planes, joined to a byte)
+        const uint8_t *s_gl = a.scales + ((size_t)(p * PL + PL - 1) * a.G + g0) * (SUB * kItemSBytes) + (16 * u + 2 * g + h) * 2;
+        const uint8_t *z_gl = a.qzeros + ((size_t)p * PL * a.G + g0) * (SUB * kItemZBytes) + 8 * u + g;
+        const size_t z_plane = (size_t)a.G * (SUB * kItemZBytes);
         auto load_sz = [&](int gg, uint32_t (&sc)[SUB], uint32_t (&zb)[SUB]) {
             // through L2 only: this kernel may start while its predecessor still runs, and the buffers may have been
             // rewritten since an earlier kernel left lines of them in this SM's L1
@@ -394,6 +405,7 @@ umma_kernel(const UmmaArgs a, const __grid_constant__ CUtensorMap w_map, const _
             for (int sub = 0; sub < SUB; ++sub) {
                 sc[sub] = __ldcg(reinterpret_cast<const unsigned short *>(s_gl + ((size_t)gg * SUB + sub) * kItemSBytes));
                 zb[sub] = __ldcg(z_gl + ((size_t)gg * SUB + sub) * kItemZBytes);
+                if (W8) zb[sub] = zb[sub] << 8 | __ldcg(z_gl + z_plane + ((size_t)gg * SUB + sub) * kItemZBytes);
             }
         };
         uint32_t sc_next[SUB], zb_next[SUB];
@@ -429,7 +441,10 @@ umma_kernel(const UmmaArgs a, const __grid_constant__ CUtensorMap w_map, const _
                 for (int sub = 0; sub < SUB; ++sub) {
                     s2[sub] = sc_next[sub] * 0x00010001u;
                     const uint32_t z = (h ? (zb_next[sub] >> 4) : (zb_next[sub] & 15u)) + z_add;   // up to 16: still exact
-                    if constexpr (BF) {
+                    if constexpr (W8) {
+                        const uint32_t z2 = zb_next[sub] >> (h ? 4 : 0);                            // high plane's nibble in bits 8..11
+                        zlo[sub] = ((z2 >> 4 & 0xf0u) | (z2 & 15u)) * 0x00010001u | MAGIC_LO;       // 1024 + z, z < 256
+                    } else if constexpr (BF) {
                         zero_constants<true>(z, zlo[sub], zhi[sub]);
                     } else {
                         zlo[sub] = (z * 0x00010001u) | MAGIC_LO;
@@ -442,6 +457,11 @@ umma_kernel(const UmmaArgs a, const __grid_constant__ CUtensorMap w_map, const _
             uint2 wv[4];
 #pragma unroll
             for (int t4 = 0; t4 < 4; ++t4) wv[t4] = lds64(wb + w_rd[t4]);
+            uint2 wl[4];                // 8-bit: the low nibbles (wv: the high ones)
+            if constexpr (W8) {
+#pragma unroll
+                for (int t4 = 0; t4 < 4; ++t4) wl[t4] = lds64(wb + kUmmaWBlockBytes + w_rd[t4]);
+            }
             // constants of the two 32-row halves of this block: the item's group (SUB = 1), the block's (2) or the
             // half's own (4); picked with selects so that the arrays stay in registers
             uint32_t s2_b[2], zlo_b[2], zhi_b[2];
@@ -461,6 +481,17 @@ umma_kernel(const UmmaArgs a, const __grid_constant__ CUtensorMap w_map, const _
                 for (int t4 = 0; t4 < 4; ++t4) {
                     uint32_t w = jj ? wv[t4].y : wv[t4].x;       // rows 32 jj + 8 t4 + (0..7), TMEM columns 16 jj + 4 t4 + (0..3)
                     uint32_t *o = r + 16 * jj + 4 * t4;
+                    if constexpr (W8) {
+                        // 1024 + 16 hi + lo is an exact fp16 number, so are q - z and its difference; one rounding with the scale
+                        const uint32_t l = jj ? wl[t4].y : wl[t4].x;
+                        o[0] = lop3_and_or(l, LO, lop3_and_or(w << 4, HI, MAGIC_LO));
+                        o[1] = lop3_and_or(l >> 4, LO, lop3_and_or(w, HI, MAGIC_LO));
+                        o[2] = lop3_and_or(l >> 8, LO, lop3_and_or(w >> 4, HI, MAGIC_LO));
+                        o[3] = lop3_and_or(l >> 12, LO, lop3_and_or(w >> 8, HI, MAGIC_LO));
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) o[e] = hmul2_u32(hsub2_u32(o[e], zlo_b[jj]), s2_b[jj]);
+                        continue;
+                    }
                     if constexpr (BF) {
                         // bfloat16: exact q - z, then one rounding in the product with the scale
                         uint32_t d[4];
@@ -847,7 +878,7 @@ __host__ __device__ constexpr int umma_ctas_per_sm(int tok, int np) { return (np
 // half-empty 256-token tile measured 15-22 % faster than two 128-token tiles on all four 7B shapes);
 // cluster size and shared-memory padding by the same rules as the mma.sync kernel.  Two panels per CTA
 // (np = 2) halve the x traffic per flop but allow only one CTA per SM and measured slower, so np = 1.
-inline UmmaPlan plan_umma(int M, int N, int K, int sm_count)
+inline UmmaPlan plan_umma(int M, int N, int K, int sm_count, bool w8 = false)
 {
     UmmaPlan pl{};
     const int tok = M <= 32 ? 32 : M <= 64 ? 64 : M <= 128 ? 128 : 256;
@@ -855,7 +886,7 @@ inline UmmaPlan plan_umma(int M, int N, int K, int sm_count)
     const int np = 1;
     const int sets = 2;
     const int G = K / kGroup, tiles = (panels / np) * ((M + tok - 1) / tok);
-    const int stage = umma_slot_bytes(tok, np);
+    const int stage = umma_slot_bytes(tok, np, w8), bps = umma_blocks_per_slot(tok, w8);
     const int cps_max = umma_ctas_per_sm(tok, np);
     int best_S = 1;
     long long best_t = -1;
@@ -882,8 +913,8 @@ inline UmmaPlan plan_umma(int M, int N, int K, int sm_count)
     int stages = (smem_cap - 2048) / stage;
     if (stages > 8) stages = 8;
     // fewer blocks in the ring than "block multiplied" barriers (see the kernel)
-    if (stages * umma_blocks_per_slot(tok) >= kUmmaDoneRing) stages = (kUmmaDoneRing - 1) / umma_blocks_per_slot(tok);
-    const int refills_per_cta = 2 * groups_per_cta / umma_blocks_per_slot(tok);
+    if (stages * bps >= kUmmaDoneRing) stages = (kUmmaDoneRing - 1) / bps;
+    const int refills_per_cta = 2 * groups_per_cta / bps;
     if (stages > refills_per_cta) stages = refills_per_cta;
     while (S > 1 && stages * stage < tok * kPanel * 4) ++stages;   // the ring doubles as the fp32 partial tile
     pl.tok = tok;
@@ -902,10 +933,10 @@ inline UmmaPlan plan_umma(int M, int N, int K, int sm_count)
         int ts = 1;
         while (ts * 2 <= (tok >= 128 ? 4 : 8) && ts * 2 <= G && r * ts * 2 <= slots) ts *= 2;
         int tstages = stages;
-        const int trefills = 2 * ((G + ts - 1) / ts) / umma_blocks_per_slot(tok);
+        const int trefills = 2 * ((G + ts - 1) / ts) / bps;
         if (tstages > trefills) tstages = trefills;
         while (tstages * stage < tok * kPanel * 4) ++tstages;      // the ring doubles as the fp32 partial tile
-        if (ts > 1 && 2048 + tstages * stage <= pl.smem_bytes && tstages * umma_blocks_per_slot(tok) < kUmmaDoneRing) {
+        if (ts > 1 && 2048 + tstages * stage <= pl.smem_bytes && tstages * bps < kUmmaDoneRing) {
             pl.tail_tiles = r;
             pl.tail_S = ts;
             pl.tail_stages = tstages;
@@ -915,11 +946,11 @@ inline UmmaPlan plan_umma(int M, int N, int K, int sm_count)
     return pl;
 }
 
-template <int TOK, int NP, int SETS, int SUB, bool BF>
+template <int TOK, int NP, int SETS, int SUB, bool BF, bool W8 = false>
 static int launch_umma_sub(const UmmaArgs &args, const CUtensorMap &w_map, const CUtensorMap &x_map,
                            const UmmaPlan &plan, int ctas, cudaStream_t s)
 {
-    auto kernel = umma_kernel<TOK, umma_a_stages(TOK, NP), NP, SETS, SUB, BF>;
+    auto kernel = umma_kernel<TOK, umma_a_stages(TOK, NP), NP, SETS, SUB, BF, W8>;
     static int configured_smem[64] = {};
     const int cfg_st = ensure_dynamic_smem((const void *)kernel, configured_smem, plan.smem_bytes);
     if (cfg_st) return cfg_st;
@@ -942,22 +973,25 @@ static int launch_umma_sub(const UmmaArgs &args, const CUtensorMap &w_map, const
 
 template <int TOK, int NP, int SETS>
 static int launch_umma_tok(const UmmaArgs &args, const CUtensorMap &w_map, const CUtensorMap &x_map,
-                           const UmmaPlan &plan, int ctas, int sub, int bf16, cudaStream_t s)
+                           const UmmaPlan &plan, int ctas, int sub, int bf16, int w8, cudaStream_t s)
 {
-    switch (sub + (bf16 ? 10 : 0)) {
+    switch (sub + (w8 ? 20 : bf16 ? 10 : 0)) {
     case 1: return launch_umma_sub<TOK, NP, SETS, 1, false>(args, w_map, x_map, plan, ctas, s);
     case 2: return launch_umma_sub<TOK, NP, SETS, 2, false>(args, w_map, x_map, plan, ctas, s);
     case 4: return launch_umma_sub<TOK, NP, SETS, 4, false>(args, w_map, x_map, plan, ctas, s);
     case 11: return launch_umma_sub<TOK, NP, SETS, 1, true>(args, w_map, x_map, plan, ctas, s);
     case 12: return launch_umma_sub<TOK, NP, SETS, 2, true>(args, w_map, x_map, plan, ctas, s);
     case 14: return launch_umma_sub<TOK, NP, SETS, 4, true>(args, w_map, x_map, plan, ctas, s);
+    case 21: return launch_umma_sub<TOK, NP, SETS, 1, false, true>(args, w_map, x_map, plan, ctas, s);
+    case 22: return launch_umma_sub<TOK, NP, SETS, 2, false, true>(args, w_map, x_map, plan, ctas, s);
+    case 24: return launch_umma_sub<TOK, NP, SETS, 4, false, true>(args, w_map, x_map, plan, ctas, s);
     default: return GPTQ_ERR_UNSUPPORTED;
     }
 }
 
 int launch_umma(const __half *x, const void *qweight, const void *qzeros, const void *scales, __half *y, int M, int N,
                 int K, int group_size, const UmmaPlan &plan, int fuse, const __half *bias, const __half *residual,
-                const int32_t *out_index, int bf16, cudaStream_t s)
+                const int32_t *out_index, int bf16, int w8, cudaStream_t s)
 {
     UmmaArgs args;
     args.scales = (const uint8_t *)scales;
@@ -974,26 +1008,26 @@ int launch_umma(const __half *x, const void *qweight, const void *qzeros, const 
     args.residual = residual;
     args.trace_slot = next_trace_slot();
     args.out_index = out_index;
-    args.trailer = reinterpret_cast<const TiledTrailer *>((const uint8_t *)qzeros + tiled_zero_bytes(N, K, group_size));
-    const int sub = kGroup / group_size;
-    if (plan.stages < 1 || plan.stages * umma_blocks_per_slot(plan.tok) >= kUmmaDoneRing) return GPTQ_ERR_UNSUPPORTED;
+    args.trailer = reinterpret_cast<const TiledTrailer *>((const uint8_t *)qzeros + tiled_zero_bytes(N, w8 ? 2 * K : K, group_size));
+    const int sub = kGroup / group_size, bps = umma_blocks_per_slot(plan.tok, w8 != 0);
+    if (plan.stages < 1 || plan.stages * bps >= kUmmaDoneRing) return GPTQ_ERR_UNSUPPORTED;
     // packed weights as rows of 64 bytes (16 words); a box is one ring slot's K64 blocks of a panel (64 rows each)
     CUtensorMap w_map, x_map;
-    const uint64_t w_rows = (uint64_t)K * N / 2 / 64;
+    const uint64_t w_rows = (uint64_t)K * N * (w8 ? 2 : 1) / 2 / 64;
     int st = make_tensor_map_2d(&w_map, CU_TENSOR_MAP_DATA_TYPE_UINT32, qweight, 16, w_rows, 64, 16,
-                                (uint32_t)(64 * umma_blocks_per_slot(plan.tok)),
+                                (uint32_t)(64 * bps),
                                 CU_TENSOR_MAP_SWIZZLE_64B);
     if (st) return st;
     // x as K / 64 tiles of [M rows, 64 k]; a box is one ring slot's tiles of one token tile
     st = make_tensor_map_ktiles(&x_map, x, (uint64_t)K, (uint64_t)M, (uint32_t)plan.tok,
-                                (uint32_t)umma_blocks_per_slot(plan.tok));
+                                (uint32_t)bps);
     if (st) return st;
     auto launch = [&](const UmmaArgs &la, int ctas) {
         switch (plan.tok) {
-        case 32: return launch_umma_tok<32, 1, 2>(la, w_map, x_map, plan, ctas, sub, bf16, s);
-        case 64: return launch_umma_tok<64, 1, 2>(la, w_map, x_map, plan, ctas, sub, bf16, s);
-        case 128: return launch_umma_tok<128, 1, 2>(la, w_map, x_map, plan, ctas, sub, bf16, s);
-        case 256: return launch_umma_tok<256, 1, 2>(la, w_map, x_map, plan, ctas, sub, bf16, s);
+        case 32: return launch_umma_tok<32, 1, 2>(la, w_map, x_map, plan, ctas, sub, bf16, w8, s);
+        case 64: return launch_umma_tok<64, 1, 2>(la, w_map, x_map, plan, ctas, sub, bf16, w8, s);
+        case 128: return launch_umma_tok<128, 1, 2>(la, w_map, x_map, plan, ctas, sub, bf16, w8, s);
+        case 256: return launch_umma_tok<256, 1, 2>(la, w_map, x_map, plan, ctas, sub, bf16, w8, s);
         default: return (int)GPTQ_ERR_UNSUPPORTED;
         }
     };

@@ -4,11 +4,12 @@
 //     (q - z) s = (hi - zh) (16 s) + (lo - zl) s.
 // A layer [K, N] of 8-bit weights is therefore the sum of two 4-bit layers over the same activations: a HIGH plane with
 // weights hi, zero points zh and scales 16 s (exact: a power of two) and a LOW plane with lo, zl and s.  The repack
-// stacks the planes along K - a 4-bit layer of 2 K rows, rows 0..K-1 the high plane - and tiles that layer as usual;
-// the matmul gathers x into [x | x] in the stacked (and, with act-order, sorted) row order and runs the 4-bit kernels
-// on 2 K rows.  The bytes streamed are those of the 8-bit layer (one byte per weight; scales and zero points twice),
-// and so is the arithmetic: the integers are exact and each plane's scale joins in fp32 (M <= 16), respectively each
-// plane's scaled weight is rounded to fp16 once (tcgen05 kernel).
+// stacks the planes along K - a 4-bit layer of 2 K rows, rows 0..K-1 the high plane - and tiles that layer as usual.
+// Up to 16 token rows the matmul gathers x into [x | x] in the stacked (and, with act-order, sorted) row order and runs
+// the 4-bit kernels on 2 K rows: the integers are exact and each plane's scale joins in fp32.  Above, the tcgen05 kernel
+// reads a block of both planes at a time, joins the nibbles to q - z in registers and rounds the scaled weight to fp16
+// once - one MMA row per weight instead of two.  The bytes streamed are those of the 8-bit layer (one byte per weight;
+// scales and zero points twice).
 //
 // Canonical 8-bit layout (the 4-bit conventions at twice the field width): qweight int32[K/4, N], byte i of a word =
 // row 4 r + i; qzeros int32[G, N/4], byte j of a word = column 4 c + j; scales fp16[G, N]; g_idx int32[K].

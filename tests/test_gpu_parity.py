@@ -1458,3 +1458,25 @@ def test_decode_kernel(K, N, gs, act, zm1, M, ws):
     if N == 22016:
         check_silu_mul(L, x_np, ws)
     assert B.gptq_check_status() == B.GPTQ_OK
+
+
+# ------------------------------------------------------------------------------- 8-bit weights joined in the tcgen05 kernel
+@pytest.mark.parametrize("K,N,gs", [(384, 256, 128), (384, 256, 64), (256, 128, 32), (2048, 4864, 128)])
+@pytest.mark.parametrize("M", [17, 33, 64, 65, 129, 257])
+def test_w8_token_tiles(K, N, gs, M, ws):
+    """Every token tile of the 8-bit tcgen05 kernel at its edges, odd numbers of K groups, split-K clusters; each weight is
+    rounded to fp16 once, so per output the error has standard deviation (2^-11 / sqrt 3) sqrt(sum x^2 w^2), of which eight
+    are allowed, plus the output's rounding."""
+    L = wl.make_linear_w8(K, N, seed=wl.seed_for("w8-tiles", K, N, gs), group_size=gs, act_order=True)
+    x = wl.make_x(M, K, wl.seed_for("w8-tiles-x", M, K))
+    D = H.upload_and_repack_w8(L)
+    H.ensure_for_w8(ws, M, D)
+    y = H.gemm_w8(H.to_device(x), D).cpu().numpy().astype(np.float64)
+    assert B.gptq_check_status() == B.GPTQ_OK
+    want = oracle.gemm_f64_w8(x, L.qweight, L.qzeros, L.scales, L.g_idx, gs)
+    w = oracle.dequant_f32_w8(L.qweight, L.qzeros, L.scales, L.g_idx, gs).astype(np.float64)
+    sigma = 2.0 ** -11 / math.sqrt(3) * np.sqrt((x.astype(np.float64) ** 2) @ (w ** 2))
+    finite = np.abs(want) < 60000
+    bound = 8 * sigma + 2.0 ** -11 * np.abs(want) + 1e-3
+    err = np.abs(y - want)
+    assert np.all(err[finite] <= bound[finite]), (err[finite] / bound[finite]).max()

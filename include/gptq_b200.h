@@ -331,10 +331,11 @@ typedef struct {
 /* A step of matmuls whose activations live in host memory (the linears of a decode step, configs of
  * Section 4's serving setting): for each problem in order, on `stream`: copy x to the device, gptq_gemm,
  * copy y back - the same results as `count` gptq_gemm_host calls, but pipelined: the copies run on two
- * internal streams (created on first use) in chunks of consecutive problems (up to 16, up to 2 MiB of activations and
+ * internal streams (created on first use) in chunks of consecutive problems (up to 8, up to 2 MiB of activations and
  * results, none sharing a staging buffer with another of the last few chunks; large problems go one by one): the x of a chunk go up, its matmuls run back to back on `stream`, its y come down, and chunk c+1 goes up
  * while chunk c computes and chunk c-1 comes down; the matmuls themselves stay in order on `stream`, and `stream`
- * completes after the last copy.  Staging buffers may be shared between problems (reuse waits for the earlier user;
+ * completes after the last copy.  Small activations in pinned memory are copied by a kernel (one per chunk) instead of the
+ * copy engines; host buffers that are not pinned, or not 16-byte aligned, always go through cudaMemcpyAsync.  Staging buffers may be shared between problems (reuse waits for the earlier user;
  * problems that share one never sit in the same chunk).
  * All problems are validated before anything is enqueued; on an invalid problem *bad_index (if not
  * NULL) receives its index and nothing runs.  If a later step fails, `stream` is still joined with the

@@ -754,6 +754,79 @@ int gptq_gemm_noalloc(const void *x, const void *qweight, const void *qzeros, co
 
 } // extern "C"
 
+// ---- small copies between pinned host memory and the device -------------------------------------------------------
+// A cudaMemcpyAsync of a decode problem's activations (8-90 KB) costs the copy engine 2-4 us however small; one kernel that
+// walks a list of segments moves a chunk's in one go.
+constexpr int kCopySegments = 16;
+struct CopySegments {
+    const uint4 *src[kCopySegments];
+    uint4 *dst[kCopySegments];
+    uint32_t end[kCopySegments];      // 16-byte pieces of segments 0 .. i together
+    int count;
+};
+constexpr int kCopyThreads = 256, kCopyUnroll = 4, kCopyBlocks = 16;
+__global__ void __launch_bounds__(kCopyThreads) copy_segments_kernel(const __grid_constant__ CopySegments c)
+{
+    const uint32_t total = c.end[c.count - 1], stride = gridDim.x * kCopyThreads;
+    // kCopyUnroll loads in flight per thread: PCIe answers after 1-2 us
+    for (uint32_t i0 = blockIdx.x * kCopyThreads + threadIdx.x; i0 < total; i0 += stride * kCopyUnroll) {
+        uint4 v[kCopyUnroll];
+        uint4 *to[kCopyUnroll];
+#pragma unroll
+        for (int u = 0; u < kCopyUnroll; ++u) {
+            const uint32_t i = i0 + u * stride;
+            to[u] = nullptr;
+            if (i < total) {
+                int s = 0;
+                while (i >= c.end[s]) ++s;
+                const uint32_t at = i - (s ? c.end[s - 1] : 0u);
+                to[u] = c.dst[s] + at;
+                asm volatile("ld.global.cv.v4.u32 {%0,%1,%2,%3}, [%4];"
+                             : "=r"(v[u].x), "=r"(v[u].y), "=r"(v[u].z), "=r"(v[u].w) : "l"(c.src[s] + at));
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < kCopyUnroll; ++u)
+            if (to[u]) *to[u] = v[u];
+    }
+}
+// The address under which the device sees host memory, if it is pinned (else nullptr).
+static void *device_address_of_host(const void *host)
+{
+    cudaPointerAttributes attr{};
+    if (cudaPointerGetAttributes(&attr, host) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return nullptr;
+    }
+    return attr.type == cudaMemoryTypeHost ? attr.devicePointer : nullptr;
+}
+// Collects the copies of a chunk: a pinned, aligned host buffer becomes a segment, any other an ordinary asynchronous copy.
+struct ChunkCopies {
+    CopySegments seg{};
+    cudaStream_t stream;
+    bool to_device;
+    int add(void *dst, const void *src, size_t bytes)
+    {
+        void *host = device_address_of_host(to_device ? src : dst);
+        if (host == nullptr || (reinterpret_cast<uintptr_t>(host) & 15u) || bytes % 16 || bytes > (1u << 30))
+            return record_cuda_error(cudaMemcpyAsync(dst, src, bytes, to_device ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToHost, stream));
+        const int i = seg.count;
+        seg.src[i] = (const uint4 *)(to_device ? host : src);
+        seg.dst[i] = (uint4 *)(to_device ? dst : host);
+        seg.end[i] = (i ? seg.end[i - 1] : 0u) + (uint32_t)(bytes / 16);
+        seg.count = i + 1;
+        return seg.count == kCopySegments ? flush() : GPTQ_OK;
+    }
+    int flush()
+    {
+        if (seg.count == 0) return GPTQ_OK;
+        const uint32_t per_block = kCopyThreads * kCopyUnroll, blocks = (seg.end[seg.count - 1] + per_block - 1) / per_block;
+        copy_segments_kernel<<<blocks < kCopyBlocks ? blocks : kCopyBlocks, kCopyThreads, 0, stream>>>(seg);
+        seg.count = 0;
+        return record_cuda_error(cudaGetLastError());
+    }
+};
+
 // mode: 0 = fp16 layers (gptq_gemm), 1 = bfloat16 layers (gptq_gemm_bf16), 2 = 8-bit layers (gptq_gemm_w8)
 static int host_batch(const gptq_host_problem_t *problems, int count, void *stream, int *bad_index, int mode)
 {
@@ -806,7 +879,7 @@ static int host_batch(const gptq_host_problem_t *problems, int count, void *stre
     // A chunk that reaches back to a staging buffer used d problems earlier must wait for that problem's chunk, so the
     // pipeline only overlaps if chunks are short against d: a chunk holds at most d / 3 problems (one problem when
     // buffers are reused every few problems, kChunk when every problem has its own).
-    constexpr int kChunk = 16;
+    constexpr int kChunk = 8;
     std::vector<int> reuse((size_t)count);
     {
         std::unordered_map<const void *, int> last_index;     // staging buffer -> the last problem that used it
@@ -834,8 +907,8 @@ static int host_batch(const gptq_host_problem_t *problems, int count, void *stre
         for (; i1 < count; ++i1) {
             if (reuse[(size_t)i1] / 3 < limit) limit = reuse[(size_t)i1] / 3;
             if (i1 - i0 >= limit) break;      // (also ends the chunk before a problem that shares a buffer with it)
+            if (bytes + io_bytes(i1) > kChunkBytes) break;
             bytes += io_bytes(i1);
-            if (bytes > kChunkBytes) break;
         }
         const int c = n_chunks++;
         // a staging buffer used by an earlier chunk is overwritten only after that chunk is done with it: after its
@@ -856,10 +929,21 @@ static int host_batch(const gptq_host_problem_t *problems, int count, void *stre
         }
         if (wait_y_in >= 0) st = check(cudaStreamWaitEvent(pipe->in, ev_y[wait_y_in], 0));
         if (!st && wait_g >= 0 && wait_g > wait_y_in) st = check(cudaStreamWaitEvent(pipe->in, ev_g[wait_g], 0));
+        // Small activations go up by one copy kernel per chunk, and the last chunk's results come down by one (nothing
+        // computes beside them any more); other results, and larger problems both ways, go through the copy engines, which
+        // move more than the few blocks the matmuls leave room for.  Eight 7B layers at M = 4: 367 us, all by kernel 390,
+        // all by copy engine 407 (452 in chunks of sixteen); four layers at M = 16: 308, 337, 279.
+        const bool by_kernel = bytes <= (size_t)(i1 - i0) * (384u << 10);
+        ChunkCopies up;
+        up.stream = pipe->in;
+        up.to_device = true;
         for (int i = i0; i < i1 && !st; ++i) {
             const gptq_host_problem_t &q = problems[i];
-            st = check(cudaMemcpyAsync(q.x_stage, q.x_host, (size_t)q.M * q.K * sizeof(__half), cudaMemcpyHostToDevice, pipe->in));
+            const size_t n = (size_t)q.M * q.K * sizeof(__half);
+            st = by_kernel ? up.add(q.x_stage, q.x_host, n)
+                           : check(cudaMemcpyAsync(q.x_stage, q.x_host, n, cudaMemcpyHostToDevice, pipe->in));
         }
+        if (!st) st = up.flush();
         if (!st) st = check(cudaEventRecord(ev_x[c], pipe->in));
         if (!st) st = check(cudaStreamWaitEvent(s, ev_x[c], 0));
         if (!st && wait_y >= 0) st = check(cudaStreamWaitEvent(s, ev_y[wait_y], 0));
@@ -875,10 +959,16 @@ static int host_batch(const gptq_host_problem_t *problems, int count, void *stre
         if (st) break;
         st = check(cudaEventRecord(ev_g[c], s));
         if (!st) st = check(cudaStreamWaitEvent(pipe->out, ev_g[c], 0));
+        ChunkCopies down;
+        down.stream = pipe->out;
+        down.to_device = false;
         for (int i = i0; i < i1 && !st; ++i) {
             const gptq_host_problem_t &q = problems[i];
-            st = check(cudaMemcpyAsync(q.y_host, q.y_stage, (size_t)q.M * q.N * sizeof(__half), cudaMemcpyDeviceToHost, pipe->out));
+            const size_t n = (size_t)q.M * q.N * sizeof(__half);
+            st = by_kernel && i1 == count ? down.add(q.y_host, q.y_stage, n)
+                           : check(cudaMemcpyAsync(q.y_host, q.y_stage, n, cudaMemcpyDeviceToHost, pipe->out));
         }
+        if (!st) st = down.flush();
         if (!st) st = check(cudaEventRecord(ev_y[c], pipe->out));
         i0 = i1;
     }

@@ -1480,3 +1480,31 @@ def test_w8_token_tiles(K, N, gs, M, ws):
     bound = 8 * sigma + 2.0 ** -11 * np.abs(want) + 1e-3
     err = np.abs(y - want)
     assert np.all(err[finite] <= bound[finite]), (err[finite] / bound[finite]).max()
+
+
+# ------------------------------------------------------------------------------- how a host batch moves its activations
+@pytest.mark.parametrize("M", [1, 3, 40])
+@pytest.mark.parametrize("count", [1, 8, 9, 21])
+def test_host_batch_copies(M, count, ws):
+    """Pinned, pageable and misaligned host buffers in one batch (copy kernel, asynchronous copies), chunks of one problem, a
+    full chunk and one more: each result is that of gptq_gemm on the device, bit for bit, and nothing around it changes."""
+    K, N = 512, 384
+    D = H.upload_and_repack(wl.make_linear(K, N, seed=wl.seed_for("host-copies")))
+    items, keep, want = [], [], []
+    for i in range(count):
+        x = torch.from_numpy(wl.make_x(M, K, wl.seed_for("host-copies-x", i, M)))
+        pad = 4 if i % 3 == 2 else 8                               # halves in front: 4 leaves the buffer off a 16-byte boundary
+        xh, yh = torch.zeros(M * K + 16, dtype=torch.float16), torch.full((M * N + 16,), 7.0, dtype=torch.float16)
+        if i % 3 != 1:
+            xh, yh = xh.pin_memory(), yh.pin_memory()
+        xh[pad:pad + M * K] = x.reshape(-1)
+        xs, ys = torch.empty((M, K), dtype=torch.float16, device="cuda"), torch.empty((M, N), dtype=torch.float16, device="cuda")
+        items.append((xh.data_ptr() + 2 * pad, D.qweight_t, D.qzeros_t, D.scales_t, None, yh.data_ptr() + 2 * pad, xs, ys, M, N, K, 128, 0))
+        keep.append((xh, yh, xs, ys, pad))
+        want.append(H.gemm(x.cuda(), D).cpu())
+    st, bad = B.gptq_gemm_host_batch(B.make_host_problems(items))
+    assert st == B.GPTQ_OK, bad
+    torch.cuda.synchronize()
+    for (xh, yh, xs, ys, pad), w in zip(keep, want):
+        assert torch.equal(yh[pad:pad + M * N].reshape(M, N), w)
+        assert bool((yh[:pad] == 7).all()) and bool((yh[pad + M * N:] == 7).all())

@@ -386,7 +386,7 @@ typedef struct {
     int kernel;       /* 1 = cluster split-K mma.sync kernel (gptq_gemm, M <= 16),
                          2 = tcgen05 kernel (gptq_gemm, M >= 17),
                          3 = stream-K mma.sync kernel (gptq_gemm_noalloc),
-                         4 = streaming tcgen05 decode kernel (gptq_gemm, M <= 4, see gptq_plan_decode) */
+                         4 = streaming tcgen05 decode kernel (gptq_gemm, M <= 2, see gptq_plan_decode) */
     int m_tile;       /* tokens per CTA tile */
     int m_chunks;     /* launches along M */
     int stages;       /* pipeline depth */
@@ -404,7 +404,7 @@ typedef struct {
 /* How the tile kernels (kernel 1 and 2) would launch this problem on a GPU with sm_count SMs: what gptq_gemm does, unless
  * gptq_plan_decode takes the problem. */
 int gptq_plan(int M, int N, int K, int group_size, int act_order, int sm_count, gptq_plan_t *out);
-/* The same for the streaming decode kernel (kernel 4), which takes fp16 problems of up to 4 token rows that fill the SMs;
+/* The same for the streaming decode kernel (kernel 4), which takes fp16 problems of one or two token rows that fill the SMs;
  * GPTQ_ERR_UNSUPPORTED for a problem that it leaves to the tile kernels.  `ctas` = clusters x cluster_size, each cluster
  * working through several panels; `stages` = depth of the weight ring in steps. */
 int gptq_plan_decode(int M, int N, int K, int group_size, int act_order, int sm_count, gptq_plan_t *out);

@@ -327,7 +327,7 @@ int gptq_plan_decode(int M, int N, int K, int group_size, int act_order, int sm_
     const DecodePlan pl = plan_decode(M, N, K, group_size, 0, 0, sm_count);
     if (!pl.use) return GPTQ_ERR_UNSUPPORTED;
     out->kernel = 4;
-    out->m_tile = pl.nx;
+    out->m_tile = kDecodeMaxRows;
     out->m_chunks = 1;
     out->stages = pl.w_slots;
     out->ctas = pl.ctas;
@@ -338,7 +338,7 @@ int gptq_plan_decode(int M, int N, int K, int group_size, int act_order, int sm_
     out->cluster_size = pl.S;
     out->tail_ctas = 0;
     out->tail_cluster_size = 1;
-    set_kernel_name(out, "decode_kernel<%d,%d>", pl.nx, pl.sub);
+    set_kernel_name(out, "decode_kernel<%d>", pl.sub);
     return GPTQ_OK;
 }
 

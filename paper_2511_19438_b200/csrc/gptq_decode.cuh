@@ -70,44 +70,34 @@ struct DecodeArgs {
     int slice_max;
 };
 
-// NX: token rows of a tile.  MMA N (eight B rows are read as sixteen: the accumulator columns of the rows behind them are
-// never looked at), accumulator columns of an item, items per step (two A stages, and two accumulators at least), and
-// accumulators in 256 columns.
-__host__ __device__ constexpr int decode_mma_n(int NX) { return NX < 4 ? 16 : 4 * NX; }
-__host__ __device__ constexpr int decode_d_cols(int NX, int SUB) { return SUB * decode_mma_n(NX); }
-__host__ __device__ constexpr int decode_step_items(int NX, int SUB)
+constexpr int kDecodeMaxRows = 2;            // token rows of a tile: eight B rows
+// MMA N (the eight B rows are read as sixteen: the accumulator columns of the rows behind them are never looked at),
+// accumulator columns of an item, items per step (two A stages, and two accumulators at least), and accumulators in 256
+// columns.
+constexpr int kDecodeN = 16;
+__host__ __device__ constexpr int decode_d_cols(int SUB) { return SUB * kDecodeN; }
+__host__ __device__ constexpr int decode_step_items(int SUB)
 {
-    return 4 * (kDecodeACols + decode_d_cols(NX, SUB)) <= (int)kDecodeCols ? 2 : 1;
+    return 4 * (kDecodeACols + decode_d_cols(SUB)) <= (int)kDecodeCols ? 2 : 1;
 }
-__host__ __device__ constexpr int decode_d_stages(int NX, int SUB)
+__host__ __device__ constexpr int decode_d_stages(int SUB)
 {
-    const int p = decode_step_items(NX, SUB);
-    return ((int)kDecodeCols - 2 * p * kDecodeACols) / (p * decode_d_cols(NX, SUB)) >= 4 ? 4 : 2;
+    const int p = decode_step_items(SUB);
+    return ((int)kDecodeCols - 2 * p * kDecodeACols) / (p * decode_d_cols(SUB)) >= 4 ? 4 : 2;
 }
-__host__ __device__ constexpr int decode_x_tile(int NX) { return NX * 512; }      // bytes of an item's B tile
-__host__ __device__ constexpr int decode_sum_bytes(int NX, int SUB, int items) { return (items * SUB * NX * 4 + 127) & ~127; }
+constexpr int kDecodeXTile = kDecodeMaxRows * 512;      // bytes of an item's B tile
+__host__ __device__ constexpr int decode_sum_bytes(int SUB, int items) { return (items * SUB * kDecodeMaxRows * 4 + 127) & ~127; }
 
-// token rows travel in vectors of 1, 2 or 4 values through the split-K exchange
-__host__ __device__ inline int decode_vec(int M) { return M >= 3 ? 4 : M; }
 __host__ __device__ inline int decode_recv_bytes(int M, int fuse, int S, int slice_max)      // of one of the two buffers
 {
-    const int v = decode_vec(M);
-    return (S * (fuse ? 2 : 1) * slice_max * ((M + v - 1) / v) * v * 4 + 127) & ~127;
+    return (S * (fuse ? 2 : 1) * slice_max * M * 4 + 127) & ~127;
 }
 
-__device__ __forceinline__ void st_async_vec(uint32_t addr, const float *v, int n, uint32_t bar)
+__device__ __forceinline__ void st_async_f32x2(uint32_t addr, float2 v, uint32_t bar)
 {
-    if (n == 4)
-        asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
-                     ::"r"(addr), "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(__float_as_uint(v[2])),
-                     "r"(__float_as_uint(v[3])), "r"(bar)
-                     : "memory");
-    else if (n == 2)
-        asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];"
-                     ::"r"(addr), "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(bar)
-                     : "memory");
-    else
-        st_async_f32(addr, v[0], bar);
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];"
+                 ::"r"(addr), "r"(__float_as_uint(v.x)), "r"(__float_as_uint(v.y)), "r"(bar)
+                 : "memory");
 }
 __device__ __forceinline__ void mbar_arrive_release_cluster(uint32_t cluster_addr)
 {
@@ -218,33 +208,24 @@ __device__ __forceinline__ void decode_store_pieces(uint32_t tile, int token, in
     }
 }
 
-template <int N>
-__device__ __forceinline__ void tmem_ld_cols(uint32_t taddr, uint32_t (&r)[N])
+__device__ __forceinline__ void tmem_ld_8(uint32_t taddr, uint32_t (&r)[8])
 {
-    static_assert(N == 8 || N == 16, "8 or 16 columns");
-    if constexpr (N == 8)
-        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-                     : "r"(taddr)
-                     : "memory");
-    else
-        asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-                       "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-                     : "r"(taddr)
-                     : "memory");
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr)
+                 : "memory");
 }
 
-// NX: token rows of a tile (2, 4); SUB: quantisation groups per item
-template <int NX, int SUB>
+// SUB: quantisation groups per item
+template <int SUB>
 __global__ void __launch_bounds__(kDecodeThreads, 2)
 decode_kernel(const DecodeArgs a, const __grid_constant__ CUtensorMap w_map)
 {
     extern __shared__ uint8_t smem_raw[];
-    constexpr int P = decode_step_items(NX, SUB);             // items per step
-    constexpr int ND = decode_d_stages(NX, SUB);              // accumulators (A stages: two, one per dequant set)
-    constexpr int kN = decode_mma_n(NX), kDCols = decode_d_cols(NX, SUB);      // columns per item
-    constexpr int kWSlot = P * kItemWBytes, kXTile = decode_x_tile(NX);
+    constexpr int P = decode_step_items(SUB);                 // items per step
+    constexpr int ND = decode_d_stages(SUB);              // accumulators (A stages: two, one per dequant set)
+    constexpr int kN = kDecodeN, kDCols = decode_d_cols(SUB);      // columns per item
+    constexpr int kWSlot = P * kItemWBytes, kXTile = kDecodeXTile, NX = kDecodeMaxRows;
     static_assert(P * (2 * kDecodeACols + ND * kDCols) <= (int)kDecodeCols, "tensor memory");
     constexpr int MC = kDecodeMetaItems / SUB;                // items per metadata chunk (whole steps)
     constexpr uint32_t kOffZ = kDecodeMetaItems * kItemSBytes;
@@ -266,7 +247,7 @@ decode_kernel(const DecodeArgs a, const __grid_constant__ CUtensorMap w_map)
     const uint32_t xtiles = wring + NW * kWSlot;
     const uint32_t meta = xtiles + a.x_tiles * kXTile;
     const uint32_t sums = meta + kDecodeMetaBufs * kDecodeMetaBytes;
-    const uint32_t recv = sums + decode_sum_bytes(NX, SUB, a.x_tiles);
+    const uint32_t recv = sums + decode_sum_bytes(SUB, a.x_tiles);
     const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const int S = a.S, cl = blockIdx.x / S, rank = blockIdx.x - cl * S;
     const int panels = a.N / kPanel;
@@ -276,9 +257,8 @@ decode_kernel(const DecodeArgs a, const __grid_constant__ CUtensorMap w_map)
     const int hsh = a.fuse ? 6 : 7, runs = a.fuse ? 2 : 1;              // `runs` runs of 2^hsh columns
     const int lo = (int)((a.slice_lo >> (8 * rank)) & 255);             // own columns of a run: [lo, lo + hw)
     const int hw = (rank + 1 < S ? (int)((a.slice_lo >> (8 * (rank + 1))) & 255) : (1 << hsh)) - lo;
-    const int V = decode_vec(a.M), MG = (a.M + V - 1) / V;
     const int wide = runs * a.slice_max;
-    const uint32_t recv_tx = (uint32_t)(S * runs * hw * MG * V * 4);
+    const uint32_t recv_tx = (uint32_t)(S * runs * hw * a.M * 4);
     const uint32_t recv_bytes = (uint32_t)decode_recv_bytes(a.M, a.fuse, S, a.slice_max);
     // the split of x goes in passes of 16 units (a unit: the 128 k of an item for one token, half a warp)
     constexpr int kUnits = kDecodeDequantWarps * 2;
@@ -513,14 +493,12 @@ decode_kernel(const DecodeArgs a, const __grid_constant__ CUtensorMap w_map)
         // this column's owner and place in the owner's receive buffer
         const int cc = n_col & ((1 << hsh) - 1), owner = ((cc + 1) * S - 1) >> hsh;
         const int pos = (n_col >> hsh) * a.slice_max + cc - (int)((a.slice_lo >> (8 * owner)) & 255);
-        const uint32_t dst = map_to_cluster_rank(recv, (uint32_t)owner) + (uint32_t)((rank * MG) * wide + pos) * (uint32_t)(V * 4);
+        const uint32_t dst = map_to_cluster_rank(recv, (uint32_t)owner) + (uint32_t)((rank * wide + pos) * a.M * 4);
         const uint32_t dbar = map_to_cluster_rank(bar_recv, (uint32_t)owner);
         constexpr uint32_t kSumItem = SUB * NX * 4;
         uint32_t mb = 0, mph = 0, sd = 0, dph = 0;
         for (int pi = 0; pi < n_panels; ++pi) {
-            uint64_t run[NX / 2];
-#pragma unroll
-            for (int m = 0; m < NX / 2; ++m) run[m] = 0;
+            uint64_t run = 0;
             uint32_t sum_at = sums;
             for (int c0 = 0; c0 < ng; c0 += MC) {
                 const int nc = (ng - c0) < MC ? (ng - c0) : MC;
@@ -549,48 +527,25 @@ decode_kernel(const DecodeArgs a, const __grid_constant__ CUtensorMap w_map)
                         __syncwarp();
                         if (lane == 0) mbar_arrive(bar_drained + 8 * sd);
                     };
-                    auto combine = [&](const uint32_t *r, int e, int j) {      // 8 columns: tokens 2 j, 2 j + 1 of group e
+                    auto combine = [&](const uint32_t (&r)[8], int e) {      // group e of the step
                         uint64_t v = fma_f32x2(pack_f32x2(r[6], r[7]), eighth, pack_f32x2(r[4], r[5]));
                         v = fma_f32x2(v, eighth, pack_f32x2(r[2], r[3]));
                         v = fma_f32x2(v, eighth, pack_f32x2(r[0], r[1]));
-                        v = fma_f32x2(nz[e], lds_f32x2(sum_at + (e % SUB) * (NX * 4) + j * 8), v);
-                        run[j] = fma_f32x2(sc[e], v, run[j]);
+                        v = fma_f32x2(nz[e], lds_f32x2(sum_at + e * (NX * 4)), v);
+                        run = fma_f32x2(sc[e], v, run);
                     };
-                    if constexpr (P == 2 && SUB == 1 && NX <= 4) {
-                        constexpr int kC = 4 * NX;
-                        uint32_t r0[kC], r1[kC];
-                        tmem_ld_cols<kC>(d0, r0);
-                        tmem_ld_cols<kC>(d0 + kDCols, r1);       // (garbage behind a lone last item)
+                    // all groups of the step at once, two at a time (garbage behind a lone last item)
+#pragma unroll
+                    for (int e = 0; e < P * SUB; e += 2) {
+                        uint32_t r0[8], r1[8];
+                        tmem_ld_8(d0 + e * kN, r0);
+                        tmem_ld_8(d0 + (e + 1) * kN, r1);
                         tmem_wait_ld();
-                        drained();
-#pragma unroll
-                        for (int j = 0; j < NX / 2; ++j) combine(r0 + 8 * j, 0, j);
-                        sum_at += kSumItem;
-                        if (two) {
-#pragma unroll
-                            for (int j = 0; j < NX / 2; ++j) combine(r1 + 8 * j, 1, j);
-                            sum_at += kSumItem;
-                            }
-                    } else {
-                        constexpr int kC = NX == 2 ? 8 : 16;         // accumulator columns at a time
-#pragma unroll
-                        for (int e = 0; e < P * SUB; ++e) {
-                            if (e < SUB || two) {
-#pragma unroll
-                                for (int c = 0; c < 4 * NX; c += kC) {
-                                    uint32_t r[kC];
-                                    tmem_ld_cols<kC>(d0 + (e / SUB) * kDCols + (e % SUB) * kN + c, r);
-                                    tmem_wait_ld();
-                                    if (c + kC == 4 * NX && e == (two ? P * SUB : SUB) - 1) drained();
-#pragma unroll
-                                    for (int j = 0; j < kC / 8; ++j) combine(r + 8 * j, e, c / 8 + j);
-                                }
-                                if (e % SUB == SUB - 1) {
-                                    sum_at += kSumItem;
-                                            }
-                            }
-                        }
+                        if (e + 2 == P * SUB) drained();
+                        if (e < SUB || two) combine(r0, e);
+                        if (e + 1 < SUB || two) combine(r1, e + 1);
                     }
+                    sum_at += P * kSumItem;
                     if (++sd == ND) { sd = 0; dph ^= 1u; }
                 }
                 __syncwarp();
@@ -605,22 +560,9 @@ decode_kernel(const DecodeArgs a, const __grid_constant__ CUtensorMap w_map)
             } else if (pi >= 2) {
                 decode_wait_cluster(bar_free + 8 * buf, (uint32_t)((pi >> 1) - 1) & 1u, flag);   // the owners have read panel pi - 2
             }
-            float v[NX];
-#pragma unroll
-            for (int j = 0; j < NX / 2; ++j) {
-                const float2 f = unpack_f32x2(run[j]);
-                v[2 * j] = f.x * 512.f;             // nibbles were q * 2^-9
-                v[2 * j + 1] = f.y * 512.f;
-            }
-            const uint32_t to = dst + buf * recv_bytes, tobar = dbar + 8 * buf;
-            if constexpr (NX == 2) {
-                if (V == 2) st_async_vec(to, v, 2, tobar);
-                else st_async_f32(to, v[0], tobar);
-            } else {
-#pragma unroll
-                for (int m = 0; m < NX; m += 4)
-                    if (m < a.M) st_async_vec(to + (uint32_t)(m / 4 * wide) * 16u, v + m, 4, tobar);
-            }
+            const float2 f = unpack_f32x2(run);     // nibbles were q * 2^-9
+            if (a.M == 2) st_async_f32x2(dst + buf * recv_bytes, make_float2(f.x * 512.f, f.y * 512.f), dbar + 8 * buf);
+            else st_async_f32(dst + buf * recv_bytes, f.x * 512.f, dbar + 8 * buf);
         }
     } else {
         // ---------------------------------------------------------------- finish: the own column slice of each panel
@@ -633,50 +575,31 @@ decode_kernel(const DecodeArgs a, const __grid_constant__ CUtensorMap w_map)
             const uint32_t buf = (uint32_t)pi & 1u;
             decode_wait_cluster(bar_recv + 8 * buf, (uint32_t)(pi >> 1) & 1u, flag);
             if (layout_ok && lds32(flag) == 0) {
-                // a thread takes V token rows of one column (with fuse: of a gate column and its up column)
-                for (int idx = lane; idx < MG * hw; idx += 32) {
-                    const int mg = idx / hw, j = idx - mg * hw;
-                    auto slice_sum = [&](int jj, float (&sum)[4]) {   // sender order
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) sum[e] = 0.f;
-                        const uint32_t at = recv + buf * recv_bytes + (uint32_t)(mg * wide + jj) * (uint32_t)(V * 4);
-                        const uint32_t step = (uint32_t)(MG * wide * V * 4);
+                // a thread takes one column (with fuse: a gate column and its up column) of one token
+                for (int idx = lane; idx < a.M * hw; idx += 32) {
+                    const int j = a.M == 2 ? idx >> 1 : idx, m = a.M == 2 ? idx & 1 : 0;
+                    auto slice_sum = [&](int jj) {   // sender order
+                        const uint32_t at = recv + buf * recv_bytes + (uint32_t)(jj * a.M + m) * 4u, step = (uint32_t)(wide * a.M) * 4u;
+                        float sum = 0.f;
 #pragma unroll
                         for (int sdr = 0; sdr < 8; ++sdr) {
                             if (sdr >= S) break;
-                            if (V == 4) {
-                                const uint4 w = lds128(at + sdr * step);
-                                sum[0] += __uint_as_float(w.x), sum[1] += __uint_as_float(w.y);
-                                sum[2] += __uint_as_float(w.z), sum[3] += __uint_as_float(w.w);
-                            } else {
-                                sum[0] += lds_f32(at + sdr * step);
-                                if (V == 2) sum[1] += lds_f32(at + sdr * step + 4);
-                            }
+                            sum += lds_f32(at + sdr * step);
                         }
+                        return sum;
                     };
-                    float v[4], up[4];
-                    slice_sum(j, v);
                     if (!a.fuse) {
                         const int n = p * kPanel + lo + j;
-                        const float bv = a.bias ? __half2float(a.bias[n]) : 0.f;
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            const int m = mg * V + e;
-                            if (e < V && m < a.M) {
-                                float o = v[e] + bv;
-                                if (a.residual) o += __half2float(a.residual[(size_t)m * a.N + n]);
-                                a.y[(size_t)m * a.N + n] = __float2half_rn(o);
-                            }
+                        float v = slice_sum(j);
+                        if (a.bias || a.residual) {
+                            v += (a.bias ? __half2float(a.bias[n]) : 0.f);
+                            if (a.residual) v += __half2float(a.residual[(size_t)m * a.N + n]);
                         }
+                        a.y[(size_t)m * a.N + n] = __float2half_rn(v);
                     } else {
-                        slice_sum(a.slice_max + j, up);
                         const int oc = p * 64 + lo + j;
-                        __half *out = a.y + (a.out_index ? a.out_index[oc] : oc);
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            const int m = mg * V + e;
-                            if (e < V && m < a.M) out[(size_t)m * (a.N / 2)] = __float2half_rn(silu_mul(v[e], up[e]));
-                        }
+                        a.y[(size_t)m * (a.N / 2) + (a.out_index ? a.out_index[oc] : oc)] =
+                            __float2half_rn(silu_mul(slice_sum(j), slice_sum(a.slice_max + j)));
                     }
                 }
             }
@@ -706,11 +629,9 @@ decode_kernel(const DecodeArgs a, const __grid_constant__ CUtensorMap w_map)
     }
 }
 
-constexpr int kDecodeMaxRows = 2;
-
 struct DecodePlan {
     bool use;       // else the mma.sync kernel takes the problem
-    int nx, sub;
+    int sub;
     int S, clusters, ctas;
     int w_slots, x_tiles, smem_bytes;
 };
@@ -729,18 +650,17 @@ inline DecodePlan plan_decode(int M, int N, int K, int group_size, int fuse, int
     DecodePlan pl{};
     const int G = K / kGroup, panels = N / kPanel;
     pl.sub = kGroup / group_size;
-    pl.nx = M <= 2 ? 2 : 4;
     if (bf16 || M > kDecodeMaxRows) return pl;
     const int budget = (227 * 1024) / 2 - 1024;                          // two launches share an SM
-    const int tile = decode_x_tile(pl.nx), step = decode_step_items(pl.nx, pl.sub) * kItemWBytes;
+    const int tile = kDecodeXTile, step = decode_step_items(pl.sub) * kItemWBytes;
     // Estimated times in microseconds, fitted to 80 shapes (K = 1024 .. 13824, N = 1024 .. 27648; the chosen kernel is within
     // 2 % of the better one on average).  Here: the busiest CTA's items.  The mma.sync kernel: the layer's items spread over
     // the SMs, but one CTA's own pace where its grid leaves one CTA per SM.  At M = 1, there and here: 4096 x 6144 5.8 and
     // 6.3 us, 1024 x 3072 2.8 and 3.4; 4096 x 4096 4.7 and 4.1, 4096 x 12288 8.3 and 7.4, 8192 x 2048 8.8 and 5.1,
     // 4096 x 22016 12.8 and 11.4, 13824 x 27648 42.3 and 35.3.
-    const double per_item = M <= 2 ? 0.21 : 0.22, fixed_time = M <= 2 ? 2.6 : 3.0;
+    const double per_item = 0.21, fixed_time = 2.6;
     const SplitKPlan sk = plan_splitk(M, N, K, group_size, sm_count);
-    const double spread = 0.0021 * panels * G, serial = sk.ctas <= sm_count ? (M <= 2 ? 0.6 : 0.75) * ((G + sk.S - 1) / sk.S) : 0;
+    const double spread = 0.0021 * panels * G, serial = sk.ctas <= sm_count ? 0.6 * ((G + sk.S - 1) / sk.S) : 0;
     const double other = 2.2 + (spread > serial ? spread : serial);
     double best = -1;
     int items = 0;      // of the busiest CTA
@@ -751,7 +671,7 @@ inline DecodePlan plan_decode(int M, int N, int K, int group_size, int fuse, int
         const int ng = (G + S - 1) / S;                                  // items of the busiest CTA, per panel
         // the B tiles of the CTA's K range have to leave four steps of weights
         const int fixed = 2048 + kDecodeMetaBufs * kDecodeMetaBytes + 2 * decode_recv_bytes(M, fuse, S, ((fuse ? 64 : kPanel) + S - 1) / S) +
-                          ng * tile + decode_sum_bytes(pl.nx, pl.sub, ng);
+                          ng * tile + decode_sum_bytes(pl.sub, ng);
         int slots = (budget - fixed) / step;
         if (ng > kDecodeMaxItems || ng * M > 16 * kDecodeMaxXPasses || slots < 4) continue;
         const double t = fixed_time + per_item * ppc * ng + 0.1 * ppc + (S > 1 ? 0.1 : 0);
@@ -772,11 +692,11 @@ inline DecodePlan plan_decode(int M, int N, int K, int group_size, int fuse, int
     return pl;
 }
 
-template <int NX, int SUB>
-static int launch_decode_nx(const DecodeArgs &args, const CUtensorMap &w_map, const DecodePlan &plan, cudaStream_t s)
+template <int SUB>
+static int launch_decode_sub(const DecodeArgs &args, const CUtensorMap &w_map, const DecodePlan &plan, cudaStream_t s)
 {
     static int configured_smem[64] = {};
-    const int cfg_st = ensure_dynamic_smem((const void *)decode_kernel<NX, SUB>, configured_smem, plan.smem_bytes);
+    const int cfg_st = ensure_dynamic_smem((const void *)decode_kernel<SUB>, configured_smem, plan.smem_bytes);
     if (cfg_st) return cfg_st;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)plan.ctas);
@@ -794,7 +714,7 @@ static int launch_decode_nx(const DecodeArgs &args, const CUtensorMap &w_map, co
     attr[2].val.clusterSchedulingPolicyPreference = cudaClusterSchedulingPolicyLoadBalancing;
     cfg.attrs = attr;
     cfg.numAttrs = 3;
-    return record_cuda_error(cudaLaunchKernelEx(&cfg, decode_kernel<NX, SUB>, args, w_map));
+    return record_cuda_error(cudaLaunchKernelEx(&cfg, decode_kernel<SUB>, args, w_map));
 }
 
 int launch_decode(const __half *x, const void *qweight, const void *qzeros, const void *scales, __half *y, int M, int N, int K,
@@ -826,13 +746,10 @@ int launch_decode(const __half *x, const void *qweight, const void *qzeros, cons
     const int st = make_tensor_map_2d(&w_map, CU_TENSOR_MAP_DATA_TYPE_UINT32, qweight, 16, (uint64_t)K * N / 2 / 64, 64, 16, 128,
                                       CU_TENSOR_MAP_SWIZZLE_64B);
     if (st) return st;
-    switch (plan.nx * 10 + plan.sub) {
-    case 21: return launch_decode_nx<2, 1>(args, w_map, plan, s);
-    case 22: return launch_decode_nx<2, 2>(args, w_map, plan, s);
-    case 24: return launch_decode_nx<2, 4>(args, w_map, plan, s);
-    case 41: return launch_decode_nx<4, 1>(args, w_map, plan, s);
-    case 42: return launch_decode_nx<4, 2>(args, w_map, plan, s);
-    case 44: return launch_decode_nx<4, 4>(args, w_map, plan, s);
+    switch (plan.sub) {
+    case 1: return launch_decode_sub<1>(args, w_map, plan, s);
+    case 2: return launch_decode_sub<2>(args, w_map, plan, s);
+    case 4: return launch_decode_sub<4>(args, w_map, plan, s);
     default: return GPTQ_ERR_UNSUPPORTED;
     }
 }

@@ -230,10 +230,15 @@ def launches_per_gemm(spec, M, name, sm_count):
     from paper_2511_19438_b200 import binding as B
     K, N = spec["shapes"][name]
     if spec.get("w8", False):       # the 4-bit kernels on the stacked planes (2 K rows), always behind the x gather
+        if B.gptq_plan_prefill(M, N, K, wl.GROUP_SIZE, 0, 1, sm_count)[0] == B.GPTQ_OK:
+            return 2
         st, pl = B.gptq_plan(M, N, 2 * K if M <= 16 else K, wl.GROUP_SIZE, 0, sm_count)     # from 17 rows on: both planes at once
         assert st == B.GPTQ_OK
         return 2 + (1 if pl.tail_ctas > 0 else 0)
-    st, pl = B.gptq_plan(M, N, K, wl.GROUP_SIZE, 1 if spec["act_order"] else 0, sm_count)
+    act = 1 if spec["act_order"] else 0
+    st, pl = B.gptq_plan_prefill(M, N, K, wl.GROUP_SIZE, act, 0, sm_count)
+    if st != B.GPTQ_OK:
+        st, pl = B.gptq_plan(M, N, K, wl.GROUP_SIZE, act, sm_count)
     assert st == B.GPTQ_OK
     return 1 + (1 if pl.tail_ctas > 0 else 0) + (1 if spec["act_order"] else 0)
 
@@ -249,6 +254,8 @@ def kernel_of(spec, M, sm_count):
         act = 1 if spec["act_order"] else 0
         st, pl = B.gptq_plan_decode(M, N, K, wl.GROUP_SIZE, act, sm_count)
         if st != B.GPTQ_OK or spec.get("bf16", False):
+            st, pl = B.gptq_plan_prefill(M, N, K, wl.GROUP_SIZE, act, spec.get("w8", False), sm_count)
+        if st != B.GPTQ_OK:
             st, pl = B.gptq_plan(M, N, K, wl.GROUP_SIZE, act, sm_count)
         assert st == B.GPTQ_OK
         names[B.plan_kernel_name(pl)] = names.get(B.plan_kernel_name(pl), 0) + K * N

@@ -386,7 +386,8 @@ typedef struct {
     int kernel;       /* 1 = cluster split-K mma.sync kernel (gptq_gemm, M <= 16),
                          2 = tcgen05 kernel (gptq_gemm, M >= 17),
                          3 = stream-K mma.sync kernel (gptq_gemm_noalloc),
-                         4 = streaming tcgen05 decode kernel (gptq_gemm, M <= 2, see gptq_plan_decode) */
+                         4 = streaming tcgen05 decode kernel (gptq_gemm, M <= 2, see gptq_plan_decode),
+                         5 = persistent tcgen05 kernel (gptq_gemm, M >= 17, see gptq_plan_prefill) */
     int m_tile;       /* tokens per CTA tile */
     int m_chunks;     /* launches along M */
     int stages;       /* pipeline depth */
@@ -402,12 +403,16 @@ typedef struct {
 } gptq_plan_t;
 
 /* How the tile kernels (kernel 1 and 2) would launch this problem on a GPU with sm_count SMs: what gptq_gemm does, unless
- * gptq_plan_decode takes the problem. */
+ * gptq_plan_decode or gptq_plan_prefill takes the problem. */
 int gptq_plan(int M, int N, int K, int group_size, int act_order, int sm_count, gptq_plan_t *out);
 /* The same for the streaming decode kernel (kernel 4), which takes fp16 problems of one or two token rows that fill the SMs;
  * GPTQ_ERR_UNSUPPORTED for a problem that it leaves to the tile kernels.  `ctas` = clusters x cluster_size, each cluster
  * working through several panels; `stages` = depth of the weight ring in steps. */
 int gptq_plan_decode(int M, int N, int K, int group_size, int act_order, int sm_count, gptq_plan_t *out);
+/* The same for the persistent kernel (kernel 5), which takes problems of 17 and more token rows unless a split of K over
+ * clusters (kernel 2) is estimated faster; eight_bit is nonzero for gptq_gemm_w8.  `m_tile` = token rows per tile, `stages` =
+ * depth of the x ring in 128-row items. */
+int gptq_plan_prefill(int M, int N, int K, int group_size, int act_order, int eight_bit, int sm_count, gptq_plan_t *out);
 /* The same for gptq_gemm_noalloc (stream-K kernel; workspace_bytes is its need of the built-in scratch). */
 int gptq_plan_noalloc(int M, int N, int K, int group_size, int act_order, int sm_count, gptq_plan_t *out);
 

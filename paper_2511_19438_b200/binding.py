@@ -98,6 +98,7 @@ _SIGNATURES = {
     "gptq_trace_read": (_i, [_vp, _i, _vp]),
     "gptq_plan": (_i, [_i, _i, _i, _i, _i, _i, ctypes.POINTER(gptq_plan_t)]),
     "gptq_plan_decode": (_i, [_i, _i, _i, _i, _i, _i, ctypes.POINTER(gptq_plan_t)]),
+    "gptq_plan_prefill": (_i, [_i, _i, _i, _i, _i, _i, _i, ctypes.POINTER(gptq_plan_t)]),
     "gptq_plan_noalloc": (_i, [_i, _i, _i, _i, _i, _i, ctypes.POINTER(gptq_plan_t)]),
     "gptq_plan_cta_range": (_i, [_i, _i, _i, ctypes.POINTER(_i), ctypes.POINTER(_i)]),
     "gptq_plan_panel_owners": (_i, [_i, _i, _i, _i, ctypes.POINTER(_i), ctypes.POINTER(_i)]),
@@ -364,6 +365,12 @@ def gptq_plan(M, N, K, group_size, act_order, sm_count):
 def gptq_plan_decode(M, N, K, group_size, act_order, sm_count):
     plan = gptq_plan_t()
     st = _lib.gptq_plan_decode(M, N, K, group_size, int(act_order), sm_count, ctypes.byref(plan))
+    return st, plan
+
+
+def gptq_plan_prefill(M, N, K, group_size, act_order, eight_bit, sm_count):
+    plan = gptq_plan_t()
+    st = _lib.gptq_plan_prefill(M, N, K, group_size, int(act_order), int(eight_bit), sm_count, ctypes.byref(plan))
     return st, plan
 
 

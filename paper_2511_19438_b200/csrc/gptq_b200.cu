@@ -6,6 +6,7 @@
 #include "gptq_splitk.cuh"
 #include "gptq_umma.cuh"
 #include "gptq_decode.cuh"
+#include "gptq_prefill.cuh"
 #include "gptq_umma2.cuh"
 #include "gptq_w8.cuh"
 #include "gptq_wn.cuh"
@@ -342,6 +343,32 @@ int gptq_plan_decode(int M, int N, int K, int group_size, int act_order, int sm_
     return GPTQ_OK;
 }
 
+int gptq_plan_prefill(int M, int N, int K, int group_size, int act_order, int eight_bit, int sm_count, gptq_plan_t *out)
+{
+    if (!out) return GPTQ_ERR_NULL;
+    int st = check_shape(M, N, K, group_size);
+    if (st) return st;
+    st = check_fast_path(N, K, group_size);
+    if (st) return st;
+    if (sm_count < 1) return GPTQ_ERR_SHAPE;
+    const PrefillPlan pl = plan_prefill(M, N, K, sm_count, eight_bit != 0);
+    if (M < kUmmaMinTokens || !pl.use) return GPTQ_ERR_UNSUPPORTED;
+    out->kernel = 5;
+    out->m_tile = pl.tok;
+    out->m_chunks = 1;
+    out->stages = pl.x_slots;
+    out->ctas = pl.ctas;
+    out->items = (N / kPanel) * (K / kGroup);
+    out->split_panels = 0;
+    out->smem_bytes = pl.smem_bytes;
+    out->workspace_bytes = gemm_workspace_need(M, eight_bit ? 2 * K : K, eight_bit ? 1 : act_order);
+    out->cluster_size = 1;
+    out->tail_ctas = 0;
+    out->tail_cluster_size = 1;
+    set_kernel_name(out, "prefill_kernel<%d>", kGroup / group_size);
+    return GPTQ_OK;
+}
+
 int gptq_plan_noalloc(int M, int N, int K, int group_size, int act_order, int sm_count, gptq_plan_t *out)
 {
     if (!out) return GPTQ_ERR_NULL;
@@ -453,7 +480,10 @@ static int gemm_dispatch(const void *x, const void *qweight, const void *qzeros,
             const Umma2Plan p2 = plan_umma2(M, N, K);
             return launch_umma2(xin, qweight, qzeros, scales, (__half *)y, M, N, K, p2, s);
         }
-        // tcgen05 kernel: 32- to 256-token tiles
+        if (const PrefillPlan pp = plan_prefill(M, N, K, sms, false); pp.use)      // one CTA per SM, no split of K
+            return launch_prefill(xin, qweight, qzeros, scales, (__half *)y, M, N, K, group_size, pp, fuse, (const __half *)bias,
+                                  (const __half *)residual, out_index, bf16, 0, s);
+        // few tiles and a long K: 32- to 256-token tiles, K split over clusters
         const UmmaPlan pl = plan_umma(M, N, K, sms);
         return launch_umma(xin, qweight, qzeros, scales, (__half *)y, M, N, K, group_size, pl, fuse, (const __half *)bias,
                            (const __half *)residual, out_index, bf16, 0, s);
@@ -594,6 +624,9 @@ int gptq_gemm_w8(const void *x, const void *qweight, const void *qzeros, const v
         // the tcgen05 kernel joins the planes itself: x once, in the row order of either plane
         st = launch_gather_x((const __half *)x, perm, (__half *)ws.ptr, M, K, (cudaStream_t)stream);
         if (st) return st;
+        if (const PrefillPlan pp = plan_prefill(M, N, K, sms, true); pp.use)
+            return launch_prefill((const __half *)ws.ptr, qweight, qzeros, scales, (__half *)y, M, N, K, tiled, pp, 0, nullptr,
+                                  nullptr, nullptr, 0, 1, (cudaStream_t)stream);
         return launch_umma((const __half *)ws.ptr, qweight, qzeros, scales, (__half *)y, M, N, K, tiled,
                            plan_umma(M, N, K, sms, true), 0, nullptr, nullptr, nullptr, 0, 1, (cudaStream_t)stream);
     }

@@ -1,0 +1,580 @@
+// Persistent tcgen05 GPTQ matmul for 17 token rows and more: what the kernel of gptq_umma.cuh does, for problems whose tiles
+// fill the SMs without a split of K.
+//
+// As there, the 128 columns of a panel are the MMA's rows, dequantised into a ring of A stages in tensor memory, and a tile of
+// token rows is its N.  An item (128 rows of K of a panel, 8 KB of packed weights) is the unit of every hand-over.  What differs:
+//   * One CTA per SM works through its tiles without leaving the kernel.  Tensor memory holds two accumulators of up to 160
+//     token rows beside the A stages, so the epilogue of a tile (four warps of its own) runs under the main loop of the next
+//     one, and the rings never drain between tiles.  The last tile, with nothing to hide under, is shared out over all 20
+//     epilogue and dequant warps.
+//   * The number of token rows of a tile is a run-time multiple of 16, so that tiles and waves come out even: 300 rows on 96
+//     panels are three tiles of 112 in two waves, where tiles of 256 cost two waves of 256.
+//   * Four sets of four dequant warps take every fourth item each: a set's pass takes about 1000 clocks, most of it latency.
+//   * x lands on the barrier of its item's A stage, so the MMA thread has one wait per item; weights run ahead in a ring of
+//     their own (and start before the previous kernel has finished).
+// What bounds it.  From 128 token rows per tile the MMA: 572 clocks per item of 512 at full rate (qkv M = 512), and then the
+// power limit (1.45-1.5 GHz in that loop).  With fewer rows the MMA thread: about 520 clocks per item for one wait, eight MMAs
+// and a commit.  Its cost is instruction fetch (a fetch group at a time, with five other warps on its scheduler), hence the
+// short loop in one elected thread (846 -> 589 clocks per item against a warp that elects for every item, o M = 512) and the
+// rolled dequant loop.  Stages of a tile of 176 or 192 rows (only two fit beside the accumulators) made the hand-over the
+// limit: 811 clocks per item of 704.
+// Measured (7B layer of four matmuls in a chain, us, kernel of gptq_umma.cuh -> this): M = 64 71.6 -> 60.2, M = 128 82 -> 71,
+// M = 300 177 -> 120, M = 512 212 -> 172, 8-bit M = 300 232 -> 164.
+#pragma once
+#include "gptq_decode.cuh"      // waits with a CTA-wide flag
+
+namespace gptq {
+
+constexpr int kPrefillSets = 4;                                      // dequant warp sets
+constexpr int kPrefillMaxTok = 160;
+// warps: x producer, MMA, epilogue x 4, dequant x 16, weight producer
+constexpr int kPrefillXWarp = 0, kPrefillFirstEpi = 2, kPrefillFirstDq = 6, kPrefillWWarp = kPrefillFirstDq + 4 * kPrefillSets;
+constexpr int kPrefillThreads = 32 * (kPrefillWWarp + 1);
+constexpr int kPrefillStage = 4 * 32 * 64;                           // epilogue: 32 tokens x 64 bytes per warp
+// A stages (of one item, 64 columns) and columns of an accumulator: tensor memory holds 2 x 128 + 4 x 64 or 2 x 160 + 3 x 64
+__host__ __device__ constexpr int prefill_a_stages(int tok) { return tok <= 128 ? 4 : 3; }
+__host__ __device__ constexpr int prefill_acc_columns(int tok) { return tok <= 128 ? 128 : 160; }
+// Weight slots.  A set's parity wait on a slot needs the slot's previous item to be in: with this many that is known, the
+// set's last pass (four items ago) has waited for the MMAs of the item that had its A stage before.  With 8-bit weights
+// (16 KB per slot) five, and the set asks.
+__host__ __device__ constexpr int prefill_w_slots(int tok, bool w8) { return w8 ? 5 : kPrefillSets + prefill_a_stages(tok); }
+
+// 16 lanes x 32 columns of tensor memory as four 8-column groups: r[4 g], r[4 g + 1] are lane T / 4, columns 8 g + 2 (T % 4) and
+// the next one, r[4 g + 2], r[4 g + 3] the same of lane T / 4 + 8 (T: thread of the warp)
+__device__ __forceinline__ void tmem_ld_16x256b_x4(uint32_t taddr, uint32_t (&r)[16])
+{
+    asm volatile("tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+                   "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+                 : "r"(taddr)
+                 : "memory");
+}
+__device__ __forceinline__ void stmatrix_x4_trans(uint32_t addr, const uint32_t (&r)[4])
+{
+    asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1,%2,%3,%4};" ::"r"(addr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3])
+                 : "memory");
+}
+__device__ __forceinline__ void ldmatrix_x4_trans(uint32_t addr, uint32_t (&r)[4])
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void sts128(uint32_t addr, uint4 v)
+{
+    asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+}
+template <bool BF>
+__device__ __forceinline__ uint32_t pack_out16(float2 v)
+{
+    if constexpr (BF) {
+        const __nv_bfloat162 b = __floats2bfloat162_rn(v.x, v.y);
+        return *reinterpret_cast<const uint32_t *>(&b);
+    } else {
+        const __half2 h = __floats2half2_rn(v.x, v.y);
+        return *reinterpret_cast<const uint32_t *>(&h);
+    }
+}
+
+struct PrefillArgs {
+    const uint8_t *scales, *qzeros;   // tiled
+    __half *y;
+    int M, N, G;                      // G: 128-row items of K (of one plane with 8-bit weights)
+    int tok, tiles, x_slots;          // token rows per tile; tiles; depth of the x ring in items (at most the A stages)
+    const TiledTrailer *trailer;
+    int fuse;
+    const __half *bias, *residual;
+    int trace_slot;
+    const int32_t *out_index;
+};
+
+template <int SUB, bool BF, bool W8>
+__global__ void __launch_bounds__(kPrefillThreads, 1)
+prefill_kernel(const PrefillArgs a, const __grid_constant__ CUtensorMap w_map, const __grid_constant__ CUtensorMap x_map)
+{
+    extern __shared__ uint8_t smem_raw[];
+    constexpr int PL = W8 ? 2 : 1;                            // nibble planes
+    const uint32_t flags = __ldg(&a.trailer->flags);          // needed late: requested first
+    if (threadIdx.x == 0) {
+        GPTQ_TRACE_MIN(a.trace_slot, first_entry);
+        GPTQ_TRACE_MAX(a.trace_slot, last_entry);
+        if (blockIdx.x == 0) {
+            GPTQ_TRACE_SET(a.trace_slot, kernel_and_ctas, (2ull << 32) | gridDim.x);
+        }
+    }
+    const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    // wfull[s]: packed weights of a ring slot have landed; afull[k]: A stage k has been written and the item's x has landed;
+    // done[n mod 16]: the MMAs of the CTA's n-th item have completed; dfull / dempty: accumulators
+    const uint32_t bar_wfull = base, bar_afull = base + 128, bar_done = base + 192, bar_dfull = base + 320,
+                   bar_dempty = base + 336;
+    const uint32_t tmem_slot = base + 352, flag = base + 356;
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+    const int tok = a.tok, G = a.G, panels = a.N / kPanel, XS = a.x_slots;
+    const int PS = prefill_a_stages(tok), WS = prefill_w_slots(tok, W8), acc = prefill_acc_columns(tok);
+    constexpr uint32_t kWSlot = PL * kItemWBytes;
+    const uint32_t x_half = (uint32_t)tok * 128, x_slot = 2 * x_half;       // an item's x: two K64 tiles
+    const uint32_t stg0 = base + 1024, w_ring = stg0 + kPrefillStage, x_ring = w_ring + WS * kWSlot;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < WS; ++s) mbar_init(bar_wfull + 8 * s, 1);
+        for (int s = 0; s < PS; ++s) mbar_init(bar_afull + 8 * s, 5);
+        for (int s = 0; s < kUmmaDoneRing; ++s) mbar_init(bar_done + 8 * s, 1);
+        for (int s = 0; s < 2; ++s) {
+            mbar_init(bar_dfull + 8 * s, 1);
+            mbar_init(bar_dempty + 8 * s, 4);
+        }
+        asm volatile("st.shared.u32 [%0], %1;" ::"r"(flag), "r"(0u) : "memory");
+        fence_barrier_init();
+        fence_proxy_async();
+    }
+    if (warp == 1) {
+        tmem_alloc(tmem_slot, 512);
+        tmem_relinquish();
+    }
+    tc_fence_before_sync();
+    __syncthreads();
+    tc_fence_after_sync();
+    const uint32_t tmem_base = __shfl_sync(0xffffffffu, lds32(tmem_slot), 0);
+    pdl_launch_dependents();
+
+    const bool is_dq = warp >= kPrefillFirstDq && warp < kPrefillWWarp, is_epi = warp >= kPrefillFirstEpi && warp < kPrefillFirstDq;
+    auto wait_done = [&](int n) { decode_wait(bar_done + 8 * (n & (kUmmaDoneRing - 1)), (uint32_t)(n / kUmmaDoneRing) & 1u, flag); };
+
+    if (warp == kPrefillXWarp || warp == kPrefillWWarp) {
+        // ---------------------------------------------------------------- TMA producers (one thread issues): x tiles and
+        // packed weights by a warp each
+        const bool xw = warp == kPrefillXWarp;
+        if (elect_one()) tma_prefetch_descriptor(xw ? &x_map : &w_map);
+        if (xw) {
+            pdl_wait();                  // weights do not depend on earlier kernels
+            GPTQ_TRACE_MIN(a.trace_slot, first_wait_done);
+            GPTQ_TRACE_MAX(a.trace_slot, last_wait_done);
+        } else {
+            GPTQ_TRACE_MIN(a.trace_slot, first_weight_issue);
+        }
+        const int NS = xw ? XS : WS;
+        int s = 0, n = 0, sa = 0;
+        for (int tile = blockIdx.x; tile < a.tiles; tile += gridDim.x) {
+            const int mt = tile / panels, p = tile - mt * panels;       // neighbouring CTAs share the x tile
+            for (int t = 0; t < G; ++t, ++n) {
+                if (n >= NS) wait_done(n - NS);
+                if (elect_one()) {
+                    if (xw) {
+                        // (the A stage's last item has been multiplied: there are at least as many stages as x slots)
+                        mbar_arrive_expect_tx(bar_afull + 8 * sa, x_slot);
+                        tma_load_3d(x_ring + s * x_slot, &x_map, 0, mt * tok, 2 * t, bar_afull + 8 * sa);     // rows >= M read as zero
+                    } else {
+                        // packed weights as rows of 64 bytes, 128 to an item
+                        mbar_arrive_expect_tx(bar_wfull + 8 * s, kWSlot);
+#pragma unroll
+                        for (int pl = 0; pl < PL; ++pl)
+                            tma_load_2d(w_ring + s * kWSlot + pl * kItemWBytes, &w_map, 0, (G * (PL * p + pl) + t) * 128, bar_wfull + 8 * s);
+                    }
+                }
+                __syncwarp();
+                if (++s == NS) s = 0;
+                if (++sa == PS) sa = 0;
+            }
+        }
+    } else if (warp == 1) {
+        // ---------------------------------------------------------------- MMA (one thread issues)
+        const uint32_t idesc = umma_idesc_f16(128, tok) | (BF ? kUmmaIdescBf16 : 0u);
+        if (elect_one()) {
+            const uint64_t desc0 = umma_desc_k_major_sw128(x_ring);
+            const uint32_t desc_lo = (uint32_t)desc0, desc_hi = (uint32_t)(desc0 >> 32);      // (the address field is in the low word)
+            const uint32_t x_step = x_slot >> 4, half_step = x_half >> 4, x_end = XS * x_step, a0 = tmem_base + 2 * acc;
+            uint32_t xo = 0, n = 0, sa = 0, ph = 0;
+            for (int tile = blockIdx.x, it = 0; tile < a.tiles; tile += gridDim.x, ++it) {
+                const uint32_t d = it & 1, d_tmem = tmem_base + d * acc;
+                decode_wait(bar_dempty + 8 * d, ((uint32_t)(it >> 1) & 1u) ^ 1u, flag);
+                uint32_t accumulate = 0;
+                for (int t = G; t > 0; --t, ++n) {
+                    decode_wait(bar_afull + 8 * sa, ph, flag);
+                    tc_fence_after_sync();
+                    if (n == 0) GPTQ_TRACE_MIN(a.trace_slot, first_data);
+                    const uint32_t a_tmem = a0 + sa * 64;
+                    const uint32_t b0 = desc_lo + xo, b1 = b0 + half_step;
+#pragma unroll
+                    for (int kk = 0; kk < 8; ++kk) {     // 16 k per MMA: 8 columns of A, 32 bytes of each x row
+                        umma_f16_ts(d_tmem, a_tmem + kk * 8, (uint64_t)desc_hi << 32 | ((kk < 4 ? b0 : b1) + (kk & 3) * 2), idesc, accumulate);
+                        accumulate = 1;
+                    }
+                    umma_commit(bar_done + 8 * (n & (kUmmaDoneRing - 1)));
+                    xo += x_step;
+                    if (xo == x_end) xo = 0;
+                    if (++sa == (uint32_t)PS) {
+                        sa = 0;
+                        ph ^= 1u;
+                    }
+                }
+                umma_commit(bar_dfull + 8 * d);
+            }
+        }
+        __syncwarp();
+    } else if (is_dq) {
+        // ---------------------------------------------------------------- dequant warps: a set's pass takes an item
+        const int q = warp & 3, set = (warp - kPrefillFirstDq) >> 2;
+        const int n_col = 32 * q + lane, u = n_col >> 4, g = n_col & 7, h = (n_col >> 3) & 1;
+        uint32_t w_rd[4];               // the column's 8 bytes (rows +0..7, +32..39) in the four chunks of a K64 block
+#pragma unroll
+        for (int t4 = 0; t4 < 4; ++t4) w_rd[t4] = w_ring + (u * 8 + g) * 64 + ((uint32_t)(t4 ^ (g >> 1)) << 4) + 8 * h;
+        const uint32_t z_add = flags & kFormatZerosMinusOne;
+        const uint32_t a_base = tmem_base + ((uint32_t)(32 * q) << 16) + 2 * acc;
+        constexpr uint32_t MAGIC_LO = 0x64006400u;
+        // Scales and zero points of the column (SUB of each per item) straight from global memory, one pass ahead.
+        const uint8_t *const s_col = a.scales + (16 * u + 2 * g + h) * 2, *const z_col = a.qzeros + 8 * u + g;
+        const size_t s_plane = (size_t)G * SUB * kItemSBytes, z_plane = (size_t)G * SUB * kItemZBytes;
+        const uint8_t *s_at = s_col, *z_at = z_col;
+        auto sz_seek = [&](int p, int t) {           // to item t of panel p
+            const size_t sub = ((size_t)(p * PL) * G + t) * SUB;
+            s_at = s_col + sub * kItemSBytes + (PL - 1) * s_plane;
+            z_at = z_col + sub * kItemZBytes;
+        };
+        uint32_t sc_next[SUB] = {}, zb_next[SUB] = {}, zl_next[SUB] = {};
+        auto load_sz = [&]() {
+#pragma unroll
+            for (int e = 0; e < SUB; ++e) {
+                sc_next[e] = __ldcg(reinterpret_cast<const unsigned short *>(s_at + e * kItemSBytes));
+                zb_next[e] = __ldcg(z_at + e * kItemZBytes);
+                if (W8) zl_next[e] = __ldcg(z_at + z_plane + e * kItemZBytes);
+            }
+        };
+        // the set's items: every fourth of the CTA's, across its tiles
+        int tile = blockIdx.x, t = set, n = set, s = set, sa = set < PS ? set : set - PS;
+        uint32_t ph = 0;
+        while (t >= G && tile < a.tiles) { t -= G; tile += gridDim.x; }
+        if (tile < a.tiles) {
+            sz_seek(tile % panels, t);
+            load_sz();
+        }
+        while (tile < a.tiles) {
+            uint32_t s2[SUB], zlo[SUB], zhi[SUB];
+#pragma unroll
+            for (int e = 0; e < SUB; ++e) {
+                s2[e] = sc_next[e] * 0x00010001u;
+                zhi[e] = 0;
+                const int sh = h ? 4 : 0;
+                if constexpr (W8) zlo[e] = ((zb_next[e] >> sh & 15u) << 4 | (zl_next[e] >> sh & 15u)) * 0x00010001u | MAGIC_LO;   // 1024 + z, z < 256
+                else zero_constants<BF>((zb_next[e] >> sh & 15u) + z_add, zlo[e], zhi[e]);
+            }
+            // the next item of this set
+            t += kPrefillSets;
+            if (t >= G) {
+                do {
+                    t -= G;
+                    tile += gridDim.x;
+                } while (t >= G);
+                sz_seek(tile % panels, t);
+            } else {
+                s_at += kPrefillSets * SUB * kItemSBytes;
+                z_at += kPrefillSets * SUB * kItemZBytes;
+            }
+            if (tile < a.tiles) load_sz();
+            if (W8 && n >= WS) wait_done(n - WS);
+            decode_wait(bar_wfull + 8 * s, ph, flag);
+#pragma unroll 1        // (unrolled, the code of the dequant warps evicts that of the MMA warp from the instruction cache)
+            for (int half = 0; half < 2; ++half) {
+                const uint32_t wofs = s * kWSlot + half * kUmmaWBlockBytes;
+                uint2 wv[4], wl[4];
+#pragma unroll
+                for (int t4 = 0; t4 < 4; ++t4) wv[t4] = lds64(wofs + w_rd[t4]);
+                if constexpr (W8) {
+#pragma unroll
+                    for (int t4 = 0; t4 < 4; ++t4) wl[t4] = lds64(wofs + kItemWBytes + w_rd[t4]);
+                }
+                uint32_t r[32];
+#pragma unroll
+                for (int jj = 0; jj < 2; ++jj)
+#pragma unroll
+                    for (int t4 = 0; t4 < 4; ++t4) {
+                        const int e0 = SUB == 4 ? jj : 0;
+                        const uint32_t w = jj ? wv[t4].y : wv[t4].x;       // rows 32 jj + 8 t4 + (0..7), TMEM columns 16 jj + 4 t4 + (0..3)
+                        uint32_t o[4];
+                        if constexpr (W8) {
+                            // bytes 16 hi + lo: nibbles 0, 2, 4, 6 and 1, 3, 5, 7 of both planes; 1024 + byte is an exact
+                            // fp16 number, so is q - z; one rounding with the scale
+                            const uint32_t l = jj ? wl[t4].y : wl[t4].x;
+                            const uint32_t even = (l & 0x0f0f0f0fu) | ((w << 4) & 0xf0f0f0f0u), odd = ((l >> 4) & 0x0f0f0f0fu) | (w & 0xf0f0f0f0u);
+                            o[0] = hsub2_u32(prmt(even, MAGIC_LO, 0x7270), zlo[e0]);
+                            o[1] = hsub2_u32(prmt(odd, MAGIC_LO, 0x7270), zlo[e0]);
+                            o[2] = hsub2_u32(prmt(even, MAGIC_LO, 0x7371), zlo[e0]);
+                            o[3] = hsub2_u32(prmt(odd, MAGIC_LO, 0x7371), zlo[e0]);
+                        } else {
+                            nibble_pairs_minus_zero<BF>(w, zlo[e0], zhi[e0], o);
+                        }
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) r[16 * jj + 4 * t4 + e] = BF ? bmul2_u32(o[e], s2[e0]) : hmul2_u32(o[e], s2[e0]);
+                    }
+                if (half == 0 && n >= PS) {
+                    wait_done(n - PS);
+                    tc_fence_after_sync();
+                }
+                __syncwarp();
+                tmem_st_32x32(a_base + sa * 64 + half * 32, r);
+                if constexpr (SUB > 1) {             // the second half's groups
+#pragma unroll
+                    for (int e = 0; e < SUB / 2; ++e) {
+                        s2[e] = s2[SUB / 2 + e];
+                        zlo[e] = zlo[SUB / 2 + e];
+                        zhi[e] = zhi[SUB / 2 + e];
+                    }
+                }
+            }
+            tmem_wait_st();
+            tc_fence_before_sync();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar_afull + 8 * sa);
+            n += kPrefillSets;
+            sa += kPrefillSets;
+            while (sa >= PS) sa -= PS;
+            s += kPrefillSets;
+            if (s >= WS) {
+                s -= WS;
+                ph ^= 1u;
+            }
+        }
+    }
+    if (is_dq || is_epi) {
+        // ---------------------------------------------------------------- epilogue
+        // A warp reads its 32 lanes (columns of y) x 32 tokens as 8 x 8 fragments, rounds them and transposes them with
+        // stmatrix into rows of 64 bytes in shared memory (16-byte chunks swizzled over pairs of rows), to be stored 16 bytes
+        // per lane.  A residual takes the way back through the same rows (ldmatrix) and joins the fp32 sum.
+        // The CTA's last tile, which nothing runs over any more, is shared out over the epilogue and the dequant warps, 32
+        // tokens at a time.
+        const int group = is_epi ? 0 : 1 + ((warp - kPrefillFirstDq) >> 2), n_groups = 1 + kPrefillSets;
+        const int q = warp & 3;
+        const bool layout_ok = ((flags & kFormatGateUp) != 0) == (a.fuse != 0) && ((flags & kFormatBf16) != 0) == BF;
+        if (!layout_ok && threadIdx.x == 32 * kPrefillFirstEpi) atomicMax(&g_device_status, (int)kStatusLayoutMismatch);
+        const uint32_t stg = (is_epi ? stg0 : w_ring + (group - 1) * kPrefillStage) + q * (32 * 64);      // (the ring is idle by then)
+        const uint32_t mrow = lane & 7, mchunk = lane >> 3;       // row and chunk that this lane addresses in a fragment store
+        const uint32_t frag = stg + mrow * 64 + ((mchunk ^ (mrow >> 1)) << 4);          // token block i: + 512 i
+        const uint32_t prow = lane >> 2, pchunk = lane & 3;       // row (+ 8 t) and chunk of its 16-byte pieces
+        const uint32_t piece = stg + prow * 64 + ((pchunk ^ (prow >> 1)) << 4);
+        const uint32_t up_piece = piece + 2 * 32 * 64;
+        const bool has_bias = a.bias != nullptr, has_res = a.residual != nullptr;
+        pdl_wait();
+        const int my_tiles = (a.tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
+        for (int it = is_epi ? 0 : my_tiles - 1; it < my_tiles; ++it) {
+            const bool last = it == my_tiles - 1;
+            const int tile = blockIdx.x + it * gridDim.x, d = it & 1;
+            const uint32_t ph = (uint32_t)(it >> 1) & 1u;
+            const int mt = tile / panels, p = tile - mt * panels, m0 = mt * tok;
+            const int rows = (a.M - m0) < tok ? (a.M - m0) : tok;
+            float bv[4] = {};                        // columns lane / 4 + 8 j of the warp's 32
+            if (has_bias) {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) bv[j] = __half2float(a.bias[(size_t)p * kPanel + 32 * q + 8 * j + (lane >> 2)]);
+            }
+            decode_wait(bar_dfull + 8 * d, ph, flag);
+            __syncwarp();
+            tc_fence_after_sync();
+            const bool ok = layout_ok && lds32(flag) == 0;
+            const uint32_t src = tmem_base + ((uint32_t)(32 * q) << 16) + d * acc;
+            const size_t y_at = (size_t)(m0 + prow) * a.N + (size_t)p * kPanel + 32 * q + 8 * pchunk;
+#pragma unroll 1
+            for (int c0 = last ? 32 * group : 0; c0 < rows; c0 += last ? 32 * n_groups : 32) {
+                uint32_t r0[16], r1[16];             // lanes 0..15 and 16..31 (columns behind the tile's: read, not looked at)
+                tmem_ld_16x256b_x4(src + c0, r0);
+                tmem_ld_16x256b_x4(src + (16u << 16) + c0, r1);
+                const int nr = rows - c0;
+                if (has_res) {
+#pragma unroll
+                    for (int t = 0; t < 4; ++t)
+                        if (prow + 8 * t < nr) sts128(piece + 512 * t, *reinterpret_cast<const uint4 *>(a.residual + y_at + (size_t)(c0 + 8 * t) * a.N));
+                    __syncwarp();
+                }
+                tmem_wait_ld();
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    float2 v[4];                     // tokens 8 i + 2 (lane % 4) + (0, 1); columns lane / 4 + 8 j
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        v[e] = make_float2(__uint_as_float(r0[4 * i + 2 * e]), __uint_as_float(r0[4 * i + 2 * e + 1]));
+                        v[2 + e] = make_float2(__uint_as_float(r1[4 * i + 2 * e]), __uint_as_float(r1[4 * i + 2 * e + 1]));
+                    }
+                    if (has_bias) {
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) v[j].x += bv[j], v[j].y += bv[j];
+                    }
+                    if (has_res) {
+                        uint32_t rr[4];
+                        ldmatrix_x4_trans(frag + 512 * i, rr);
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&rr[j]));
+                            v[j].x += f.x, v[j].y += f.y;
+                        }
+                        __syncwarp();
+                    }
+                    uint32_t o[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) o[j] = pack_out16<BF>(v[j]);
+                    stmatrix_x4_trans(frag + 512 * i, o);
+                }
+                if (!a.fuse) {
+                    __syncwarp();
+#pragma unroll
+                    for (int t = 0; t < 4; ++t)
+                        if (ok && (int)prow + 8 * t < nr) *reinterpret_cast<uint4 *>(a.y + y_at + (size_t)(c0 + 8 * t) * a.N) = lds128(piece + 512 * t);
+                    __syncwarp();
+                } else {
+                    // gate (warps of lanes 0..63) and up columns are both rounded to fp16 first; the gate warps store
+                    named_bar_sync(1 + group, 128);
+                    if (q < 2 && ok) {
+                        const int oc = p * 64 + 32 * q + 8 * pchunk;
+#pragma unroll 1
+                        for (int t = 0; t < 4; ++t) {
+                            if ((int)prow + 8 * t >= nr) break;
+                            const uint4 gv = lds128(piece + 512 * t), uv = lds128(up_piece + 512 * t);
+                            const uint32_t gw[4] = {gv.x, gv.y, gv.z, gv.w}, uw[4] = {uv.x, uv.y, uv.z, uv.w};
+                            uint32_t ow[4];
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) {
+                                const float2 gf = __half22float2(*reinterpret_cast<const __half2 *>(&gw[e]));
+                                const float2 uf = __half22float2(*reinterpret_cast<const __half2 *>(&uw[e]));
+                                const __half2 o = __floats2half2_rn(silu_mul(gf.x, uf.x), silu_mul(gf.y, uf.y));
+                                ow[e] = *reinterpret_cast<const uint32_t *>(&o);
+                            }
+                            __half *orow = a.y + (size_t)(m0 + c0 + prow + 8 * t) * (a.N / 2);
+                            if (a.out_index == nullptr) {
+                                *reinterpret_cast<uint4 *>(orow + oc) = make_uint4(ow[0], ow[1], ow[2], ow[3]);
+                            } else {
+                                // scattered columns: eight destinations (two 16-byte index loads), eight 2-byte stores
+                                const int4 ia = *reinterpret_cast<const int4 *>(a.out_index + oc);
+                                const int4 ib = *reinterpret_cast<const int4 *>(a.out_index + oc + 4);
+                                const int dst[8] = {ia.x, ia.y, ia.z, ia.w, ib.x, ib.y, ib.z, ib.w};
+#pragma unroll
+                                for (int e = 0; e < 8; ++e)
+                                    orow[dst[e]] = __ushort_as_half((unsigned short)(ow[e >> 1] >> (16 * (e & 1))));
+                            }
+                        }
+                    }
+                    named_bar_sync(1 + group, 128);
+                }
+            }
+            tc_fence_before_sync();
+            __syncwarp();
+            if (!last && lane == 0) mbar_arrive(bar_dempty + 8 * d);
+        }
+        if (threadIdx.x == 32 * kPrefillFirstEpi) GPTQ_TRACE_MAX(a.trace_slot, last_exit);
+    }
+    tc_fence_before_sync();
+    __syncthreads();
+    if (lds32(flag) != 0) {         // a wait gave up: leave time for the copies in flight to land
+        const uint64_t start = global_timer_ns();
+        while (global_timer_ns() - start < 200000ull) { }
+        __syncthreads();
+    }
+    if (warp == 1) {
+        tc_fence_after_sync();
+        tmem_dealloc(tmem_base, 512);
+    }
+}
+
+struct PrefillPlan {
+    bool use;
+    int tok, tiles, ctas, x_slots, smem_bytes;
+};
+
+// Token rows per tile with the smallest number of clocks: waves of tiles x items x the slower of the MMA (4 clocks per token
+// row) and what an item costs at any size (the MMA thread, or dequantising 8-bit weights), plus a part per wave; of equals the
+// larger tile, which dequantises less.
+//
+// The kernel is used unless the cluster split of gptq_umma.cuh is estimated faster: it puts several SMs to a tile, which wins
+// where tiles are few and K long.  Its planner's estimate is scaled to clocks by what was measured per kernel variant (K = 2048
+// to 11008, 8 to 216 panels).  Both sides, us: K = 11008, M = 64: 64 panels 27.2 here, 24.2 there; 80 panels 28.5 / 38.7.
+// K = 4096, M = 64: 32 panels 10.6 / 9.5, 40 panels 10.8 / 11.6.  K = 4096, M = 256: 16 panels 13.6 / 15.6.  M = 16 (the
+// mma.sync kernel's) on 96 panels 11.4 / 11.1, on 32 panels 10.0 / 5.8.
+inline PrefillPlan plan_prefill(int M, int N, int K, int sm_count, bool w8)
+{
+    PrefillPlan pl{};
+    const int panels = N / kPanel, G = K / kGroup;
+    if (G < kPrefillSets) return pl;
+    long long best = -1;
+    for (int most = kPrefillMaxTok; most >= 32; most -= 16) {
+        const int t = (M + most - 1) / most;
+        const int tok = ((M + t - 1) / t + 15) & ~15;
+        const long long tiles = (long long)panels * t, waves = (tiles + sm_count - 1) / sm_count;
+        const int any = w8 ? (tok > 128 ? 800 : 670) : 520, mma = 4 * tok + 60;
+        const long long clocks = waves * ((long long)G * (mma > any ? mma : any) + 1500) + 900;
+        if (tiles < (1 << 30) && (best < 0 || clocks < best)) {
+            best = clocks;
+            pl.tok = tok;
+            pl.tiles = (int)tiles;
+        }
+    }
+    if (best < 0) return pl;
+    const UmmaPlan split = plan_umma(M, N, K, sm_count, w8);
+    const int percent = (split.tok <= 64 ? 100 : split.tok == 128 ? 117 : 150) * (w8 ? (split.tok <= 128 ? 18 : 13) : 10) / 10;
+    if (split.one_wave && 6500 + split.estimate * 243 * percent / 1000 < best) return pl;
+    pl.use = true;
+    pl.ctas = pl.tiles < sm_count ? pl.tiles : sm_count;
+    const int fixed = 2048 + kPrefillStage + prefill_w_slots(pl.tok, w8) * (w8 ? 2 : 1) * kItemWBytes, x_slot = pl.tok * 256;
+    pl.x_slots = (227 * 1024 - fixed) / x_slot;
+    if (pl.x_slots > prefill_a_stages(pl.tok)) pl.x_slots = prefill_a_stages(pl.tok);
+    pl.smem_bytes = fixed + pl.x_slots * x_slot;
+    const int floor_one_per_sm = (227 * 1024) / 2 + 512;                 // the CTA owns all tensor memory
+    if (pl.smem_bytes < floor_one_per_sm) pl.smem_bytes = floor_one_per_sm;
+    return pl;
+}
+
+template <int SUB, bool BF, bool W8>
+static int launch_prefill_sub(const PrefillArgs &args, const CUtensorMap &w_map, const CUtensorMap &x_map, const PrefillPlan &plan,
+                              cudaStream_t s)
+{
+    static int configured_smem[64] = {};
+    const int cfg_st = ensure_dynamic_smem((const void *)prefill_kernel<SUB, BF, W8>, configured_smem, plan.smem_bytes);
+    if (cfg_st) return cfg_st;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)plan.ctas);
+    cfg.blockDim = dim3(kPrefillThreads);
+    cfg.dynamicSmemBytes = (size_t)plan.smem_bytes;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return record_cuda_error(cudaLaunchKernelEx(&cfg, prefill_kernel<SUB, BF, W8>, args, w_map, x_map));
+}
+
+int launch_prefill(const __half *x, const void *qweight, const void *qzeros, const void *scales, __half *y, int M, int N, int K,
+                   int group_size, const PrefillPlan &plan, int fuse, const __half *bias, const __half *residual,
+                   const int32_t *out_index, int bf16, int w8, cudaStream_t s)
+{
+    PrefillArgs args;
+    args.scales = (const uint8_t *)scales;
+    args.qzeros = (const uint8_t *)qzeros;
+    args.y = y;
+    args.M = M;
+    args.N = N;
+    args.G = K / kGroup;
+    args.tok = plan.tok;
+    args.tiles = plan.tiles;
+    args.x_slots = plan.x_slots;
+    args.trailer = reinterpret_cast<const TiledTrailer *>((const uint8_t *)qzeros + tiled_zero_bytes(N, w8 ? 2 * K : K, group_size));
+    args.fuse = fuse;
+    args.bias = bias;
+    args.residual = residual;
+    args.trace_slot = next_trace_slot();
+    args.out_index = out_index;
+    CUtensorMap w_map, x_map;
+    int st = make_tensor_map_2d(&w_map, CU_TENSOR_MAP_DATA_TYPE_UINT32, qweight, 16, (uint64_t)K * N * (w8 ? 2 : 1) / 2 / 64, 64, 16, 128,
+                                CU_TENSOR_MAP_SWIZZLE_64B);
+    if (st) return st;
+    st = make_tensor_map_ktiles(&x_map, x, (uint64_t)K, (uint64_t)M, (uint32_t)plan.tok, 2);
+    if (st) return st;
+    switch (kGroup / group_size + (w8 ? 20 : bf16 ? 10 : 0)) {
+    case 1: return launch_prefill_sub<1, false, false>(args, w_map, x_map, plan, s);
+    case 2: return launch_prefill_sub<2, false, false>(args, w_map, x_map, plan, s);
+    case 4: return launch_prefill_sub<4, false, false>(args, w_map, x_map, plan, s);
+    case 11: return launch_prefill_sub<1, true, false>(args, w_map, x_map, plan, s);
+    case 12: return launch_prefill_sub<2, true, false>(args, w_map, x_map, plan, s);
+    case 14: return launch_prefill_sub<4, true, false>(args, w_map, x_map, plan, s);
+    case 21: return launch_prefill_sub<1, false, true>(args, w_map, x_map, plan, s);
+    case 22: return launch_prefill_sub<2, false, true>(args, w_map, x_map, plan, s);
+    case 24: return launch_prefill_sub<4, false, true>(args, w_map, x_map, plan, s);
+    default: return GPTQ_ERR_UNSUPPORTED;
+    }
+}
+
+}  // namespace gptq

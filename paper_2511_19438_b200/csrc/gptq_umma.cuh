@@ -867,6 +867,8 @@ struct UmmaPlan {
     // When the tiles fill the SMs more than once and the last wave would leave most SMs idle, that wave's tiles
     // go to a second launch that splits K over clusters of tail_S CTAs (0 tiles: no second launch).
     int tail_tiles, tail_S, tail_stages;
+    bool one_wave;          // all CTAs are resident at once
+    long long estimate;     // of the time, in the planner's own unit (about 24 clocks)
 };
 
 // A-ring depth per panel: with two panels the 512 tensor-memory columns hold exactly 2 x (128 + 4 x 32)
@@ -905,6 +907,8 @@ inline UmmaPlan plan_umma(int M, int N, int K, int sm_count, bool w8 = false)
         }
     }
     const int S = best_S;
+    pl.one_wave = tiles <= sm_count * cps_max;
+    pl.estimate = best_t;
     const int groups_per_cta = (G + S - 1) / S;
     int per_sm = (tiles * S + sm_count - 1) / sm_count;
     if (per_sm > cps_max) per_sm = cps_max;

@@ -1482,6 +1482,27 @@ def test_w8_token_tiles(K, N, gs, M, ws):
     assert np.all(err[finite] <= bound[finite]), (err[finite] / bound[finite]).max()
 
 
+# ------------------------------------------------------------------------------- persistent tcgen05 kernel
+@pytest.mark.parametrize("K,N,gs,act,zm1", [
+    (512, 19200, 128, False, False),      # 150 panels: more tiles than SMs from one token tile on; the fewest K groups
+    (640, 256, 64, True, True),           # K groups that the four dequant sets share unevenly
+    (1152, 384, 32, False, False),        # four groups per item, nine items
+])
+@pytest.mark.parametrize("M", [17, 128, 129, 161, 300, 650])      # tiles of 32 to 160 rows, one to six of them, most with a remainder
+def test_prefill_kernel(K, N, gs, act, zm1, M, ws):
+    """Token tiles, waves and group sizes of the persistent kernel, with the plain, bias + residual and gate/up epilogues.
+    The arithmetic is that of the other tcgen05 kernel: weights rounded to 16 bits once, fp32 sums."""
+    assert B.gptq_plan_prefill(M, N, K, gs, int(act), 0, 148)[0] == B.GPTQ_OK, "the planner no longer takes this shape: choose another"
+    L = wl.make_linear(K, N, seed=wl.seed_for("prefill", K, N, gs), group_size=gs, act_order=act, zeros_minus_one=zm1)
+    x_np = wl.make_x(M, K, wl.seed_for("prefill-x", M, K))
+    y, _ = run_gemm(L, x_np, ws)
+    assert_close(y, oracle.gemm_f64(x_np, L.qweight, L.qzeros, L.scales, L.g_idx, gs, zeros_minus_one=zm1), K, M)
+    if not zm1:
+        check_bias_residual(L, M, ws, True, True)
+    check_silu_mul(L, x_np, ws)
+    assert B.gptq_check_status() == B.GPTQ_OK
+
+
 # ------------------------------------------------------------------------------- how a host batch moves its activations
 @pytest.mark.parametrize("M", [1, 3, 40])
 @pytest.mark.parametrize("count", [1, 8, 9, 21])

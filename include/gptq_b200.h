@@ -396,7 +396,7 @@ typedef struct {
     int split_panels; /* panels whose K range is shared by several CTAs */
     int smem_bytes;   /* dynamic shared memory per CTA */
     size_t workspace_bytes;
-    int cluster_size; /* CTAs that share one panel (kernel 1) or one output tile (kernel 2); 1 for kernel 3 */
+    int cluster_size; /* CTAs that share one panel (kernel 1) or one output tile (kernels 2 and 5); 1 for kernel 3 */
     int tail_ctas;    /* kernel 2 only: grid of a second launch that takes the tiles of a partly filled last
                          wave and splits K over clusters (`ctas` is then the first launch alone); 0 = none */
     int tail_cluster_size; /* cluster size of that second launch (1 when there is none) */
@@ -409,9 +409,9 @@ int gptq_plan(int M, int N, int K, int group_size, int act_order, int sm_count, 
  * GPTQ_ERR_UNSUPPORTED for a problem that it leaves to the tile kernels.  `ctas` = clusters x cluster_size, each cluster
  * working through several panels; `stages` = depth of the weight ring in steps. */
 int gptq_plan_decode(int M, int N, int K, int group_size, int act_order, int sm_count, gptq_plan_t *out);
-/* The same for the persistent kernel (kernel 5), which takes problems of 17 and more token rows unless a split of K over
- * clusters (kernel 2) is estimated faster; eight_bit is nonzero for gptq_gemm_w8.  `m_tile` = token rows per tile, `stages` =
- * depth of the x ring in 128-row items. */
+/* The same for the persistent kernel (kernel 5), which takes problems of 17 and more token rows unless kernel 2 is
+ * estimated faster; eight_bit is nonzero for gptq_gemm_w8.  `m_tile` = token rows per tile, `stages` =
+ * depth of the x ring in 128-row items, `cluster_size` = CTAs that share the K range of a tile. */
 int gptq_plan_prefill(int M, int N, int K, int group_size, int act_order, int eight_bit, int sm_count, gptq_plan_t *out);
 /* The same for gptq_gemm_noalloc (stream-K kernel; workspace_bytes is its need of the built-in scratch). */
 int gptq_plan_noalloc(int M, int N, int K, int group_size, int act_order, int sm_count, gptq_plan_t *out);

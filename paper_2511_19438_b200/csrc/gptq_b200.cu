@@ -351,7 +351,7 @@ int gptq_plan_prefill(int M, int N, int K, int group_size, int act_order, int ei
     st = check_fast_path(N, K, group_size);
     if (st) return st;
     if (sm_count < 1) return GPTQ_ERR_SHAPE;
-    const PrefillPlan pl = plan_prefill(M, N, K, sm_count, eight_bit != 0);
+    const PrefillPlan pl = plan_prefill(M, N, K, sm_count, eight_bit != 0, true);
     if (M < kUmmaMinTokens || !pl.use) return GPTQ_ERR_UNSUPPORTED;
     out->kernel = 5;
     out->m_tile = pl.tok;
@@ -359,10 +359,10 @@ int gptq_plan_prefill(int M, int N, int K, int group_size, int act_order, int ei
     out->stages = pl.x_slots;
     out->ctas = pl.ctas;
     out->items = (N / kPanel) * (K / kGroup);
-    out->split_panels = 0;
+    out->split_panels = pl.S > 1 ? N / kPanel : 0;
     out->smem_bytes = pl.smem_bytes;
     out->workspace_bytes = gemm_workspace_need(M, eight_bit ? 2 * K : K, eight_bit ? 1 : act_order);
-    out->cluster_size = 1;
+    out->cluster_size = pl.S;
     out->tail_ctas = 0;
     out->tail_cluster_size = 1;
     set_kernel_name(out, "prefill_kernel<%d>", kGroup / group_size);
@@ -480,10 +480,10 @@ static int gemm_dispatch(const void *x, const void *qweight, const void *qzeros,
             const Umma2Plan p2 = plan_umma2(M, N, K);
             return launch_umma2(xin, qweight, qzeros, scales, (__half *)y, M, N, K, p2, s);
         }
-        if (const PrefillPlan pp = plan_prefill(M, N, K, sms, false); pp.use)      // one CTA per SM, no split of K
+        if (const PrefillPlan pp = plan_prefill(M, N, K, sms, false, !fuse); pp.use)
             return launch_prefill(xin, qweight, qzeros, scales, (__half *)y, M, N, K, group_size, pp, fuse, (const __half *)bias,
                                   (const __half *)residual, out_index, bf16, 0, s);
-        // few tiles and a long K: 32- to 256-token tiles, K split over clusters
+        // few tiles and a long K: 32- to 256-token tiles, K split over clusters of up to eight
         const UmmaPlan pl = plan_umma(M, N, K, sms);
         return launch_umma(xin, qweight, qzeros, scales, (__half *)y, M, N, K, group_size, pl, fuse, (const __half *)bias,
                            (const __half *)residual, out_index, bf16, 0, s);
@@ -624,7 +624,7 @@ int gptq_gemm_w8(const void *x, const void *qweight, const void *qzeros, const v
         // the tcgen05 kernel joins the planes itself: x once, in the row order of either plane
         st = launch_gather_x((const __half *)x, perm, (__half *)ws.ptr, M, K, (cudaStream_t)stream);
         if (st) return st;
-        if (const PrefillPlan pp = plan_prefill(M, N, K, sms, true); pp.use)
+        if (const PrefillPlan pp = plan_prefill(M, N, K, sms, true, true); pp.use)
             return launch_prefill((const __half *)ws.ptr, qweight, qzeros, scales, (__half *)y, M, N, K, tiled, pp, 0, nullptr,
                                   nullptr, nullptr, 0, 1, (cudaStream_t)stream);
         return launch_umma((const __half *)ws.ptr, qweight, qzeros, scales, (__half *)y, M, N, K, tiled,

@@ -1,7 +1,6 @@
-// Persistent tcgen05 GPTQ matmul for 17 token rows and more: what the kernel of gptq_umma.cuh does, for problems whose tiles
-// fill the SMs without a split of K.
+// Persistent tcgen05 GPTQ matmul for 17 token rows and more.
 //
-// As there, the 128 columns of a panel are the MMA's rows, dequantised into a ring of A stages in tensor memory, and a tile of
+// As in gptq_umma.cuh, the 128 columns of a panel are the MMA's rows, dequantised into a ring of A stages in tensor memory, and a tile of
 // token rows is its N.  An item (128 rows of K of a panel, 8 KB of packed weights) is the unit of every hand-over.  What differs:
 //   * One CTA per SM works through its tiles without leaving the kernel.  Tensor memory holds two accumulators of up to 160
 //     token rows beside the A stages, so the epilogue of a tile (four warps of its own) runs under the main loop of the next
@@ -12,14 +11,16 @@
 //   * Four sets of four dequant warps take every fourth item each: a set's pass takes about 1000 clocks, most of it latency.
 //   * x lands on the barrier of its item's A stage, so the MMA thread has one wait per item; weights run ahead in a ring of
 //     their own (and start before the previous kernel has finished).
+//   * Where tiles are few, clusters of two or four CTAs share the K range of a tile (one tile per cluster then).
 // What bounds it.  From 128 token rows per tile the MMA: 572 clocks per item of 512 at full rate (qkv M = 512), and then the
-// power limit (1.45-1.5 GHz in that loop).  With fewer rows the MMA thread: about 520 clocks per item for one wait, eight MMAs
-// and a commit.  Its cost is instruction fetch (a fetch group at a time, with five other warps on its scheduler), hence the
-// short loop in one elected thread (846 -> 589 clocks per item against a warp that elects for every item, o M = 512) and the
-// rolled dequant loop.  Stages of a tile of 176 or 192 rows (only two fit beside the accumulators) made the hand-over the
+// power limit (1.45-1.5 GHz in that loop).  With fewer rows instruction issue: about 520 clocks per item, for four dequant
+// warps on every scheduler and the MMA thread among them (a second MMA thread with an accumulator of its own made it 560).  The
+// MMA thread pays for every instruction it fetches between theirs, hence its short loop (765 -> 589 clocks per item against a
+// warp that elects for every item, o M = 512) and the rolled dequant loop.  Stages of a tile of 176 or 192 rows (only two fit beside the accumulators) made the hand-over the
 // limit: 811 clocks per item of 704.
-// Measured (7B layer of four matmuls in a chain, us, kernel of gptq_umma.cuh -> this): M = 64 71.6 -> 60.2, M = 128 82 -> 71,
-// M = 300 177 -> 120, M = 512 212 -> 172, 8-bit M = 300 232 -> 164.
+// Measured (7B layer of four matmuls in a chain, us, kernel of gptq_umma.cuh alone -> this where it is chosen): M = 17
+// 59.4 -> 51.5, M = 64 71.6 -> 55.7, M = 128 82 -> 68.6, M = 300 177 -> 122, M = 512 212 -> 172; 8-bit M = 128 124 -> 102,
+// M = 300 232 -> 167.
 #pragma once
 #include "gptq_decode.cuh"      // waits with a CTA-wide flag
 
@@ -63,6 +64,13 @@ __device__ __forceinline__ void sts128(uint32_t addr, uint4 v)
 {
     asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
+// bulk copy from this CTA's shared memory to a CTA of the cluster, completion counted in bytes on that CTA's mbarrier
+__device__ __forceinline__ void bulk_s2s_cluster(uint32_t dst, uint32_t src, uint32_t bytes, uint32_t bar)
+{
+    asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "r"(src),
+                 "r"(bytes), "r"(bar)
+                 : "memory");
+}
 template <bool BF>
 __device__ __forceinline__ uint32_t pack_out16(float2 v)
 {
@@ -79,6 +87,7 @@ struct PrefillArgs {
     const uint8_t *scales, *qzeros;   // tiled
     __half *y;
     int M, N, G;                      // G: 128-row items of K (of one plane with 8-bit weights)
+    int S;                            // CTAs (a cluster) that share the K range of a tile; then every cluster has one tile
     int tok, tiles, x_slots;          // token rows per tile; tiles; depth of the x ring in items (at most the A stages)
     const TiledTrailer *trailer;
     int fuse;
@@ -87,7 +96,7 @@ struct PrefillArgs {
     const int32_t *out_index;
 };
 
-template <int SUB, bool BF, bool W8>
+template <int SUB, bool BF, bool W8, bool SPLIT>
 __global__ void __launch_bounds__(kPrefillThreads, 1)
 prefill_kernel(const PrefillArgs a, const __grid_constant__ CUtensorMap w_map, const __grid_constant__ CUtensorMap x_map)
 {
@@ -106,9 +115,12 @@ prefill_kernel(const PrefillArgs a, const __grid_constant__ CUtensorMap w_map, c
     // done[n mod 16]: the MMAs of the CTA's n-th item have completed; dfull / dempty: accumulators
     const uint32_t bar_wfull = base, bar_afull = base + 128, bar_done = base + 192, bar_dfull = base + 320,
                    bar_dempty = base + 336;
-    const uint32_t tmem_slot = base + 352, flag = base + 356;
+    const uint32_t tmem_slot = base + 352, flag = base + 356, bar_recv = base + 360;
     const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
-    const int tok = a.tok, G = a.G, panels = a.N / kPanel, XS = a.x_slots;
+    const int S = SPLIT ? a.S : 1, rank = SPLIT ? (int)blockIdx.x % S : 0, tile0 = SPLIT ? (int)blockIdx.x / S : (int)blockIdx.x;
+    const int tile_step = SPLIT ? (int)gridDim.x / S : (int)gridDim.x;
+    const int g0 = SPLIT ? a.G * rank / S : 0, G = SPLIT ? a.G * (rank + 1) / S - g0 : a.G;           // items of a tile that are this CTA's
+    const int tok = a.tok, panels = a.N / kPanel, XS = a.x_slots;
     const int PS = prefill_a_stages(tok), WS = prefill_w_slots(tok, W8), acc = prefill_acc_columns(tok);
     constexpr uint32_t kWSlot = PL * kItemWBytes;
     const uint32_t x_half = (uint32_t)tok * 128, x_slot = 2 * x_half;       // an item's x: two K64 tiles
@@ -123,7 +135,12 @@ prefill_kernel(const PrefillArgs a, const __grid_constant__ CUtensorMap w_map, c
             mbar_init(bar_dempty + 8 * s, 4);
         }
         asm volatile("st.shared.u32 [%0], %1;" ::"r"(flag), "r"(0u) : "memory");
+        if (SPLIT) mbar_init(bar_recv, 1);
         fence_barrier_init();
+        if (SPLIT) {
+            const int m0 = tile0 / panels * tok, rows = (a.M - m0) < tok ? (a.M - m0) : tok;
+            mbar_arrive_expect_tx(bar_recv, (uint32_t)((S - 1) * rows * (kPanel / S) * 4));
+        }
         fence_proxy_async();
     }
     if (warp == 1) {
@@ -153,7 +170,7 @@ prefill_kernel(const PrefillArgs a, const __grid_constant__ CUtensorMap w_map, c
         }
         const int NS = xw ? XS : WS;
         int s = 0, n = 0, sa = 0;
-        for (int tile = blockIdx.x; tile < a.tiles; tile += gridDim.x) {
+        for (int tile = tile0; tile < a.tiles; tile += tile_step) {
             const int mt = tile / panels, p = tile - mt * panels;       // neighbouring CTAs share the x tile
             for (int t = 0; t < G; ++t, ++n) {
                 if (n >= NS) wait_done(n - NS);
@@ -161,13 +178,13 @@ prefill_kernel(const PrefillArgs a, const __grid_constant__ CUtensorMap w_map, c
                     if (xw) {
                         // (the A stage's last item has been multiplied: there are at least as many stages as x slots)
                         mbar_arrive_expect_tx(bar_afull + 8 * sa, x_slot);
-                        tma_load_3d(x_ring + s * x_slot, &x_map, 0, mt * tok, 2 * t, bar_afull + 8 * sa);     // rows >= M read as zero
+                        tma_load_3d(x_ring + s * x_slot, &x_map, 0, mt * tok, 2 * (g0 + t), bar_afull + 8 * sa);     // rows >= M read as zero
                     } else {
                         // packed weights as rows of 64 bytes, 128 to an item
                         mbar_arrive_expect_tx(bar_wfull + 8 * s, kWSlot);
 #pragma unroll
                         for (int pl = 0; pl < PL; ++pl)
-                            tma_load_2d(w_ring + s * kWSlot + pl * kItemWBytes, &w_map, 0, (G * (PL * p + pl) + t) * 128, bar_wfull + 8 * s);
+                            tma_load_2d(w_ring + s * kWSlot + pl * kItemWBytes, &w_map, 0, (a.G * (PL * p + pl) + g0 + t) * 128, bar_wfull + 8 * s);
                     }
                 }
                 __syncwarp();
@@ -183,7 +200,7 @@ prefill_kernel(const PrefillArgs a, const __grid_constant__ CUtensorMap w_map, c
             const uint32_t desc_lo = (uint32_t)desc0, desc_hi = (uint32_t)(desc0 >> 32);      // (the address field is in the low word)
             const uint32_t x_step = x_slot >> 4, half_step = x_half >> 4, x_end = XS * x_step, a0 = tmem_base + 2 * acc;
             uint32_t xo = 0, n = 0, sa = 0, ph = 0;
-            for (int tile = blockIdx.x, it = 0; tile < a.tiles; tile += gridDim.x, ++it) {
+            for (int tile = tile0, it = 0; tile < a.tiles; tile += tile_step, ++it) {
                 const uint32_t d = it & 1, d_tmem = tmem_base + d * acc;
                 decode_wait(bar_dempty + 8 * d, ((uint32_t)(it >> 1) & 1u) ^ 1u, flag);
                 uint32_t accumulate = 0;
@@ -222,10 +239,10 @@ prefill_kernel(const PrefillArgs a, const __grid_constant__ CUtensorMap w_map, c
         constexpr uint32_t MAGIC_LO = 0x64006400u;
         // Scales and zero points of the column (SUB of each per item) straight from global memory, one pass ahead.
         const uint8_t *const s_col = a.scales + (16 * u + 2 * g + h) * 2, *const z_col = a.qzeros + 8 * u + g;
-        const size_t s_plane = (size_t)G * SUB * kItemSBytes, z_plane = (size_t)G * SUB * kItemZBytes;
+        const size_t s_plane = (size_t)a.G * SUB * kItemSBytes, z_plane = (size_t)a.G * SUB * kItemZBytes;
         const uint8_t *s_at = s_col, *z_at = z_col;
         auto sz_seek = [&](int p, int t) {           // to item t of panel p
-            const size_t sub = ((size_t)(p * PL) * G + t) * SUB;
+            const size_t sub = ((size_t)(p * PL) * a.G + g0 + t) * SUB;
             s_at = s_col + sub * kItemSBytes + (PL - 1) * s_plane;
             z_at = z_col + sub * kItemZBytes;
         };
@@ -239,9 +256,9 @@ prefill_kernel(const PrefillArgs a, const __grid_constant__ CUtensorMap w_map, c
             }
         };
         // the set's items: every fourth of the CTA's, across its tiles
-        int tile = blockIdx.x, t = set, n = set, s = set, sa = set < PS ? set : set - PS;
+        int tile = tile0, t = set, n = set, s = set, sa = set < PS ? set : set - PS;
         uint32_t ph = 0;
-        while (t >= G && tile < a.tiles) { t -= G; tile += gridDim.x; }
+        while (t >= G && tile < a.tiles) { t -= G; tile += tile_step; }
         if (tile < a.tiles) {
             sz_seek(tile % panels, t);
             load_sz();
@@ -261,7 +278,7 @@ prefill_kernel(const PrefillArgs a, const __grid_constant__ CUtensorMap w_map, c
             if (t >= G) {
                 do {
                     t -= G;
-                    tile += gridDim.x;
+                    tile += tile_step;
                 } while (t >= G);
                 sz_seek(tile % panels, t);
             } else {
@@ -333,17 +350,92 @@ prefill_kernel(const PrefillArgs a, const __grid_constant__ CUtensorMap w_map, c
             }
         }
     }
-    if (is_dq || is_epi) {
+    if constexpr (SPLIT) {
+        // ---------------------------------------------------------------- the cluster's partial tiles
+        // After its main loop a CTA's rings are idle: it parks its partial sums there as [owner][token][own column] floats (a
+        // CTA owns 128 / S neighbouring columns).  Once every CTA has, bulk copies through distributed shared memory bring
+        // each owner its part, [sender][token][own column] behind the parked tile, and the owner adds in rank order.
+        // (st.async of single floats took about 55 clocks per token row: o M = 128 11.6 us.)
+        const bool layout_ok = ((flags & kFormatGateUp) != 0) == (a.fuse != 0) && ((flags & kFormatBf16) != 0) == BF;
+        if (!layout_ok && threadIdx.x == 32 * kPrefillFirstEpi) atomicMax(&g_device_status, (int)kStatusLayoutMismatch);
+        const int group = is_epi ? 0 : 1 + ((warp - kPrefillFirstDq) >> 2), n_groups = 1 + kPrefillSets;
+        const int mt = tile0 / panels, p = tile0 - mt * panels, m0 = mt * tok, W = kPanel / S;
+        const int rows = (a.M - m0) < tok ? (a.M - m0) : tok;
+        const uint32_t part = (uint32_t)(rows * W * 4), park = w_ring, recv = park + (uint32_t)((rows + 31) & ~31) * (kPanel * 4);
+        if (is_dq || is_epi) {
+            const int q = warp & 3, n = 32 * q + lane, owner = n / W, lc = n - owner * W;
+            pdl_wait();
+            decode_wait(bar_dfull, 0, flag);
+            __syncwarp();
+            tc_fence_after_sync();
+            const uint32_t at = park + owner * part + (uint32_t)lc * 4u;
+#pragma unroll 1
+            for (int c0 = 32 * group; c0 < rows; c0 += 32 * n_groups) {
+                uint32_t r[32];
+                tmem_ld_32x32(tmem_base + ((uint32_t)(32 * q) << 16) + c0, r);
+                tmem_wait_ld();
+#pragma unroll
+                for (int i = 0; i < 32; ++i)
+                    if (c0 + i < rows) sts_f32(at + (uint32_t)((c0 + i) * W) * 4u, __uint_as_float(r[i]));
+            }
+            fence_proxy_async();
+        }
+        __syncwarp();
+        cluster_arrive_release();
+        cluster_wait_acquire();
+        const bool ok = layout_ok && lds32(flag) == 0;
+        if (warp == kPrefillXWarp && ok && elect_one()) {
+            for (int k = 1; k < S; ++k) {
+                const int to = rank + k < S ? rank + k : rank + k - S;
+                const int slot = rank < to ? rank : rank - 1;              // (nobody sends to itself)
+                bulk_s2s_cluster(map_to_cluster_rank(recv + slot * part, (uint32_t)to), park + to * part, part,
+                                 map_to_cluster_rank(bar_recv, (uint32_t)to));
+            }
+        }
+        __syncwarp();
+        if ((is_dq || is_epi) && ok) {
+            decode_wait_cluster(bar_recv, 0, flag);
+            if (lds32(flag) == 0) {
+                const int w4 = W >> 2;
+                for (int idx = threadIdx.x - 32 * kPrefillFirstEpi; idx < rows * w4; idx += 128 * n_groups) {
+                    const int m = idx / w4, c = 4 * (idx - m * w4);
+                    const size_t col = (size_t)p * kPanel + rank * W + c, at = (size_t)(m0 + m) * a.N + col;
+                    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+                    for (int k = 0; k < S; ++k) {
+                        const uint32_t from = k == rank ? park + rank * part : recv + (k < rank ? k : k - 1) * part;
+                        const uint4 u = lds128(from + (uint32_t)(m * W + c) * 4u);
+                        v.x += __uint_as_float(u.x);
+                        v.y += __uint_as_float(u.y);
+                        v.z += __uint_as_float(u.z);
+                        v.w += __uint_as_float(u.w);
+                    }
+                    auto add4 = [&](const __half *from) {
+                        const uint2 b = *reinterpret_cast<const uint2 *>(from);
+                        const float2 b0 = __half22float2(*reinterpret_cast<const __half2 *>(&b.x));
+                        const float2 b1 = __half22float2(*reinterpret_cast<const __half2 *>(&b.y));
+                        v.x += b0.x, v.y += b0.y, v.z += b1.x, v.w += b1.y;
+                    };
+                    if (a.bias) add4(a.bias + col);
+                    if (a.residual) add4(a.residual + at);
+                    *reinterpret_cast<uint2 *>(a.y + at) = make_uint2(pack_out16<BF>(make_float2(v.x, v.y)), pack_out16<BF>(make_float2(v.z, v.w)));
+                }
+            }
+        }
+        // no CTA may leave while its parked sums are being read; what it sent has landed once all have received
+        __syncwarp();
+        cluster_arrive_release();
+        cluster_wait_acquire();
+    } else if (is_dq || is_epi) {
         // ---------------------------------------------------------------- epilogue
         // A warp reads its 32 lanes (columns of y) x 32 tokens as 8 x 8 fragments, rounds them and transposes them with
         // stmatrix into rows of 64 bytes in shared memory (16-byte chunks swizzled over pairs of rows), to be stored 16 bytes
         // per lane.  A residual takes the way back through the same rows (ldmatrix) and joins the fp32 sum.
         // The CTA's last tile, which nothing runs over any more, is shared out over the epilogue and the dequant warps, 32
         // tokens at a time.
-        const int group = is_epi ? 0 : 1 + ((warp - kPrefillFirstDq) >> 2), n_groups = 1 + kPrefillSets;
-        const int q = warp & 3;
         const bool layout_ok = ((flags & kFormatGateUp) != 0) == (a.fuse != 0) && ((flags & kFormatBf16) != 0) == BF;
         if (!layout_ok && threadIdx.x == 32 * kPrefillFirstEpi) atomicMax(&g_device_status, (int)kStatusLayoutMismatch);
+        const int group = is_epi ? 0 : 1 + ((warp - kPrefillFirstDq) >> 2), n_groups = 1 + kPrefillSets;
+        const int q = warp & 3;
         const uint32_t stg = (is_epi ? stg0 : w_ring + (group - 1) * kPrefillStage) + q * (32 * 64);      // (the ring is idle by then)
         const uint32_t mrow = lane & 7, mchunk = lane >> 3;       // row and chunk that this lane addresses in a fragment store
         const uint32_t frag = stg + mrow * 64 + ((mchunk ^ (mrow >> 1)) << 4);          // token block i: + 512 i
@@ -352,10 +444,10 @@ prefill_kernel(const PrefillArgs a, const __grid_constant__ CUtensorMap w_map, c
         const uint32_t up_piece = piece + 2 * 32 * 64;
         const bool has_bias = a.bias != nullptr, has_res = a.residual != nullptr;
         pdl_wait();
-        const int my_tiles = (a.tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
+        const int my_tiles = (a.tiles - tile0 + tile_step - 1) / tile_step;
         for (int it = is_epi ? 0 : my_tiles - 1; it < my_tiles; ++it) {
             const bool last = it == my_tiles - 1;
-            const int tile = blockIdx.x + it * gridDim.x, d = it & 1;
+            const int tile = tile0 + it * tile_step, d = it & 1;
             const uint32_t ph = (uint32_t)(it >> 1) & 1u;
             const int mt = tile / panels, p = tile - mt * panels, m0 = mt * tok;
             const int rows = (a.M - m0) < tok ? (a.M - m0) : tok;
@@ -459,7 +551,8 @@ prefill_kernel(const PrefillArgs a, const __grid_constant__ CUtensorMap w_map, c
     }
     tc_fence_before_sync();
     __syncthreads();
-    if (lds32(flag) != 0) {         // a wait gave up: leave time for the copies in flight to land
+    if (lds32(flag) != 0) {
+        // A wait gave up: leave time for the copies in flight to land.
         const uint64_t start = global_timer_ns();
         while (global_timer_ns() - start < 200000ull) { }
         __syncthreads();
@@ -472,34 +565,40 @@ prefill_kernel(const PrefillArgs a, const __grid_constant__ CUtensorMap w_map, c
 
 struct PrefillPlan {
     bool use;
-    int tok, tiles, ctas, x_slots, smem_bytes;
+    int S, tok, tiles, ctas, x_slots, smem_bytes;
 };
 
-// Token rows per tile with the smallest number of clocks: waves of tiles x items x the slower of the MMA (4 clocks per token
-// row) and what an item costs at any size (the MMA thread, or dequantising 8-bit weights), plus a part per wave; of equals the
-// larger tile, which dequantises less.
+// Token rows per tile and CTAs per tile with the smallest number of clocks: waves of tiles x items x the slower of the MMA
+// (4 clocks per token row) and what an item costs at any size (dequantisation and the MMA thread), plus a part per wave; of
+// equals the larger tile, which dequantises less.  A split of K over clusters of two or four CTAs (one tile per cluster) costs
+// about 6000 clocks for the exchange; it wins where tiles are few: K = 11008, 32 panels, M = 100 15.6 us against 19.7 on the
+// kernel of gptq_umma.cuh and 27 without a split.
 //
-// The kernel is used unless the cluster split of gptq_umma.cuh is estimated faster: it puts several SMs to a tile, which wins
-// where tiles are few and K long.  Its planner's estimate is scaled to clocks by what was measured per kernel variant (K = 2048
-// to 11008, 8 to 216 panels).  Both sides, us: K = 11008, M = 64: 64 panels 27.2 here, 24.2 there; 80 panels 28.5 / 38.7.
-// K = 4096, M = 64: 32 panels 10.6 / 9.5, 40 panels 10.8 / 11.6.  K = 4096, M = 256: 16 panels 13.6 / 15.6.  M = 16 (the
-// mma.sync kernel's) on 96 panels 11.4 / 11.1, on 32 panels 10.0 / 5.8.
-inline PrefillPlan plan_prefill(int M, int N, int K, int sm_count, bool w8)
+// The kernel is used unless that one is estimated faster: it splits K finer and puts several CTAs on an SM.  Its planner's
+// estimate is scaled to clocks by what was measured per kernel variant (K = 2048 to 11008, 8 to 216 panels).  Both sides, us,
+// this kernel without a split: K = 11008, M = 64: 64 panels 27.2 here, 24.2 there; 80 panels 28.5 / 38.7.  K = 4096, M = 64:
+// 32 panels 10.6 / 9.5, 40 panels 10.8 / 11.6.  K = 4096, M = 256: 16 panels 13.6 / 15.6.  M = 16 (the mma.sync kernel's) on
+// 96 panels 11.4 / 11.1, on 32 panels 10.0 / 5.8.
+inline PrefillPlan plan_prefill(int M, int N, int K, int sm_count, bool w8, bool may_split)
 {
     PrefillPlan pl{};
     const int panels = N / kPanel, G = K / kGroup;
     if (G < kPrefillSets) return pl;
     long long best = -1;
-    for (int most = kPrefillMaxTok; most >= 32; most -= 16) {
-        const int t = (M + most - 1) / most;
-        const int tok = ((M + t - 1) / t + 15) & ~15;
-        const long long tiles = (long long)panels * t, waves = (tiles + sm_count - 1) / sm_count;
-        const int any = w8 ? (tok > 128 ? 800 : 670) : 520, mma = 4 * tok + 60;
-        const long long clocks = waves * ((long long)G * (mma > any ? mma : any) + 1500) + 900;
-        if (tiles < (1 << 30) && (best < 0 || clocks < best)) {
-            best = clocks;
-            pl.tok = tok;
-            pl.tiles = (int)tiles;
+    for (int S = 1; S <= (may_split ? 4 : 1); S *= 2) {
+        for (int most = kPrefillMaxTok; most >= 32; most -= 16) {
+            const int t = (M + most - 1) / most;
+            const int tok = ((M + t - 1) / t + 15) & ~15;
+            const long long tiles = (long long)panels * t, waves = S > 1 ? 1 : (tiles + sm_count - 1) / sm_count;
+            if (tiles >= (1 << 30) || (S > 1 && tiles > decode_max_clusters(S, sm_count))) continue;
+            const int any = w8 ? (tok > 128 ? 800 : 670) : 520, mma = 4 * tok + 60;
+            const long long clocks = waves * ((long long)((G + S - 1) / S) * (mma > any ? mma : any) + 1500) + 900 + (S > 1 ? 6000 : 0);
+            if (best < 0 || clocks < best) {
+                best = clocks;
+                pl.S = S;
+                pl.tok = tok;
+                pl.tiles = (int)tiles;
+            }
         }
     }
     if (best < 0) return pl;
@@ -507,7 +606,7 @@ inline PrefillPlan plan_prefill(int M, int N, int K, int sm_count, bool w8)
     const int percent = (split.tok <= 64 ? 100 : split.tok == 128 ? 117 : 150) * (w8 ? (split.tok <= 128 ? 18 : 13) : 10) / 10;
     if (split.one_wave && 6500 + split.estimate * 243 * percent / 1000 < best) return pl;
     pl.use = true;
-    pl.ctas = pl.tiles < sm_count ? pl.tiles : sm_count;
+    pl.ctas = pl.S > 1 ? pl.tiles * pl.S : pl.tiles < sm_count ? pl.tiles : sm_count;
     const int fixed = 2048 + kPrefillStage + prefill_w_slots(pl.tok, w8) * (w8 ? 2 : 1) * kItemWBytes, x_slot = pl.tok * 256;
     pl.x_slots = (227 * 1024 - fixed) / x_slot;
     if (pl.x_slots > prefill_a_stages(pl.tok)) pl.x_slots = prefill_a_stages(pl.tok);
@@ -517,24 +616,37 @@ inline PrefillPlan plan_prefill(int M, int N, int K, int sm_count, bool w8)
     return pl;
 }
 
-template <int SUB, bool BF, bool W8>
-static int launch_prefill_sub(const PrefillArgs &args, const CUtensorMap &w_map, const CUtensorMap &x_map, const PrefillPlan &plan,
+template <int SUB, bool BF, bool W8, bool SPLIT>
+static int launch_prefill_split(const PrefillArgs &args, const CUtensorMap &w_map, const CUtensorMap &x_map, const PrefillPlan &plan,
                               cudaStream_t s)
 {
     static int configured_smem[64] = {};
-    const int cfg_st = ensure_dynamic_smem((const void *)prefill_kernel<SUB, BF, W8>, configured_smem, plan.smem_bytes);
+    const int cfg_st = ensure_dynamic_smem((const void *)prefill_kernel<SUB, BF, W8, SPLIT>, configured_smem, plan.smem_bytes);
     if (cfg_st) return cfg_st;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)plan.ctas);
     cfg.blockDim = dim3(kPrefillThreads);
     cfg.dynamicSmemBytes = (size_t)plan.smem_bytes;
     cfg.stream = s;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)args.S;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return record_cuda_error(cudaLaunchKernelEx(&cfg, prefill_kernel<SUB, BF, W8>, args, w_map, x_map));
+    cfg.numAttrs = SPLIT ? 2 : 1;        // (a launch with clusters of one took 0.4 us longer)
+    return record_cuda_error(cudaLaunchKernelEx(&cfg, prefill_kernel<SUB, BF, W8, SPLIT>, args, w_map, x_map));
+}
+
+template <int SUB, bool BF, bool W8>
+static int launch_prefill_sub(const PrefillArgs &args, const CUtensorMap &w_map, const CUtensorMap &x_map, const PrefillPlan &plan,
+                              cudaStream_t s)
+{
+    // (a template: with the number of CTAs per tile known only at run time, launches without a split were 7 % slower)
+    return plan.S > 1 ? launch_prefill_split<SUB, BF, W8, true>(args, w_map, x_map, plan, s)
+                      : launch_prefill_split<SUB, BF, W8, false>(args, w_map, x_map, plan, s);
 }
 
 int launch_prefill(const __half *x, const void *qweight, const void *qzeros, const void *scales, __half *y, int M, int N, int K,
@@ -548,6 +660,7 @@ int launch_prefill(const __half *x, const void *qweight, const void *qzeros, con
     args.M = M;
     args.N = N;
     args.G = K / kGroup;
+    args.S = plan.S;
     args.tok = plan.tok;
     args.tiles = plan.tiles;
     args.x_slots = plan.x_slots;

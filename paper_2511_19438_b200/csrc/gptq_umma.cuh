@@ -17,8 +17,8 @@
 // accumulator with tcgen05.ld, round once to fp16, turn each 32-token chunk around through the
 // idle ring and store whole lines of y.
 //
-// The two single threads (TMA producer, MMA issue) pay 60-110 cycles for every instruction, so
-// both loops are kept short: a ring refill is one wait, one arrive-and-expect, one weight copy and
+// The two single threads (TMA producer, MMA issue) share their schedulers with the dequant warps
+// and pay for every instruction they fetch, so both loops are kept short: a ring refill is one wait, one arrive-and-expect, one weight copy and
 // one 3-D x copy per K group; an MMA step is one wait, four MMAs and one commit per K64 block.
 //
 // Small problems split K over a thread-block cluster (partial tiles meet through distributed
@@ -33,8 +33,7 @@ namespace gptq {
 
 // warp 0: TMA producer, warp 1: MMA issue + TMEM, then four dequant/epilogue warps per panel of the CTA
 // (two sets of them, taking alternate K groups, when one warp per scheduler cannot keep up with the MMA)
-// MMA-issuing warps: one thread pays 60-110 cycles for every instruction it issues (and more when its scheduler is
-// shared with busy dequant warps).  With 64-token tiles each dequant warp set gets an issuing warp and an accumulator
+// MMA-issuing warps: one thread's loop is slow where its scheduler is shared with busy dequant warps.  With 64-token tiles each dequant warp set gets an issuing warp and an accumulator
 // of its own, and the epilogue adds the accumulators (measured 0-6 % faster there; with 32-token tiles the third
 // resident CTA that a single accumulator leaves room for is worth more).
 __host__ __device__ constexpr int umma_issuers(int TOK, int SETS) { return (TOK == 64 && SETS == 2) ? 2 : 1; }
@@ -328,9 +327,8 @@ umma_kernel(const UmmaArgs a, const __grid_constant__ CUtensorMap w_map, const _
         // ---------------------------------------------------------------- MMA issue (one thread per issuing warp)
         if (elect_one()) {
             constexpr uint32_t idesc = umma_idesc_f16(128, TOK) | (BF ? kUmmaIdescBf16 : 0u);
-            // Every instruction this thread issues costs it 60-110 cycles (a tcgen05.mma about 60, a commit
-            // about 80, a barrier wait about 100 even when the barrier is ready), so the loop is kept to one wait
-            // per panel, the four MMAs and one commit per K64 block.  It does not wait for the slot's TMA data
+            // Every instruction counts here (a barrier wait takes 53 clocks even when the barrier is ready, an MMA 9
+            // at N = 16 and the pipe's time from N = 64 on), so the loop is kept to one wait per panel, the four MMAs and one commit per K64 block.  It does not wait for the slot's TMA data
             // itself: the dequant warps did before they wrote the A stage, and their a_full arrival orders it.
             // With one issuer it takes the blocks in order; with two, issuer t takes the blocks of dequant set t
             // (K groups t, t + SETS, ...) and accumulates them in its own tensor-memory columns.

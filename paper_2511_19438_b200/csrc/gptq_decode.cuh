@@ -43,6 +43,9 @@ constexpr int kDecodeDequantWarps = 8, kDecodeDrainWarps = 4;
 constexpr int kDecodeFirstDq = 2;                                              // warp 0: weights, warp 1: MMA + TMEM
 constexpr int kDecodeFirstDrain = kDecodeFirstDq + kDecodeDequantWarps;        // 10
 constexpr int kDecodeFinishWarp = kDecodeFirstDrain + kDecodeDrainWarps;       // 14
+// Steps still to be requested when the next launch may start.  7B layer of four matmuls in a chain, M = 1 / 2, us: 1 28.7 / 29.5,
+// 3 27.6 / 28.5, 5 26.4 / 27.7; from the start of the launch on 37.7 (M = 1).
+constexpr int kDecodeLead = 5;
 constexpr int kDecodeThreads = 32 * (kDecodeFinishWarp + 1);
 constexpr int kDecodeMetaBufs = 3;
 constexpr int kDecodeMetaItems = 8;          // items (of SUB = 1) whose scales and zero points travel together
@@ -293,18 +296,27 @@ decode_kernel(const DecodeArgs a, const __grid_constant__ CUtensorMap w_map)
         tmem_alloc(tmem_slot, kDecodeCols);
         tmem_relinquish();
     }
-    tc_fence_before_sync();
-    __syncthreads();
-    tc_fence_after_sync();
+    // The weights warp, which set up the barriers, does not wait for the others: its first copies leave while tensor memory is
+    // still being allocated.
+    if (warp == 0) {
+        __syncwarp();
+        asm volatile("bar.arrive 1, %0;" ::"r"(kDecodeThreads) : "memory");
+    } else {
+        tc_fence_before_sync();
+        asm volatile("bar.sync 1, %0;" ::"r"(kDecodeThreads) : "memory");
+        tc_fence_after_sync();
+    }
     cluster_arrive_release();           // "my receive barriers are armed"; waited for before the first send
-    const uint32_t tmem_base = __shfl_sync(0xffffffffu, lds32(tmem_slot), 0);
+    const uint32_t tmem_base = __shfl_sync(0xffffffffu, lds32(tmem_slot), 0);      // (not read by the weights warp)
     const uint32_t d_base = tmem_base + 2 * P * kDecodeACols;
 
     if (warp == 0) {
         // ---------------------------------------------------------------- weights (one thread issues)
         if (elect_one()) tma_prefetch_descriptor(&w_map);
         GPTQ_TRACE_MIN(a.trace_slot, first_weight_issue);
-        int s = 0, mb = 0;
+        // The next launch may start when the last kDecodeLead steps are about to be requested: earlier its prefetch would queue
+        // in front of this launch's own loads, later it would not be under way before this launch has ended.
+        int s = 0, mb = 0, left = n_panels * spp;
         uint32_t eph = 1, mph = 1;  // parities that pass in the first round
         for (int p = cl; p < panels; p += a.clusters) {
             for (int c0 = 0; c0 < ng; c0 += MC) {
@@ -319,6 +331,7 @@ decode_kernel(const DecodeArgs a, const __grid_constant__ CUtensorMap w_map)
                 }
                 __syncwarp();
                 for (int i = 0; i < nc; i += P) {
+                    if (left-- == kDecodeLead) pdl_launch_dependents();
                     decode_wait(bar_wempty + 8 * s, eph, flag);
                     if (elect_one()) {
                         const bool two = P == 2 && i + 1 < nc;
@@ -333,8 +346,7 @@ decode_kernel(const DecodeArgs a, const __grid_constant__ CUtensorMap w_map)
                 if (++mb == kDecodeMetaBufs) { mb = 0; mph ^= 1u; }
             }
         }
-        // only now may the next launch start: its prefetch would otherwise queue in front of this launch's own loads
-        pdl_launch_dependents();
+        if (n_panels * spp < kDecodeLead) pdl_launch_dependents();
         cluster_wait_acquire();
     } else if (warp == 1) {
         // ---------------------------------------------------------------- MMA (one thread issues)

@@ -148,7 +148,7 @@ int gptq_set_workspace(void *ptr, size_t bytes);
  * y fp16[M,N] = x fp16[M,K] . dequant(W).  qweight/qzeros/scales are the REPACKED buffers from
  * gptq_repack; with act_order != 0, g_idx is gptq_repack's perm_out (16-byte aligned like every other pointer, else
  * GPTQ_ERR_ALIGN; without act-order it may be NULL).
- * fp32 accumulation, one round-to-nearest-even conversion to fp16 (an infinite x may give NaN).  Any M >= 1.  Up to 16 rows the
+ * fp32 accumulation, one round-to-nearest-even conversion to fp16.  Any M >= 1.  Up to 16 rows the
  * weights enter the MMA as exact integers q - z and the scale multiplies fp32 group sums; above
  * that each scaled weight is rounded to fp16 once before the MMA.
  * The kernels begin fetching weights before earlier work on the stream has finished

@@ -8,8 +8,9 @@
 // `(w >> 4) & 0x0f0f0f0f` are A operands of tcgen05.mma kind::f8f6f4 - three instructions per eight weights where q - z as
 // fp16 takes nine (and twice the tensor memory).  The activations are split without error into four e5m2 pieces: the upper
 // byte of an fp16 number is its e5m2 truncation p0, (x - p0) * 8 is again an fp16 number, and after four steps nothing is
-// left: x = p0 + p1 / 8 + p2 / 64 + p3 / 512 (an infinite x gives NaN).  Two tokens are eight rows of the B operand.  Products
-// and sums are exact to fp32 (measured: 8e-8 of the sum of magnitudes).  Every quantisation group has an accumulator of its
+// left: x = p0 + p1 / 8 + p2 / 64 + p3 / 512.  Two tokens are eight rows of the B operand.  Products and sums are exact to fp32
+// (measured: 8e-8 of the sum of magnitudes).  An infinity or NaN in x makes every sum of its row NaN: such outputs are formed at
+// the end, from those activations alone.  Every quantisation group has an accumulator of its
 // own; the drain warps recombine the pieces, subtract z * sum(x) and apply the scale in fp32.
 //
 // Warp roles, each with its own pace:
@@ -158,6 +159,13 @@ __device__ __forceinline__ uint64_t lds_f32x2(uint32_t addr)
     asm volatile("ld.shared.b64 %0, [%1];" : "=l"(v) : "r"(addr) : "memory");
     return v;
 }
+// Bits of the CTA's flag word
+constexpr uint32_t kDecodeGaveUp = 1u;      // a wait gave up
+constexpr uint32_t kDecodeNotFinite = 2u;   // outputs whose sum is NaN have not been stored yet
+__device__ __forceinline__ void raise_flag(uint32_t flag, uint32_t bits)
+{
+    asm volatile("red.shared.or.b32 [%0], %1;" ::"r"(flag), "r"(bits) : "memory");
+}
 // A wait without a result.  One that gives up raises the CTA's flag, and from then on no wait of the CTA waits: everything
 // runs through on whatever data there is, the status word tells the host, and the CTA leaves after a pause that covers
 // its copies in flight.
@@ -166,10 +174,10 @@ __device__ __noinline__ void decode_wait_slow(uint32_t bar, uint32_t parity, uin
     for (int it = 0; it < kWaitTries; ++it)
         if (mbar_try_wait(bar, parity)) return;
     const uint64_t start = global_timer_ns();
-    while (lds32(flag) == 0) {
+    while ((lds32(flag) & kDecodeGaveUp) == 0) {
         if (mbar_try_wait(bar, parity)) return;
         if (global_timer_ns() - start > kWaitLimitNs) {
-            asm volatile("st.shared.u32 [%0], %1;" ::"r"(flag), "r"(1u) : "memory");
+            raise_flag(flag, kDecodeGaveUp);
             atomicMax(&g_device_status, (int)kStatusWaitTimeout);
         }
     }
@@ -184,10 +192,10 @@ __device__ __noinline__ void decode_wait_cluster(uint32_t bar, uint32_t parity, 
     for (int it = 0; it < kWaitTries; ++it)
         if (mbar_try_wait_cluster(bar, parity)) return;
     const uint64_t start = global_timer_ns();
-    while (lds32(flag) == 0) {
+    while ((lds32(flag) & kDecodeGaveUp) == 0) {
         if (mbar_try_wait_cluster(bar, parity)) return;
         if (global_timer_ns() - start > kWaitLimitNs) {
-            asm volatile("st.shared.u32 [%0], %1;" ::"r"(flag), "r"(1u) : "memory");
+            raise_flag(flag, kDecodeGaveUp);
             atomicMax(&g_device_status, (int)kStatusWaitTimeout);
         }
     }
@@ -219,10 +227,89 @@ __device__ __forceinline__ void tmem_ld_8(uint32_t taddr, uint32_t (&r)[8])
                  : "memory");
 }
 
+// nonzero if one of the two fp16 numbers is an infinity or NaN
+__device__ __forceinline__ uint32_t half2_not_finite(uint32_t v) { return ((v & 0x7c007c00u) + 0x04000400u) & 0x80008000u; }
+
+// Sum of token m and tiled column n as the mma.sync kernel forms it, s * sum((q - z) x) per quantisation group, for outputs
+// that come out as NaN.  Unless `all`, only what decides about them is looked at: infinities and NaNs of x, and groups whose
+// scale is one; `met` is set if there are any (what the rest would add is finite).
+template <int SUB>
+__device__ __forceinline__ float decode_sum_not_finite(const DecodeArgs &a, int m, int n, uint32_t z_plus, bool all, bool &met)
+{
+    constexpr int kRows = kGroup / SUB;
+    const __half *const x = a.x + (size_t)m * a.G * kGroup;
+    float run = 0.f;
+#pragma unroll 1
+    for (int group = 0; group < a.G * SUB; ++group) {
+        const float s = __half2float(__ldcg(reinterpret_cast<const __half *>(a.scales) + repacked_scale_index(group, n, a.G * SUB)));
+        const bool whole = all || !(fabsf(s) <= 65504.f);
+        uint32_t found = whole;
+#pragma unroll 1
+        for (int j = 0; j < kRows / 8; ++j) {
+            const uint4 v = ldg128_cg(x + group * kRows + 8 * j);
+            found |= half2_not_finite(v.x) | half2_not_finite(v.y) | half2_not_finite(v.z) | half2_not_finite(v.w);
+        }
+        if (!found) continue;
+        met = true;
+        int hi, slot;
+        const uint32_t zb = __ldcg(a.qzeros + repacked_zero_byte(group, n, a.G * SUB, &hi));
+        const float z = (float)((hi ? zb >> 4 : zb & 15u) + z_plus);
+        float v = 0.f;
+#pragma unroll 1
+        for (int i = group * kRows; i < (group + 1) * kRows; ++i) {
+            const float xi = __half2float(__ldcg(x + i));
+            if (!whole && fabsf(xi) <= 65504.f) continue;
+            const size_t at = repacked_word_offset(i, n, a.G, &slot);
+            v += ((float)(__ldcg(reinterpret_cast<const uint32_t *>(a.qweight + at)) >> (4 * slot) & 15u) - z) * xi;
+        }
+        run += s * v;
+    }
+    return run;
+}
+// The outputs of the panels cl, cl + clusters, ... and own columns [lo, lo + hw) of a run whose sum is NaN (the finish warp has
+// not stored them): an infinity or NaN in x, or a scale that is one.  A call that works out everything again: values kept for
+// it in registers, or a branch to it in the finish warp's loop, made every launch slower (M = 1 2 %, M = 2 5 to 20 %).
+template <int SUB>
+__device__ __noinline__ void decode_store_not_finite(const DecodeArgs &a)
+{
+    pdl_wait();                                 // (x is read: long since through)
+    const uint32_t z_plus = a.trailer->flags & kFormatZerosMinusOne;
+    const int S = a.S, cl = blockIdx.x / S, rank = blockIdx.x - cl * S, n_panels = (a.N / kPanel - cl + a.clusters - 1) / a.clusters;
+    const int lo = (int)((a.slice_lo >> (8 * rank)) & 255);
+    const int hw = (rank + 1 < S ? (int)((a.slice_lo >> (8 * (rank + 1))) & 255) : a.fuse ? 64 : kPanel) - lo;
+#pragma unroll 1
+    for (int idx = threadIdx.x; idx < n_panels * a.M * hw; idx += kDecodeThreads) {
+        const int pi = idx / (a.M * hw), rest = idx - pi * a.M * hw, m = rest / hw, c = lo + rest - m * hw;
+        const int p = cl + pi * a.clusters, n = p * kPanel + c;
+        bool met = false, met_up = false, all = false;
+        float v = 0.f, up = 0.f;
+#pragma unroll 1
+        for (int k = 0; k < (a.fuse ? 4 : 1); ++k) {        // sum of the column, of the matching up column; whatever of the two has been left out
+            if (k >= 2 && !all) break;
+            bool &seen = k & 1 ? met_up : met;
+            if (k >= 2 && seen) continue;
+            const float f = decode_sum_not_finite<SUB>(a, m, n + 64 * (k & 1), z_plus, all, seen);
+            if (k & 1) up = f;
+            else v = f;
+            if (k == 1) all = met || met_up;
+        }
+        if (!met && !met_up) continue;
+        if (!a.fuse) {
+            if (a.bias) v += __half2float(a.bias[n]);
+            __half *const y = a.y + (size_t)m * a.N + n;
+            if (a.residual) v += __half2float(a.residual[(size_t)m * a.N + n]);
+            *y = __float2half_rn(v);
+        } else {
+            const int oc = p * 64 + c;
+            a.y[(size_t)m * (a.N / 2) + (a.out_index ? a.out_index[oc] : oc)] = __float2half_rn(silu_mul(v, up));
+        }
+    }
+}
+
 // SUB: quantisation groups per item
 template <int SUB>
 __global__ void __launch_bounds__(kDecodeThreads, 2)
-decode_kernel(const DecodeArgs a, const __grid_constant__ CUtensorMap w_map)
+decode_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ CUtensorMap w_map)
 {
     extern __shared__ uint8_t smem_raw[];
     constexpr int P = decode_step_items(SUB);                 // items per step
@@ -582,11 +669,12 @@ decode_kernel(const DecodeArgs a, const __grid_constant__ CUtensorMap w_map)
         if (!layout_ok && lane == 0) atomicMax(&g_device_status, (int)kStatusLayoutMismatch);
         pdl_wait();
         cluster_wait_acquire();
+        bool any_nan = false;
         for (int pi = 0; pi < n_panels; ++pi) {
             const int p = cl + pi * a.clusters;
             const uint32_t buf = (uint32_t)pi & 1u;
             decode_wait_cluster(bar_recv + 8 * buf, (uint32_t)(pi >> 1) & 1u, flag);
-            if (layout_ok && lds32(flag) == 0) {
+            if (layout_ok && (lds32(flag) & kDecodeGaveUp) == 0) {
                 // a thread takes one column (with fuse: a gate column and its up column) of one token
                 for (int idx = lane; idx < a.M * hw; idx += 32) {
                     const int j = a.M == 2 ? idx >> 1 : idx, m = a.M == 2 ? idx & 1 : 0;
@@ -603,15 +691,19 @@ decode_kernel(const DecodeArgs a, const __grid_constant__ CUtensorMap w_map)
                     if (!a.fuse) {
                         const int n = p * kPanel + lo + j;
                         float v = slice_sum(j);
+                        const bool is_nan = isnan(v);
                         if (a.bias || a.residual) {
                             v += (a.bias ? __half2float(a.bias[n]) : 0.f);
                             if (a.residual) v += __half2float(a.residual[(size_t)m * a.N + n]);
                         }
-                        a.y[(size_t)m * a.N + n] = __float2half_rn(v);
+                        if (!is_nan) a.y[(size_t)m * a.N + n] = __float2half_rn(v);
+                        any_nan |= is_nan;
                     } else {
                         const int oc = p * 64 + lo + j;
-                        a.y[(size_t)m * (a.N / 2) + (a.out_index ? a.out_index[oc] : oc)] =
-                            __float2half_rn(silu_mul(slice_sum(j), slice_sum(a.slice_max + j)));
+                        const float gate = slice_sum(j), up = slice_sum(a.slice_max + j);
+                        const bool is_nan = isnan(gate) || isnan(up);
+                        if (!is_nan) a.y[(size_t)m * (a.N / 2) + (a.out_index ? a.out_index[oc] : oc)] = __float2half_rn(silu_mul(gate, up));
+                        any_nan |= is_nan;
                     }
                 }
             }
@@ -622,11 +714,13 @@ decode_kernel(const DecodeArgs a, const __grid_constant__ CUtensorMap w_map)
                 if (lane < S) mbar_arrive_release_cluster(map_to_cluster_rank(bar_free + 8 * buf, (uint32_t)lane));
             }
         }
+        if (any_nan) raise_flag(flag, kDecodeNotFinite);
         if (lane == 0) GPTQ_TRACE_MAX(a.trace_slot, last_exit);
     }
     tc_fence_before_sync();
     __syncthreads();
-    if (lds32(flag) != 0) {
+    const uint32_t raised = lds32(flag);
+    if (raised & kDecodeGaveUp) {
         // A wait gave up: leave time for the copies in flight to land, and stay until the other CTAs of the cluster have
         // left or come here too (they may still send; one that left in order has nothing more to receive).
         const uint64_t start = global_timer_ns();
@@ -634,6 +728,8 @@ decode_kernel(const DecodeArgs a, const __grid_constant__ CUtensorMap w_map)
         __syncthreads();
         cluster_arrive_release();
         cluster_wait_acquire();
+    } else if (raised) {
+        decode_store_not_finite<SUB>(a);
     }
     if (warp == 1) {
         tc_fence_after_sync();

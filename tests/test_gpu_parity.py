@@ -1460,6 +1460,56 @@ def test_decode_kernel(K, N, gs, act, zm1, M, ws):
     assert B.gptq_check_status() == B.GPTQ_OK
 
 
+@pytest.mark.parametrize("K,N,gs,act,zm1", [(4096, 4096, 128, False, False), (4224, 12288, 64, True, False), (3328, 22016, 32, False, True)])
+def test_decode_kernel_infinite_and_nan_activations(K, N, gs, act, zm1, ws):
+    """An infinite activation gives what the sum in 64 bits gives, with one row as with three (the mma.sync kernel): an infinity of
+    the sign of (q - z) x, NaN where q = z and where infinities of both signs or a NaN meet.  Rows without one are not touched,
+    and a residual that is y itself is read before it is overwritten."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    L = wl.make_linear(K, N, seed=wl.seed_for("decode-inf", K, N, gs), group_size=gs, act_order=act, zeros_minus_one=zm1)
+    D = H.upload_and_repack(L)
+    ws.ensure_for(3, D)
+    x = wl.make_x(8, K, wl.seed_for("decode-inf-x", K))
+    x[0, K // 2 + 5] = np.inf
+    x[2, 0], x[2, 1] = -np.inf, np.inf                # one group
+    x[3, 7], x[3, K - 1] = np.inf, np.inf             # the first group and the last
+    x[4, K - 40] = np.nan
+    x[6, K // 3] = -np.inf
+    x[7] = 65504                                       # the largest finite values: sums stay finite in fp32
+    with np.errstate(invalid="ignore"):
+        want = oracle.gemm_f64(x, L.qweight, L.qzeros, L.scales, L.g_idx, gs, zeros_minus_one=zm1)
+    assert np.isposinf(want[0]).any() and np.isneginf(want[0]).any() and np.isnan(want[0]).any()
+
+    def check(y, w, rows):
+        assert np.array_equal(np.isnan(y), np.isnan(w)), rows
+        assert np.array_equal(np.isposinf(y), np.isposinf(w)) and np.array_equal(np.isneginf(y), np.isneginf(w)), rows
+        fin = np.isfinite(w)
+        assert np.all(np.abs(y[fin] - w[fin]) <= 1e-4 * math.sqrt(K / 4096) + 2.0 ** -11 * np.abs(w[fin])), rows
+
+    for rows in ([0], [1], [4], [6], [0, 1], [1, 2], [3, 4], [5, 6], [0, 1, 2], [3, 4, 5]):
+        if sms == 148 and len(rows) <= 2:
+            assert B.gptq_plan_decode(len(rows), N, K, gs, int(act), sms)[0] == B.GPTQ_OK, "the planner no longer takes this shape: choose another"
+        xr = H.to_device(np.ascontiguousarray(x[rows]))
+        check(H.gemm(xr, D).cpu().numpy().astype(np.float64), want[rows], rows)
+        y = torch.full((len(rows), N), 3.0, dtype=torch.float16, device="cuda")
+        H.gemm_bias_residual(xr, D, None, y, y=y)
+        check(y.cpu().numpy().astype(np.float64), want[rows] + 3.0, rows)
+    y = H.gemm(H.to_device(x[7:8]), D).cpu().numpy()
+    sure = np.abs(want[7]) > 1000                      # (fp32 sums of terms of up to 65504 x 16)
+    assert not np.isnan(y).any() and np.array_equal(np.sign(y[0][sure]), np.sign(want[7][sure]))
+    if N % 256 == 0:                                   # gate and up columns, one of them or both infinite
+        D = H.upload_and_repack(L, gate_up=True)
+        with np.errstate(invalid="ignore", over="ignore"):
+            w = oracle.silu_mul_f64(want[:3])
+        for rows in ([0], [0, 1], [1, 2]):
+            y = H.gemm_silu_mul(H.to_device(np.ascontiguousarray(x[rows])), D).cpu().numpy().astype(np.float64)
+            bad = ~np.isfinite(want[rows].reshape(len(rows), 2, N // 2)).all(axis=1)
+            for a, b in ((np.isnan(y), np.isnan(w[rows])), (np.isposinf(y), np.isposinf(w[rows])), (np.isneginf(y), np.isneginf(w[rows]))):
+                assert np.array_equal(a & bad, b & bad), rows
+            assert np.isfinite(y[~bad]).all()
+    assert B.gptq_check_status() == B.GPTQ_OK
+
+
 # ------------------------------------------------------------------------------- 8-bit weights joined in the tcgen05 kernel
 @pytest.mark.parametrize("K,N,gs", [(384, 256, 128), (384, 256, 64), (256, 128, 32), (2048, 4864, 128)])
 @pytest.mark.parametrize("M", [17, 33, 64, 65, 129, 257])

@@ -200,9 +200,10 @@ int gptq_gemm_bias_residual(const void *x, const void *qweight, const void *qzer
 /* (No counterpart in the paper: an epilogue fused into the product of Sections 1 and 3.)
  * out fp16[M, N / 2] = silu(y[:, :N/2]) * y[:, N/2:], silu(g) = g / (1 + exp(-g)), for y = x . dequant(W) of a layer
  * repacked with GPTQ_FORMAT_GATE_UP: the activation of a Llama MLP block applied before the product leaves the chip,
- * so y itself is never written.  Other arguments as for gptq_gemm; N counts both halves.  Up to 16 token rows the
- * two factors are the fp32 sums; above that each is rounded to fp16 first unless the K range was split across CTAs;
- * silu and the product are evaluated in fp32 (fast exponential, relative error ~1e-6), then rounded to fp16 once.
+ * so y itself is never written.  Other arguments as for gptq_gemm; N counts both halves.  The two factors are the fp32
+ * sums (above 16 token rows, where the one-tile-per-CTA tcgen05 kernel takes the call without splitting K, each is rounded to
+ * fp16 first; see gptq_plan_prefill); silu and the product are evaluated in fp32 (fast exponential, relative error ~1e-6),
+ * then rounded to fp16 once.
  * A layer repacked without the flag (or a flagged layer given to gptq_gemm / gptq_gemm_noalloc) stores nothing and
  * makes the next gptq_check_status return GPTQ_ERR_LAYOUT.  The CTA-pair switch below does not apply to it. */
 int gptq_gemm_silu_mul(const void *x, const void *qweight, const void *qzeros, const void *scales,

@@ -436,12 +436,12 @@ prefill_kernel(const PrefillArgs a, const __grid_constant__ CUtensorMap w_map, c
         if (!layout_ok && threadIdx.x == 32 * kPrefillFirstEpi) atomicMax(&g_device_status, (int)kStatusLayoutMismatch);
         const int group = is_epi ? 0 : 1 + ((warp - kPrefillFirstDq) >> 2), n_groups = 1 + kPrefillSets;
         const int q = warp & 3;
-        const uint32_t stg = (is_epi ? stg0 : w_ring + (group - 1) * kPrefillStage) + q * (32 * 64);      // (the ring is idle by then)
+        // (the ring is idle by then; with the gate/up epilogue a gate warp has the room of its up warp too)
+        const uint32_t stg = (is_epi ? stg0 : w_ring + (group - 1) * kPrefillStage) + (a.fuse ? (q & 1) * 4096 : q * (32 * 64));
         const uint32_t mrow = lane & 7, mchunk = lane >> 3;       // row and chunk that this lane addresses in a fragment store
         const uint32_t frag = stg + mrow * 64 + ((mchunk ^ (mrow >> 1)) << 4);          // token block i: + 512 i
         const uint32_t prow = lane >> 2, pchunk = lane & 3;       // row (+ 8 t) and chunk of its 16-byte pieces
         const uint32_t piece = stg + prow * 64 + ((pchunk ^ (prow >> 1)) << 4);
-        const uint32_t up_piece = piece + 2 * 32 * 64;
         const bool has_bias = a.bias != nullptr, has_res = a.residual != nullptr;
         pdl_wait();
         const int my_tiles = (a.tiles - tile0 + tile_step - 1) / tile_step;
@@ -475,65 +475,76 @@ prefill_kernel(const PrefillArgs a, const __grid_constant__ CUtensorMap w_map, c
                     __syncwarp();
                 }
                 tmem_wait_ld();
+                if (a.fuse) {
+                    // The up warps hand their fp32 sums to the gate warps, which hold the same fragments 64 columns lower:
+                    // [value][lane] words in the gate warp's part of the stage.
+                    const uint32_t at = stg + lane * 4;
+                    if (q >= 2) {
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    float2 v[4];                     // tokens 8 i + 2 (lane % 4) + (0, 1); columns lane / 4 + 8 j
+                        for (int e = 0; e < 16; ++e) sts_f32(at + e * 128, __uint_as_float(r0[e]));
 #pragma unroll
-                    for (int e = 0; e < 2; ++e) {
-                        v[e] = make_float2(__uint_as_float(r0[4 * i + 2 * e]), __uint_as_float(r0[4 * i + 2 * e + 1]));
-                        v[2 + e] = make_float2(__uint_as_float(r1[4 * i + 2 * e]), __uint_as_float(r1[4 * i + 2 * e + 1]));
+                        for (int e = 0; e < 16; ++e) sts_f32(at + 2048 + e * 128, __uint_as_float(r1[e]));
                     }
-                    if (has_bias) {
+                    named_bar_sync(1 + group, 128);
+                    if (q < 2) {
 #pragma unroll
-                        for (int j = 0; j < 4; ++j) v[j].x += bv[j], v[j].y += bv[j];
-                    }
-                    if (has_res) {
-                        uint32_t rr[4];
-                        ldmatrix_x4_trans(frag + 512 * i, rr);
+                        for (int e = 0; e < 16; ++e) r0[e] = __float_as_uint(silu_mul(__uint_as_float(r0[e]), lds_f32(at + e * 128)));
 #pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&rr[j]));
-                            v[j].x += f.x, v[j].y += f.y;
-                        }
+                        for (int e = 0; e < 16; ++e) r1[e] = __float_as_uint(silu_mul(__uint_as_float(r1[e]), lds_f32(at + 2048 + e * 128)));
                         __syncwarp();
                     }
-                    uint32_t o[4];
+                }
+                if (!a.fuse || q < 2) {
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) o[j] = pack_out16<BF>(v[j]);
-                    stmatrix_x4_trans(frag + 512 * i, o);
+                    for (int i = 0; i < 4; ++i) {
+                        float2 v[4];                 // tokens 8 i + 2 (lane % 4) + (0, 1); columns lane / 4 + 8 j
+#pragma unroll
+                        for (int e = 0; e < 2; ++e) {
+                            v[e] = make_float2(__uint_as_float(r0[4 * i + 2 * e]), __uint_as_float(r0[4 * i + 2 * e + 1]));
+                            v[2 + e] = make_float2(__uint_as_float(r1[4 * i + 2 * e]), __uint_as_float(r1[4 * i + 2 * e + 1]));
+                        }
+                        if (has_bias) {
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) v[j].x += bv[j], v[j].y += bv[j];
+                        }
+                        if (has_res) {
+                            uint32_t rr[4];
+                            ldmatrix_x4_trans(frag + 512 * i, rr);
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) {
+                                const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&rr[j]));
+                                v[j].x += f.x, v[j].y += f.y;
+                            }
+                            __syncwarp();
+                        }
+                        uint32_t o[4];
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) o[j] = pack_out16<BF>(v[j]);
+                        stmatrix_x4_trans(frag + 512 * i, o);
+                    }
+                    __syncwarp();
                 }
                 if (!a.fuse) {
-                    __syncwarp();
 #pragma unroll
                     for (int t = 0; t < 4; ++t)
                         if (ok && (int)prow + 8 * t < nr) *reinterpret_cast<uint4 *>(a.y + y_at + (size_t)(c0 + 8 * t) * a.N) = lds128(piece + 512 * t);
                     __syncwarp();
                 } else {
-                    // gate (warps of lanes 0..63) and up columns are both rounded to fp16 first; the gate warps store
-                    named_bar_sync(1 + group, 128);
                     if (q < 2 && ok) {
                         const int oc = p * 64 + 32 * q + 8 * pchunk;
 #pragma unroll 1
                         for (int t = 0; t < 4; ++t) {
                             if ((int)prow + 8 * t >= nr) break;
-                            const uint4 gv = lds128(piece + 512 * t), uv = lds128(up_piece + 512 * t);
-                            const uint32_t gw[4] = {gv.x, gv.y, gv.z, gv.w}, uw[4] = {uv.x, uv.y, uv.z, uv.w};
-                            uint32_t ow[4];
-#pragma unroll
-                            for (int e = 0; e < 4; ++e) {
-                                const float2 gf = __half22float2(*reinterpret_cast<const __half2 *>(&gw[e]));
-                                const float2 uf = __half22float2(*reinterpret_cast<const __half2 *>(&uw[e]));
-                                const __half2 o = __floats2half2_rn(silu_mul(gf.x, uf.x), silu_mul(gf.y, uf.y));
-                                ow[e] = *reinterpret_cast<const uint32_t *>(&o);
-                            }
+                            const uint4 ov = lds128(piece + 512 * t);
                             __half *orow = a.y + (size_t)(m0 + c0 + prow + 8 * t) * (a.N / 2);
                             if (a.out_index == nullptr) {
-                                *reinterpret_cast<uint4 *>(orow + oc) = make_uint4(ow[0], ow[1], ow[2], ow[3]);
+                                *reinterpret_cast<uint4 *>(orow + oc) = ov;
                             } else {
                                 // scattered columns: eight destinations (two 16-byte index loads), eight 2-byte stores
                                 const int4 ia = *reinterpret_cast<const int4 *>(a.out_index + oc);
                                 const int4 ib = *reinterpret_cast<const int4 *>(a.out_index + oc + 4);
                                 const int dst[8] = {ia.x, ia.y, ia.z, ia.w, ib.x, ib.y, ib.z, ib.w};
+                                const uint32_t ow[4] = {ov.x, ov.y, ov.z, ov.w};
 #pragma unroll
                                 for (int e = 0; e < 8; ++e)
                                     orow[dst[e]] = __ushort_as_half((unsigned short)(ow[e >> 1] >> (16 * (e & 1))));

@@ -1555,6 +1555,26 @@ def test_prefill_kernel(K, N, gs, act, zm1, M, ws):
     assert B.gptq_check_status() == B.GPTQ_OK
 
 
+@pytest.mark.parametrize("M", [17, 31, 64, 130, 300])
+def test_prefill_kernel_silu_mul_keeps_fp32_factors(M, ws):
+    """With power-of-two scales the weights are exact in fp16, so gate and up are fp32 sums (2e-6 of the sum of magnitudes
+    allowed) and the output is rounded once: half an ulp.  Rounding the factors to fp16 first triples that."""
+    K, N = 1024, 19200                                    # 150 panels: several tiles per CTA, and the shared last one
+    L0 = wl.make_linear(K, N, seed=wl.seed_for("silu-fp32"))
+    s = (2.0 ** np.random.default_rng(3).integers(-9, -5, (K // 128, N))).astype(np.float16)
+    L = wl.QuantLinear(K, N, 128, L0.qweight, L0.qzeros, s, None, 0)
+    x = wl.make_x(M, K, wl.seed_for("silu-fp32-x", M))
+    out = H.gemm_silu_mul(H.to_device(x), H.upload_and_repack(L, gate_up=True)).cpu().numpy().astype(np.float64)
+    assert B.gptq_check_status() == B.GPTQ_OK
+    y = oracle.gemm_f64(x, L.qweight, L.qzeros, L.scales, None, 128)
+    w = np.abs(oracle.dequant_f32(L.qweight, L.qzeros, L.scales, None, 128).astype(np.float64))
+    e = 2e-6 * (np.abs(x.astype(np.float64)) @ w)
+    g, u, eg, eu = y[:, :N // 2], y[:, N // 2:], e[:, :N // 2], e[:, N // 2:]
+    want = oracle.silu_mul_f64(y)
+    bound = 2.0 ** -11 * np.abs(want) + 1.1 * eg * np.abs(u) + np.abs(g / (1 + np.exp(-g))) * eu + 2e-6 * np.abs(want) + 2.0 ** -25
+    assert np.all(np.abs(out - want) <= bound), (np.abs(out - want) / bound).max()
+
+
 # ------------------------------------------------------------------------------- how a host batch moves its activations
 @pytest.mark.parametrize("M", [1, 3, 40])
 @pytest.mark.parametrize("count", [1, 8, 9, 21])

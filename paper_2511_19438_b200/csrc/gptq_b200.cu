@@ -834,12 +834,23 @@ static void *device_address_of_host(const void *host)
     return attr.type == cudaMemoryTypeHost ? attr.devicePointer : nullptr;
 }
 // Collects the copies of a chunk: a pinned, aligned host buffer becomes a segment, any other an ordinary asynchronous copy.
+// The segments of a launch are copied in no particular order, so a copy whose destination overlaps a collected one's (several
+// results for one host buffer: the last one stays) starts a new launch.
 struct ChunkCopies {
     CopySegments seg{};
+    const uint8_t *dst_begin[kCopySegments], *dst_end[kCopySegments];      // of the collected segments, as the caller gave them
     cudaStream_t stream;
     bool to_device;
     int add(void *dst, const void *src, size_t bytes)
     {
+        const uint8_t *const begin = (const uint8_t *)dst, *const end = begin + bytes;
+        for (int i = 0; i < seg.count; ++i) {
+            if (begin < dst_end[i] && dst_begin[i] < end) {
+                const int st = flush();
+                if (st) return st;
+                break;
+            }
+        }
         void *host = device_address_of_host(to_device ? src : dst);
         if (host == nullptr || (reinterpret_cast<uintptr_t>(host) & 15u) || bytes % 16 || bytes > (1u << 30))
             return record_cuda_error(cudaMemcpyAsync(dst, src, bytes, to_device ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToHost, stream));
@@ -847,6 +858,8 @@ struct ChunkCopies {
         seg.src[i] = (const uint4 *)(to_device ? host : src);
         seg.dst[i] = (uint4 *)(to_device ? dst : host);
         seg.end[i] = (i ? seg.end[i - 1] : 0u) + (uint32_t)(bytes / 16);
+        dst_begin[i] = begin;
+        dst_end[i] = end;
         seg.count = i + 1;
         return seg.count == kCopySegments ? flush() : GPTQ_OK;
     }

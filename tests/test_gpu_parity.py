@@ -1601,3 +1601,29 @@ def test_host_batch_copies(M, count, ws):
     for (xh, yh, xs, ys, pad), w in zip(keep, want):
         assert torch.equal(yh[pad:pad + M * N].reshape(M, N), w)
         assert bool((yh[:pad] == 7).all()) and bool((yh[pad + M * N:] == 7).all())
+
+
+def test_host_batch_results_for_one_host_buffer(ws):
+    """Problems whose results go to the same host buffer, or to buffers that overlap: the copies down are in the order of the
+    problems, so the last one's result stays, whole."""
+    K, N, count = 512, 2048, 8
+    D = H.upload_and_repack(wl.make_linear(K, N, seed=wl.seed_for("host-overlap")))
+    big = torch.zeros(8 * N, dtype=torch.float16).pin_memory()
+    for rnd in range(20):
+        items, keep, want = [], [], []
+        for i in range(count):
+            M = 1 + (i + rnd) % 3
+            x = torch.from_numpy(wl.make_x(M, K, wl.seed_for("host-overlap-x", i, rnd)))
+            xh = x.pin_memory()
+            xs, ys = torch.empty((M, K), dtype=torch.float16, device="cuda"), torch.empty((M, N), dtype=torch.float16, device="cuda")
+            at = N // 2 * (i % 3)                       # rows of one buffer, half a row apart
+            items.append((xh, D.qweight_t, D.qzeros_t, D.scales_t, None, big.data_ptr() + 2 * at, xs, ys, M, N, K, 128, 0))
+            keep.append((xh, xs, ys))
+            want.append((at, H.gemm(x.cuda(), D).cpu().reshape(-1)))
+        big.fill_(7.0)
+        expect = big.clone()
+        for at, y in want:
+            expect[at:at + y.numel()] = y
+        assert B.gptq_gemm_host_batch(B.make_host_problems(items))[0] == B.GPTQ_OK
+        torch.cuda.synchronize()
+        assert torch.equal(big, expect), rnd

@@ -336,7 +336,8 @@ typedef struct {
  * results, none sharing a staging buffer with another of the last few chunks; large problems go one by one): the x of a chunk go up, its matmuls run back to back on `stream`, its y come down, and chunk c+1 goes up
  * while chunk c computes and chunk c-1 comes down; the matmuls themselves stay in order on `stream`, and `stream`
  * completes after the last copy.  Small activations in pinned memory are copied by a kernel (one per chunk) instead of the
- * copy engines; host buffers that are not pinned, or not 16-byte aligned, always go through cudaMemcpyAsync.  Staging buffers may be shared between problems (reuse waits for the earlier user;
+ * copy engines; host buffers that are not pinned in one piece, or not
+ * 16-byte aligned, always go through cudaMemcpyAsync.  Staging buffers may be shared between problems (reuse waits for the earlier user;
  * problems that share one never sit in the same chunk).
  * All problems are validated before anything is enqueued; on an invalid problem *bad_index (if not
  * NULL) receives its index and nothing runs.  If a later step fails, `stream` is still joined with the
@@ -424,6 +425,10 @@ int gptq_plan_noalloc(int M, int N, int K, int group_size, int act_order, int sm
  * in that order. */
 int gptq_plan_cta_range(int items, int ctas, int cta, int *first_item, int *end_item);
 int gptq_plan_panel_owners(int items, int ctas, int groups, int panel, int *first_cta, int *last_cta);
+/* Likewise: 1 if gptq_gemm_host_batch's copy kernel may walk a host buffer of `bytes` that the device sees at device_address,
+ * in an allocation or registration [range_start, range_start + range_bytes); 0 if it is left to cudaMemcpyAsync. */
+int gptq_plan_host_copy(int pinned_host, unsigned long long device_address, unsigned long long range_start,
+                        unsigned long long range_bytes, unsigned long long bytes);
 
 #ifdef __cplusplus
 }

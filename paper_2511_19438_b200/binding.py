@@ -102,6 +102,7 @@ _SIGNATURES = {
     "gptq_plan_noalloc": (_i, [_i, _i, _i, _i, _i, _i, ctypes.POINTER(gptq_plan_t)]),
     "gptq_plan_cta_range": (_i, [_i, _i, _i, ctypes.POINTER(_i), ctypes.POINTER(_i)]),
     "gptq_plan_panel_owners": (_i, [_i, _i, _i, _i, ctypes.POINTER(_i), ctypes.POINTER(_i)]),
+    "gptq_plan_host_copy": (_i, [_i] + [ctypes.c_ulonglong] * 4),
 }
 for _name, (_res, _args) in _SIGNATURES.items():
     _fn = getattr(_lib, _name)
@@ -393,3 +394,8 @@ def gptq_plan_panel_owners(items, ctas, groups, panel):
     a, b = ctypes.c_int(), ctypes.c_int()
     st = _lib.gptq_plan_panel_owners(items, ctas, groups, panel, ctypes.byref(a), ctypes.byref(b))
     return st, a.value, b.value
+
+
+def gptq_plan_host_copy(pinned_host, device_address, range_start, range_bytes, nbytes):
+    """1 if the host batch's copy kernel may walk such a host buffer, 0 if it is left to cudaMemcpyAsync.  Host-only."""
+    return _lib.gptq_plan_host_copy(int(pinned_host), device_address, range_start, range_bytes, nbytes)

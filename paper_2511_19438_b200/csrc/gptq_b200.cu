@@ -823,15 +823,36 @@ __global__ void __launch_bounds__(kCopyThreads) copy_segments_kernel(const __gri
             if (to[u]) *to[u] = v[u];
     }
 }
-// The address under which the device sees host memory, if it is pinned (else nullptr).
-static void *device_address_of_host(const void *host)
+// Whether the copy kernel may walk a host buffer: pinned host memory (not managed) whose one allocation or registration holds
+// all of it, in whole aligned 16-byte pieces.  A buffer that only begins in pinned memory is the copy engine's, which returns
+// an error where the kernel would fault.
+static bool host_copy_by_kernel(bool pinned_host, uint64_t device_address, uint64_t range_start, uint64_t range_bytes, uint64_t bytes)
 {
-    cudaPointerAttributes attr{};
-    if (cudaPointerGetAttributes(&attr, host) != cudaSuccess) {
-        (void)cudaGetLastError();
-        return nullptr;
+    return pinned_host && device_address % 16 == 0 && bytes % 16 == 0 && bytes <= (1u << 30) && device_address >= range_start &&
+           bytes <= range_bytes && device_address - range_start <= range_bytes - bytes;
+}
+// The address under which the device sees a host buffer that the copy kernel may walk, else nullptr.
+static void *device_address_of_host(const void *host, size_t bytes)
+{
+    typedef CUresult (*AttributesFn)(unsigned int, CUpointer_attribute *, void **, CUdeviceptr);
+    static std::atomic<AttributesFn> cached{nullptr};
+    AttributesFn get = cached.load(std::memory_order_acquire);
+    if (get == nullptr) {
+        void *fn = nullptr;
+        cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
+        if (cudaGetDriverEntryPoint("cuPointerGetAttributes", &fn, cudaEnableDefault, &q) != cudaSuccess) (void)cudaGetLastError();
+        if (q != cudaDriverEntryPointSuccess || fn == nullptr) return nullptr;
+        get = (AttributesFn)fn;
+        cached.store(get, std::memory_order_release);
     }
-    return attr.type == cudaMemoryTypeHost ? attr.devicePointer : nullptr;
+    CUpointer_attribute what[5] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED, CU_POINTER_ATTRIBUTE_DEVICE_POINTER,
+                                   CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    unsigned int type = 0, managed = 0;
+    CUdeviceptr device = 0, start = 0;
+    size_t size = 0;                            // (stays 0 for memory that the driver does not know)
+    void *into[5] = {&type, &managed, &device, &start, &size};
+    if (get(5, what, into, (CUdeviceptr)(uintptr_t)host) != CUDA_SUCCESS) return nullptr;
+    return host_copy_by_kernel(type == CU_MEMORYTYPE_HOST && !(managed & 255u), device, start, size, bytes) ? (void *)(uintptr_t)device : nullptr;
 }
 // Collects the copies of a chunk: a pinned, aligned host buffer becomes a segment, any other an ordinary asynchronous copy.
 // The segments of a launch are copied in no particular order, so a copy whose destination overlaps a collected one's (several
@@ -851,8 +872,8 @@ struct ChunkCopies {
                 break;
             }
         }
-        void *host = device_address_of_host(to_device ? src : dst);
-        if (host == nullptr || (reinterpret_cast<uintptr_t>(host) & 15u) || bytes % 16 || bytes > (1u << 30))
+        void *host = device_address_of_host(to_device ? src : dst, bytes);
+        if (host == nullptr)
             return record_cuda_error(cudaMemcpyAsync(dst, src, bytes, to_device ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToHost, stream));
         const int i = seg.count;
         seg.src[i] = (const uint4 *)(to_device ? host : src);
@@ -1027,6 +1048,12 @@ static int host_batch(const gptq_host_problem_t *problems, int count, void *stre
 }
 
 extern "C" {
+
+int gptq_plan_host_copy(int pinned_host, unsigned long long device_address, unsigned long long range_start,
+                        unsigned long long range_bytes, unsigned long long bytes)
+{
+    return host_copy_by_kernel(pinned_host != 0, device_address, range_start, range_bytes, bytes) ? 1 : 0;
+}
 
 int gptq_gemm_host_batch(const gptq_host_problem_t *problems, int count, void *stream, int *bad_index)
 {

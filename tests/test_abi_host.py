@@ -144,6 +144,23 @@ def test_host_batch_validates_every_problem_before_running():
     assert B._lib.gptq_gemm_host_batch(arr, 0, 0, None) == B.GPTQ_OK      # an empty step is fine
 
 
+def test_host_batch_copy_kernel_stays_inside_one_pinned_range():
+    """Only pinned memory that one allocation or registration holds from the first byte to the last is walked by the kernel: a
+    buffer that runs out of it (into pageable memory, or into another registration) is left to cudaMemcpyAsync."""
+    start, size = 0x7f0000000000, 1 << 20
+    ok = B.gptq_plan_host_copy
+    assert ok(1, start, start, size, size) == 1 and ok(1, start + 4096, start, size, 8192) == 1
+    assert ok(1, start + size - 16, start, size, 16) == 1
+    assert ok(0, start, start, size, 4096) == 0                       # pageable or managed
+    assert ok(1, start + size - 4096, start, size, 4112) == 0          # begins inside, ends outside
+    assert ok(1, start, start, size, size + 16) == 0
+    assert ok(1, start + size, start, size, 16) == 0 and ok(1, start - 16, start, size, 32) == 0
+    assert ok(1, start, start, 0, 16) == 0 and ok(1, start, 0, 0, 16) == 0    # a range the driver does not tell
+    assert ok(1, start + 8, start, size, 4096) == 0 and ok(1, start, start, size, 4104) == 0      # 16-byte pieces
+    assert ok(1, start, start, 1 << 40, (1 << 30) + 16) == 0
+    assert ok(1, (1 << 64) - 64, start, size, 128) == 0                # no wrap-around
+
+
 def test_repack_bytes_equal_canonical_sizes_plus_trailer():
     for (K, N) in list(wl.SHAPES_7B.values()) + list(wl.SHAPES_13B.values()):
         G = K // 128

@@ -430,7 +430,7 @@ umma_kernel(const UmmaArgs a, const __grid_constant__ CUtensorMap w_map, const _
                 // A set skips the other sets' slots, so its parity wait on a slot is only unambiguous once the slot's
                 // previous refill is known to have landed: the MMAs of that refill's last block have completed.
                 const int c = (b / BPS - NS) * BPS + BPS - 1;
-                if (c > 0) ok = __all_sync(0xffffffffu, wait(bar_done + 8 * (c & (kUmmaDoneRing - 1)), (uint32_t)((c / kUmmaDoneRing) & 1)));
+                if (c >= 0) ok = __all_sync(0xffffffffu, wait(bar_done + 8 * (c & (kUmmaDoneRing - 1)), (uint32_t)((c / kUmmaDoneRing) & 1)));
                 ok = ok && __all_sync(0xffffffffu, wait(bar_full + 8 * s, ph));   // warp-uniform
                 if (!ok) break;
             }

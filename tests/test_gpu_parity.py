@@ -1575,6 +1575,20 @@ def test_prefill_kernel_silu_mul_keeps_fp32_factors(M, ws):
     assert np.all(np.abs(out - want) <= bound), (np.abs(out - want) / bound).max()
 
 
+def test_umma_ring_of_one_block_slots_wraps(ws):
+    """128-token tiles of the one-tile-per-CTA kernel hold one K64 block per ring slot: five slots for the six blocks of K = 384,
+    so the first slot is used again, and what it held is the block the other waits are measured from (number 0)."""
+    K, N, M = 384, 19200, 100                             # 150 panels: two CTAs on an SM
+    st, pl = B.gptq_plan(M, N, K, 128, 0, 148)
+    assert st == B.GPTQ_OK and pl.stages == 5 and pl.m_tile == 128 and B.gptq_plan_prefill(M, N, K, 128, 0, 0, 148)[0] == B.GPTQ_ERR_UNSUPPORTED
+    L = wl.make_linear(K, N, seed=wl.seed_for("ring-wrap"))
+    x = wl.make_x(M, K, wl.seed_for("ring-wrap-x"))
+    y, D = run_gemm(L, x, ws)
+    sampled_check(L, x, y, 20000, seed=5)
+    for _ in range(3):
+        assert np.array_equal(H.gemm(H.to_device(x), D).cpu().numpy(), y)
+
+
 # ------------------------------------------------------------------------------- how a host batch moves its activations
 @pytest.mark.parametrize("M", [1, 3, 40])
 @pytest.mark.parametrize("count", [1, 8, 9, 21])

@@ -35,6 +35,12 @@ constexpr int kPrefillStage = 4 * 32 * 64;                           // epilogue
 // A stages (of one item, 64 columns) and columns of an accumulator: tensor memory holds 2 x 128 + 4 x 64 or 2 x 160 + 3 x 64
 __host__ __device__ constexpr int prefill_a_stages(int tok) { return tok <= 128 ? 4 : 3; }
 __host__ __device__ constexpr int prefill_acc_columns(int tok) { return tok <= 128 ? 128 : 160; }
+// Fewest items of a tile that a CTA works through alone (without a split of K).  The dequant warps take part in the epilogue of
+// the CTA's last tile only, and wait for its accumulator by parity without having waited for the tile before the last but one,
+// which used the same accumulator: if that were still being multiplied, the wait would pass at once.  It is not: a set's last
+// item, one of the CTA's last kPrefillSets, has waited for the MMAs of the item an A ring earlier, and two tiles lie behind.
+constexpr int kPrefillMinItems = 4;
+static_assert(2 * kPrefillMinItems + 1 > kPrefillSets + prefill_a_stages(0), "a dequant warp's wait for the last tile's accumulator would be ambiguous");
 // Weight slots.  A set's parity wait on a slot needs the slot's previous item to be in: with this many that is known, the
 // set's last pass (four items ago) has waited for the MMAs of the item that had its A stage before.  With 8-bit weights
 // (16 KB per slot) five, and the set asks.
@@ -456,7 +462,7 @@ prefill_kernel(const PrefillArgs a, const __grid_constant__ CUtensorMap w_map, c
 #pragma unroll
                 for (int j = 0; j < 4; ++j) bv[j] = __half2float(a.bias[(size_t)p * kPanel + 32 * q + 8 * j + (lane >> 2)]);
             }
-            decode_wait(bar_dfull + 8 * d, ph, flag);
+            decode_wait(bar_dfull + 8 * d, ph, flag);        // (unambiguous for the dequant warps too: kPrefillMinItems)
             __syncwarp();
             tc_fence_after_sync();
             const bool ok = layout_ok && lds32(flag) == 0;
@@ -594,7 +600,7 @@ inline PrefillPlan plan_prefill(int M, int N, int K, int sm_count, bool w8, bool
 {
     PrefillPlan pl{};
     const int panels = N / kPanel, G = K / kGroup;
-    if (G < kPrefillSets) return pl;
+    if (G < kPrefillMinItems) return pl;     // (a condition of correctness, see there)
     long long best = -1;
     for (int S = 1; S <= (may_split ? 4 : 1); S *= 2) {
         for (int most = kPrefillMaxTok; most >= 32; most -= 16) {

@@ -161,6 +161,56 @@ def test_host_batch_copy_kernel_stays_inside_one_pinned_range():
     assert ok(1, (1 << 64) - 64, start, size, 128) == 0                # no wrap-around
 
 
+@pytest.mark.parametrize("sms", [148, 132, 7])
+def test_persistent_plan_is_consistent(sms):
+    """gptq_plan_prefill: nothing below 17 rows and four 128-row items; tiles cover the rows and a grid covers the tiles, at most
+    one CTA (or cluster of two or four, one tile each) per SM; an x ring of at least one item inside the shared memory."""
+    taken = 0
+    for K in (128, 384, 512, 640, 4096, 11008, 13824):
+        for N in (128, 256, 4096, 4480, 12288, 22016, 27648):
+            for M in (1, 16, 17, 33, 64, 100, 128, 129, 161, 300, 512, 1000, 4096):
+                for w8 in (0, 1):
+                    st, pl = B.gptq_plan_prefill(M, N, K, 128, 0, w8, sms)
+                    if M < 17 or K < 512:
+                        assert st == B.GPTQ_ERR_UNSUPPORTED
+                    if st != B.GPTQ_OK:
+                        assert st == B.GPTQ_ERR_UNSUPPORTED
+                        continue
+                    taken += 1
+                    assert pl.kernel == 5 and pl.m_tile % 16 == 0 and 16 <= pl.m_tile <= 160
+                    tiles = (N // 128) * -(-M // pl.m_tile)
+                    assert pl.cluster_size in (1, 2, 4) and pl.cluster_size <= K // 128
+                    if pl.cluster_size == 1:
+                        assert pl.ctas == min(tiles, sms)
+                    else:
+                        assert pl.ctas == tiles * pl.cluster_size <= sms
+                    assert 1 <= pl.stages <= 4 and 113 * 1024 < pl.smem_bytes <= 227 * 1024
+    assert taken > 100
+
+
+@pytest.mark.parametrize("sms", [148, 132])
+def test_decode_plan_is_consistent(sms):
+    """gptq_plan_decode: one or two rows only; a grid of whole clusters within the SMs, none of them without a panel; two CTAs fit an
+    SM and a third does not; at least four steps of weights."""
+    taken = 0
+    for gs in (128, 64, 32):
+        for K in (1024, 4096, 5120, 8192, 11008, 13824, 27648):
+            for N in (1024, 2048, 4096, 12288, 22016, 27648):
+                for M in (1, 2, 3):
+                    st, pl = B.gptq_plan_decode(M, N, K, gs, 0, sms)
+                    if M > 2:
+                        assert st == B.GPTQ_ERR_UNSUPPORTED
+                    if st != B.GPTQ_OK:
+                        assert st == B.GPTQ_ERR_UNSUPPORTED
+                        continue
+                    taken += 1
+                    clusters = pl.ctas // pl.cluster_size
+                    assert pl.kernel == 4 and 1 <= pl.cluster_size <= 8 and pl.ctas == clusters * pl.cluster_size <= sms
+                    assert clusters <= N // 128 and pl.stages >= 4
+                    assert 2 * (pl.smem_bytes + 1024) <= 227 * 1024 < 3 * (pl.smem_bytes + 1024)
+    assert taken > 20
+
+
 def test_repack_bytes_equal_canonical_sizes_plus_trailer():
     for (K, N) in list(wl.SHAPES_7B.values()) + list(wl.SHAPES_13B.values()):
         G = K // 128

@@ -149,7 +149,10 @@ splitk_kernel(const SplitKArgs a, const __grid_constant__ CUtensorMap x_map)
     const uint32_t bar_empty = smem_base + 64;            // stages x 8 B
     const uint32_t bar_recv = smem_base + 128;
     const uint32_t ring = smem_base + kRingOffset;
-    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // warp: uniform
+    // The warp's number comes from a shuffle, so that it is known to be uniform - but for 16 rows in groups of 32, whose register
+    // allocation that pushed over the three resident CTAs' 72: 128 bytes of spill loads per item (7B layer of four, M = 12: 59.2 us, 56.4 without).
+    constexpr bool kPlainWarp = MT == 2 && SUB == 4 && !BF;
+    const int warp = kPlainWarp ? (int)threadIdx.x >> 5 : __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const int S = a.S;
     const int p = blockIdx.x / S, rank = blockIdx.x - p * S;   // cluster = the S CTAs of panel p
     const int g0 = rank * a.G / S, g1 = (rank + 1) * a.G / S;  // this CTA's groups

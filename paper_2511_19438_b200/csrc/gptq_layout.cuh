@@ -290,8 +290,60 @@ gather_x_rows_kernel(const __half *__restrict__ x, const int32_t *__restrict__ p
     }
 }
 
+// The gather in front of the decode kernel (one or two rows): x_out[m][i] = x[m][perm[i]] for i < n, kCols columns per thread, so
+// that its few blocks find room on the SMs that the decode kernel's grid leaves over.  A block that shares an SM with a decode
+// CTA keeps the next launch's CTA from joining them - two of those fill the registers - and that launch's prefetch waits for the
+// gather.  Four columns up to n = 8192 (less to do per block), eight above (fewer blocks).  Chains of one layer at M = 1, us, with
+// one column per thread / four / eight: 4096 x 12288 with act-order 7.8 / 8.1 / 8.8, 5120 x 27648 19.2 / 13.7 / 13.7,
+// 13824 x 27648 with 8-bit weights 103 / 104 / 72; the mma.sync kernel takes 9.8, 18.1 and 78.
+constexpr int kGatherWideRows = 2, kGatherWideThreads = 256;
+template <int kCols>
+__global__ void __launch_bounds__(kGatherWideThreads) gather_x_wide_kernel(const __half *__restrict__ x, const int32_t *__restrict__ perm,
+                                                                           __half *__restrict__ x_out, int M, int K, int n)
+{
+    pdl_launch_dependents();   // as in gather_x_kernel
+    pdl_wait();
+    const int i = kCols * (blockIdx.x * kGatherWideThreads + threadIdx.x);
+    if (i >= n) return;
+    int4 idx[kCols / 4];
+#pragma unroll
+    for (int c = 0; c < kCols / 4; ++c) idx[c] = *reinterpret_cast<const int4 *>(perm + i + 4 * c);
+#pragma unroll 2
+    for (int m = 0; m < M; ++m) {
+        const __half *const row = x + (size_t)m * K;
+        __half2 v[kCols / 2];
+#pragma unroll
+        for (int c = 0; c < kCols / 4; ++c) {
+            v[2 * c] = __halves2half2(row[idx[c].x], row[idx[c].y]);
+            v[2 * c + 1] = __halves2half2(row[idx[c].z], row[idx[c].w]);
+        }
+#pragma unroll
+        for (int c = 0; c < kCols / 4; ++c) {
+            const uint2 w = make_uint2(*reinterpret_cast<const uint32_t *>(&v[2 * c]), *reinterpret_cast<const uint32_t *>(&v[2 * c + 1]));
+            *reinterpret_cast<uint2 *>(x_out + (size_t)m * n + i + 4 * c) = w;
+        }
+    }
+}
+// n: K, or 2 K where an 8-bit layer's rows are stacked; a multiple of 8
+int launch_gather_x_wide(const __half *x, const int32_t *perm, __half *x_out, int M, int K, int n, cudaStream_t s)
+{
+    const int cols = n <= 8192 ? 4 : 8;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)((n / cols + kGatherWideThreads - 1) / kGatherWideThreads));
+    cfg.blockDim = dim3(kGatherWideThreads);
+    cfg.dynamicSmemBytes = 0;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return record_cuda_error(cudaLaunchKernelEx(&cfg, cols == 4 ? gather_x_wide_kernel<4> : gather_x_wide_kernel<8>, x, perm, x_out, M, K, n));
+}
+
 int launch_gather_x(const __half *x, const int32_t *perm, __half *x_out, int M, int K, cudaStream_t s)
 {
+    if (M <= kGatherWideRows && K % 8 == 0) return launch_gather_x_wide(x, perm, x_out, M, K, K, s);
     const size_t rows_smem = (size_t)kGatherRows * K * sizeof(__half);
     // measured on the 7B shapes: pays from about a thousand rows on (M = 4096: 17-57 us instead of 48-250), from 512
     // rows on the long-K layers; below that its few blocks leave most SMs idle and the element-per-thread kernel wins

@@ -98,6 +98,7 @@ __global__ void w8_gather_x_kernel(const __half *__restrict__ x, const int32_t *
 
 int launch_w8_gather_x(const __half *x, const int32_t *perm, __half *x_out, int M, int K, cudaStream_t s)
 {
+    if (M <= kGatherWideRows) return launch_gather_x_wide(x, perm, x_out, M, K, 2 * K, s);
     const int T = 256;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((2 * K + T - 1) / T, (unsigned)min(M, 64));

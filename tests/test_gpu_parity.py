@@ -1510,6 +1510,24 @@ def test_decode_kernel_infinite_and_nan_activations(K, N, gs, act, zm1, ws):
     assert B.gptq_check_status() == B.GPTQ_OK
 
 
+@pytest.mark.parametrize("K", [128, 1024, 4224, 8192, 8320])       # four columns per thread up to 8192, eight above; last blocks partly used
+@pytest.mark.parametrize("M", [1, 2, 3])
+def test_gather_of_few_rows(K, M, ws):
+    """The gathered activations of an act-order layer are those of a caller who sorts them: the same bits; 8-bit layers gather 2 K."""
+    L = wl.make_linear(K, 256, seed=wl.seed_for("gather", K), act_order=True)
+    x_np = wl.make_x(M, K, wl.seed_for("gather-x", M, K))
+    y, D = run_gemm(L, x_np, ws)
+    x = H.to_device(x_np)
+    assert np.array_equal(H.gemm_presorted(x[:, D.perm.long()].contiguous(), D).cpu().numpy(), y)
+    L8 = wl.make_linear_w8(K, 256, seed=wl.seed_for("gather-w8", K), act_order=True)
+    D8 = H.upload_and_repack_w8(L8)
+    H.ensure_for_w8(ws, M, D8)
+    y8 = H.gemm_w8(x, D8).cpu().numpy().astype(np.float64)
+    want = oracle.gemm_f64_w8(x_np, L8.qweight, L8.qzeros, L8.scales, L8.g_idx, 128)
+    assert np.all(np.abs(y8 - want) <= 16 * 1e-4 * max(1.0, math.sqrt(K / 4096)) + 2.0 ** -11 * np.abs(want))
+    assert B.gptq_check_status() == B.GPTQ_OK
+
+
 # ------------------------------------------------------------------------------- 8-bit weights joined in the tcgen05 kernel
 @pytest.mark.parametrize("K,N,gs", [(384, 256, 128), (384, 256, 64), (256, 128, 32), (2048, 4864, 128)])
 @pytest.mark.parametrize("M", [17, 33, 64, 65, 129, 257])

@@ -150,7 +150,10 @@ int gptq_set_workspace(void *ptr, size_t bytes);
  * GPTQ_ERR_ALIGN; without act-order it may be NULL).
  * fp32 accumulation, one round-to-nearest-even conversion to fp16.  Any M >= 1.  Up to 16 rows the
  * weights enter the MMA as exact integers q - z and the scale multiplies fp32 group sums; above
- * that each scaled weight is rounded to fp16 once before the MMA.
+ * that each scaled weight is rounded to fp16 once before the MMA.  (One and two rows, where gptq_plan_decode takes the
+ * problem: sum q x and z sum x are formed apart, both in fp32, and subtracted per group.  The error before the one
+ * rounding of y is then that of fp32 sums of q |x| + z |x| instead of |q - z| |x|: about 1e-7 s sum (q + z) |x|, so a
+ * column with q = z throughout gives y of that size instead of 0.)
  * The kernels begin fetching weights before earlier work on the stream has finished
  * (programmatic dependent launch); x, y and the workspace are only touched afterwards.  The
  * weight buffers must therefore not be written by a kernel launched immediately before this
@@ -412,7 +415,8 @@ int gptq_plan(int M, int N, int K, int group_size, int act_order, int sm_count, 
  * working through several panels; `stages` = depth of the weight ring in steps. */
 int gptq_plan_decode(int M, int N, int K, int group_size, int act_order, int sm_count, gptq_plan_t *out);
 /* The same for the persistent kernel (kernel 5), which takes problems of 17 and more token rows unless kernel 2 is
- * estimated faster; eight_bit is nonzero for gptq_gemm_w8.  `m_tile` = token rows per tile, `stages` =
+ * estimated faster; eight_bit is nonzero for gptq_gemm_w8.  What it says holds
+ * for calls without the gate/up epilogue: with it the K range is never split.  `m_tile` = token rows per tile, `stages` =
  * depth of the x ring in 128-row items, `cluster_size` = CTAs that share the K range of a tile. */
 int gptq_plan_prefill(int M, int N, int K, int group_size, int act_order, int eight_bit, int sm_count, gptq_plan_t *out);
 /* The same for gptq_gemm_noalloc (stream-K kernel; workspace_bytes is its need of the built-in scratch). */

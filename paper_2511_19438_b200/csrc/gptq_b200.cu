@@ -351,7 +351,7 @@ int gptq_plan_prefill(int M, int N, int K, int group_size, int act_order, int ei
     st = check_fast_path(N, K, group_size);
     if (st) return st;
     if (sm_count < 1) return GPTQ_ERR_SHAPE;
-    const PrefillPlan pl = plan_prefill(M, N, K, sm_count, eight_bit != 0, true);
+    const PrefillPlan pl = plan_prefill(M, N, K, group_size, sm_count, eight_bit != 0, true);
     if (M < kUmmaMinTokens || !pl.use) return GPTQ_ERR_UNSUPPORTED;
     out->kernel = 5;
     out->m_tile = pl.tok;
@@ -480,10 +480,11 @@ static int gemm_dispatch(const void *x, const void *qweight, const void *qzeros,
             const Umma2Plan p2 = plan_umma2(M, N, K);
             return launch_umma2(xin, qweight, qzeros, scales, (__half *)y, M, N, K, p2, s);
         }
-        if (const PrefillPlan pp = plan_prefill(M, N, K, sms, false, !fuse); pp.use)
+        if (const PrefillPlan pp = plan_prefill(M, N, K, group_size, sms, false, !fuse); pp.use)
             return launch_prefill(xin, qweight, qzeros, scales, (__half *)y, M, N, K, group_size, pp, fuse, (const __half *)bias,
                                   (const __half *)residual, out_index, bf16, 0, s);
-        // few tiles and a long K: 32- to 256-token tiles, K split over clusters of up to eight
+        // what the persistent kernel leaves: K below 512; few tiles and a long K (34 to 37 panels, up to 64 rows), split over
+        // clusters of up to eight; many rows in groups of 32
         const UmmaPlan pl = plan_umma(M, N, K, sms);
         return launch_umma(xin, qweight, qzeros, scales, (__half *)y, M, N, K, group_size, pl, fuse, (const __half *)bias,
                            (const __half *)residual, out_index, bf16, 0, s);
@@ -624,7 +625,7 @@ int gptq_gemm_w8(const void *x, const void *qweight, const void *qzeros, const v
         // the tcgen05 kernel joins the planes itself: x once, in the row order of either plane
         st = launch_gather_x((const __half *)x, perm, (__half *)ws.ptr, M, K, (cudaStream_t)stream);
         if (st) return st;
-        if (const PrefillPlan pp = plan_prefill(M, N, K, sms, true, true); pp.use)
+        if (const PrefillPlan pp = plan_prefill(M, N, K, tiled, sms, true, true); pp.use)
             return launch_prefill((const __half *)ws.ptr, qweight, qzeros, scales, (__half *)y, M, N, K, tiled, pp, 0, nullptr,
                                   nullptr, nullptr, 0, 1, (cudaStream_t)stream);
         return launch_umma((const __half *)ws.ptr, qweight, qzeros, scales, (__half *)y, M, N, K, tiled,

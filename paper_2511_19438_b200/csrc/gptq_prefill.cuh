@@ -596,12 +596,12 @@ struct PrefillPlan {
 // this kernel without a split: K = 11008, M = 64: 64 panels 27.2 here, 24.2 there; 80 panels 28.5 / 38.7.  K = 4096, M = 64:
 // 32 panels 10.6 / 9.5, 40 panels 10.8 / 11.6.  K = 4096, M = 256: 16 panels 13.6 / 15.6.  M = 16 (the mma.sync kernel's) on
 // 96 panels 11.4 / 11.1, on 32 panels 10.0 / 5.8.
-inline PrefillPlan plan_prefill(int M, int N, int K, int sm_count, bool w8, bool may_split)
+inline PrefillPlan plan_prefill(int M, int N, int K, int group_size, int sm_count, bool w8, bool may_split)
 {
     PrefillPlan pl{};
     const int panels = N / kPanel, G = K / kGroup;
     if (G < kPrefillMinItems) return pl;     // (a condition of correctness, see there)
-    long long best = -1;
+    long long best = -1, best_waves = 0;
     for (int S = 1; S <= (may_split ? 4 : 1); S *= 2) {
         for (int most = kPrefillMaxTok; most >= 32; most -= 16) {
             const int t = (M + most - 1) / most;
@@ -612,6 +612,7 @@ inline PrefillPlan plan_prefill(int M, int N, int K, int sm_count, bool w8, bool
             const long long clocks = waves * ((long long)((G + S - 1) / S) * (mma > any ? mma : any) + 1500) + 900 + (S > 1 ? 6000 : 0);
             if (best < 0 || clocks < best) {
                 best = clocks;
+                best_waves = waves;
                 pl.S = S;
                 pl.tok = tok;
                 pl.tiles = (int)tiles;
@@ -622,6 +623,17 @@ inline PrefillPlan plan_prefill(int M, int N, int K, int sm_count, bool w8, bool
     const UmmaPlan split = plan_umma(M, N, K, sm_count, w8);
     const int percent = (split.tok <= 64 ? 100 : split.tok == 128 ? 117 : 150) * (w8 ? (split.tok <= 128 ? 18 : 13) : 10) / 10;
     if (split.one_wave && 6500 + split.estimate * 243 * percent / 1000 < best) return pl;
+    // Groups of 32 rows cost this kernel about 0.25 us per item beside the MMA, which tiles of 256 rows pay half as often.  Both
+    // kernels' times in us, fitted to 208 problems of 150 rows and more (K = 1408 to 13824, N = 2048 to 27648): the choice is
+    // 0.6 % off the better one on average, this kernel always 3.8 %.  There / here: 13824 x 27648, 200 rows 155 / 237, 1000 rows
+    // 676 / 802; 11008 x 4096, 900 rows 71 / 86; 4096 x 4096, 900 rows 27 / 31; 5120 x 15360, 320 rows 62 / 41.
+    if (group_size == 32 && !w8 && may_split && split.tok == 256) {
+        const int tail = split.tail_tiles > 0, waves = (split.ctas + sm_count - 1) / sm_count + tail;
+        const int items = split.S > 1 ? (G + split.S - 1) / split.S : (waves - tail) * G + (tail ? (G + split.tail_S - 1) / split.tail_S : 0);
+        const double there = 0.85 * items + 4.5 * waves - 5.3 + (split.S > 1 || tail ? 6.5 : 0);
+        const double here = (double)best_waves * (((G + pl.S - 1) / pl.S) * (0.00208 * pl.tok + 0.25) + 0.45) - 1.2 + (pl.S > 1 ? 5.7 : 0);
+        if (1.05 * there < here) return pl;
+    }
     pl.use = true;
     pl.ctas = pl.S > 1 ? pl.tiles * pl.S : pl.tiles < sm_count ? pl.tiles : sm_count;
     const int fixed = 2048 + kPrefillStage + prefill_w_slots(pl.tok, w8) * (w8 ? 2 : 1) * kItemWBytes, x_slot = pl.tok * 256;

@@ -211,6 +211,14 @@ def test_decode_plan_is_consistent(sms):
     assert taken > 20
 
 
+def test_persistent_plan_leaves_many_rows_in_groups_of_32():
+    """In groups of 32 the kernel with 256-row tiles keeps the row counts that fill its tiles; other formats are not concerned."""
+    for (K, N, M, left) in ((13824, 27648, 1000, True), (11008, 4096, 900, True), (4096, 12288, 256, True), (4096, 12288, 300, False),
+                            (5120, 15360, 320, False), (13824, 27648, 128, False), (4096, 4096, 64, False)):
+        assert (B.gptq_plan_prefill(M, N, K, 32, 0, 0, 148)[0] == B.GPTQ_ERR_UNSUPPORTED) == left, (K, N, M)
+        assert B.gptq_plan_prefill(M, N, K, 32, 0, 1, 148)[0] == B.GPTQ_OK and B.gptq_plan_prefill(M, N, K, 128, 0, 0, 148)[0] == B.GPTQ_OK
+
+
 def test_repack_bytes_equal_canonical_sizes_plus_trailer():
     for (K, N) in list(wl.SHAPES_7B.values()) + list(wl.SHAPES_13B.values()):
         G = K // 128

@@ -9,8 +9,10 @@
 //   * The number of token rows of a tile is a run-time multiple of 16, so that tiles and waves come out even: 300 rows on 96
 //     panels are three tiles of 112 in two waves, where tiles of 256 cost two waves of 256.
 //   * Four sets of four dequant warps take every fourth item each: a set's pass takes about 1000 clocks, most of it latency.
-//   * x lands on the barrier of its item's A stage, so the MMA thread has one wait per item; weights run ahead in a ring of
-//     their own (and start before the previous kernel has finished).
+//   * x lands on the barrier that the item's dequant warps arrive on, so the MMA thread has one wait per item.  These barriers are
+//     a ring of 16, so x may be requested further ahead than there are A stages: an x tile arrives 1500 clocks after its request,
+//     and with tiles of 160 rows, which have three A stages, four slots of x instead of three give 1 to 4 % (2048 x 4096 x 12288
+//     149 -> 143 us).  Weights run ahead in a ring of their own (and start before the previous kernel has finished).
 //   * Where tiles are few, clusters of two or four CTAs share the K range of a tile (one tile per cluster then).
 // What bounds it.  From 128 token rows per tile the MMA: 572 clocks per item of 512 at full rate (qkv M = 512), and then the
 // power limit (1.45-1.5 GHz in that loop).  With fewer rows instruction issue: about 520 clocks per item, for four dequant
@@ -41,6 +43,7 @@ __host__ __device__ constexpr int prefill_acc_columns(int tok) { return tok <= 1
 // item, one of the CTA's last kPrefillSets, has waited for the MMAs of the item an A ring earlier, and two tiles lie behind.
 constexpr int kPrefillMinItems = 4;
 static_assert(2 * kPrefillMinItems + 1 > kPrefillSets + prefill_a_stages(0), "a dequant warp's wait for the last tile's accumulator would be ambiguous");
+constexpr int kPrefillXSlots = 4;            // of x, at most: more gained nothing at 128 rows and less, up to 16 were tried
 // Weight slots.  A set's parity wait on a slot needs the slot's previous item to be in: with this many that is known, the
 // set's last pass (four items ago) has waited for the MMAs of the item that had its A stage before.  With 8-bit weights
 // (16 KB per slot) five, and the set asks.
@@ -94,7 +97,7 @@ struct PrefillArgs {
     __half *y;
     int M, N, G;                      // G: 128-row items of K (of one plane with 8-bit weights)
     int S;                            // CTAs (a cluster) that share the K range of a tile; then every cluster has one tile
-    int tok, tiles, x_slots;          // token rows per tile; tiles; depth of the x ring in items (at most the A stages)
+    int tok, tiles, x_slots;          // token rows per tile; tiles; depth of the x ring in items
     const TiledTrailer *trailer;
     int fuse;
     const __half *bias, *residual;
@@ -117,9 +120,9 @@ prefill_kernel(const PrefillArgs a, const __grid_constant__ CUtensorMap w_map, c
         }
     }
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-    // wfull[s]: packed weights of a ring slot have landed; afull[k]: A stage k has been written and the item's x has landed;
-    // done[n mod 16]: the MMAs of the CTA's n-th item have completed; dfull / dempty: accumulators
-    const uint32_t bar_wfull = base, bar_afull = base + 128, bar_done = base + 192, bar_dfull = base + 320,
+    // wfull[s]: packed weights of a ring slot have landed; afull[n mod 16]: the A operand of the CTA's n-th item has been written and
+    // its x has landed; done[n mod 16]: the MMAs of the CTA's n-th item have completed; dfull / dempty: accumulators
+    const uint32_t bar_wfull = base, bar_afull = base + 384, bar_done = base + 192, bar_dfull = base + 320,
                    bar_dempty = base + 336;
     const uint32_t tmem_slot = base + 352, flag = base + 356, bar_recv = base + 360;
     const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
@@ -134,8 +137,10 @@ prefill_kernel(const PrefillArgs a, const __grid_constant__ CUtensorMap w_map, c
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < WS; ++s) mbar_init(bar_wfull + 8 * s, 1);
-        for (int s = 0; s < PS; ++s) mbar_init(bar_afull + 8 * s, 5);
-        for (int s = 0; s < kUmmaDoneRing; ++s) mbar_init(bar_done + 8 * s, 1);
+        for (int s = 0; s < kUmmaDoneRing; ++s) {
+            mbar_init(bar_afull + 8 * s, 5);
+            mbar_init(bar_done + 8 * s, 1);
+        }
         for (int s = 0; s < 2; ++s) {
             mbar_init(bar_dfull + 8 * s, 1);
             mbar_init(bar_dempty + 8 * s, 4);
@@ -175,16 +180,17 @@ prefill_kernel(const PrefillArgs a, const __grid_constant__ CUtensorMap w_map, c
             GPTQ_TRACE_MIN(a.trace_slot, first_weight_issue);
         }
         const int NS = xw ? XS : WS;
-        int s = 0, n = 0, sa = 0;
+        int s = 0, n = 0;
         for (int tile = tile0; tile < a.tiles; tile += tile_step) {
             const int mt = tile / panels, p = tile - mt * panels;       // neighbouring CTAs share the x tile
             for (int t = 0; t < G; ++t, ++n) {
                 if (n >= NS) wait_done(n - NS);
                 if (elect_one()) {
                     if (xw) {
-                        // (the A stage's last item has been multiplied: there are at least as many stages as x slots)
-                        mbar_arrive_expect_tx(bar_afull + 8 * sa, x_slot);
-                        tma_load_3d(x_ring + s * x_slot, &x_map, 0, mt * tok, 2 * (g0 + t), bar_afull + 8 * sa);     // rows >= M read as zero
+                        // (item n - 16, the last on this barrier, has been multiplied: there are at most 16 slots)
+                        const uint32_t bar = bar_afull + 8 * (n & (kUmmaDoneRing - 1));
+                        mbar_arrive_expect_tx(bar, x_slot);
+                        tma_load_3d(x_ring + s * x_slot, &x_map, 0, mt * tok, 2 * (g0 + t), bar);     // rows >= M read as zero
                     } else {
                         // packed weights as rows of 64 bytes, 128 to an item
                         mbar_arrive_expect_tx(bar_wfull + 8 * s, kWSlot);
@@ -195,7 +201,6 @@ prefill_kernel(const PrefillArgs a, const __grid_constant__ CUtensorMap w_map, c
                 }
                 __syncwarp();
                 if (++s == NS) s = 0;
-                if (++sa == PS) sa = 0;
             }
         }
     } else if (warp == 1) {
@@ -205,13 +210,13 @@ prefill_kernel(const PrefillArgs a, const __grid_constant__ CUtensorMap w_map, c
             const uint64_t desc0 = umma_desc_k_major_sw128(x_ring);
             const uint32_t desc_lo = (uint32_t)desc0, desc_hi = (uint32_t)(desc0 >> 32);      // (the address field is in the low word)
             const uint32_t x_step = x_slot >> 4, half_step = x_half >> 4, x_end = XS * x_step, a0 = tmem_base + 2 * acc;
-            uint32_t xo = 0, n = 0, sa = 0, ph = 0;
+            uint32_t xo = 0, n = 0, sa = 0;
             for (int tile = tile0, it = 0; tile < a.tiles; tile += tile_step, ++it) {
                 const uint32_t d = it & 1, d_tmem = tmem_base + d * acc;
                 decode_wait(bar_dempty + 8 * d, ((uint32_t)(it >> 1) & 1u) ^ 1u, flag);
                 uint32_t accumulate = 0;
                 for (int t = G; t > 0; --t, ++n) {
-                    decode_wait(bar_afull + 8 * sa, ph, flag);
+                    decode_wait(bar_afull + 8 * (n & (kUmmaDoneRing - 1)), n / kUmmaDoneRing & 1u, flag);
                     tc_fence_after_sync();
                     if (n == 0) GPTQ_TRACE_MIN(a.trace_slot, first_data);
                     const uint32_t a_tmem = a0 + sa * 64;
@@ -224,10 +229,7 @@ prefill_kernel(const PrefillArgs a, const __grid_constant__ CUtensorMap w_map, c
                     umma_commit(bar_done + 8 * (n & (kUmmaDoneRing - 1)));
                     xo += x_step;
                     if (xo == x_end) xo = 0;
-                    if (++sa == (uint32_t)PS) {
-                        sa = 0;
-                        ph ^= 1u;
-                    }
+                    if (++sa == (uint32_t)PS) sa = 0;
                 }
                 umma_commit(bar_dfull + 8 * d);
             }
@@ -345,7 +347,7 @@ prefill_kernel(const PrefillArgs a, const __grid_constant__ CUtensorMap w_map, c
             tmem_wait_st();
             tc_fence_before_sync();
             __syncwarp();
-            if (lane == 0) mbar_arrive(bar_afull + 8 * sa);
+            if (lane == 0) mbar_arrive(bar_afull + 8 * (n & (kUmmaDoneRing - 1)));       // (item n - 16 has been multiplied: n - PS has)
             n += kPrefillSets;
             sa += kPrefillSets;
             while (sa >= PS) sa -= PS;
@@ -638,7 +640,7 @@ inline PrefillPlan plan_prefill(int M, int N, int K, int group_size, int sm_coun
     pl.ctas = pl.S > 1 ? pl.tiles * pl.S : pl.tiles < sm_count ? pl.tiles : sm_count;
     const int fixed = 2048 + kPrefillStage + prefill_w_slots(pl.tok, w8) * (w8 ? 2 : 1) * kItemWBytes, x_slot = pl.tok * 256;
     pl.x_slots = (227 * 1024 - fixed) / x_slot;
-    if (pl.x_slots > prefill_a_stages(pl.tok)) pl.x_slots = prefill_a_stages(pl.tok);
+    if (pl.x_slots > kPrefillXSlots) pl.x_slots = kPrefillXSlots;
     pl.smem_bytes = fixed + pl.x_slots * x_slot;
     const int floor_one_per_sm = (227 * 1024) / 2 + 512;                 // the CTA owns all tensor memory
     if (pl.smem_bytes < floor_one_per_sm) pl.smem_bytes = floor_one_per_sm;

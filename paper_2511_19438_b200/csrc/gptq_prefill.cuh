@@ -80,6 +80,22 @@ __device__ __forceinline__ void bulk_s2s_cluster(uint32_t dst, uint32_t src, uin
                  "r"(bytes), "r"(bar)
                  : "memory");
 }
+// 16 bytes into the shared memory of a CTA of the cluster, counted on that CTA's mbarrier
+__device__ __forceinline__ void st_async_b32x4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d, uint32_t bar)
+{
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
+                 ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d), "r"(bar)
+                 : "memory");
+}
+__device__ __forceinline__ void tmem_ld_32x16(uint32_t taddr, uint32_t (&r)[16])
+{
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr)
+        : "memory");
+}
 template <bool BF>
 __device__ __forceinline__ uint32_t pack_out16(float2 v)
 {
@@ -91,6 +107,10 @@ __device__ __forceinline__ uint32_t pack_out16(float2 v)
         return *reinterpret_cast<const uint32_t *>(&h);
     }
 }
+
+// Tiles of at most this many token rows exchange their parts by stores into the owners' shared memory, taller ones by bulk copies
+// (8-bit weights: see prefill_kernel).
+__host__ __device__ constexpr int prefill_push_rows(bool w8) { return w8 ? 64 : 112; }
 
 struct PrefillArgs {
     const uint8_t *scales, *qzeros;   // tiled
@@ -105,7 +125,9 @@ struct PrefillArgs {
     const int32_t *out_index;
 };
 
-template <int SUB, bool BF, bool W8, bool SPLIT>
+// SPLIT: K shared by a cluster, the partial tiles parked and copied, or stored into the owners' shared memory
+constexpr int kParkParts = 1, kPushParts = 2;
+template <int SUB, bool BF, bool W8, int SPLIT>
 __global__ void __launch_bounds__(kPrefillThreads, 1)
 prefill_kernel(const PrefillArgs a, const __grid_constant__ CUtensorMap w_map, const __grid_constant__ CUtensorMap x_map)
 {
@@ -124,7 +146,7 @@ prefill_kernel(const PrefillArgs a, const __grid_constant__ CUtensorMap w_map, c
     // its x has landed; done[n mod 16]: the MMAs of the CTA's n-th item have completed; dfull / dempty: accumulators
     const uint32_t bar_wfull = base, bar_afull = base + 384, bar_done = base + 192, bar_dfull = base + 320,
                    bar_dempty = base + 336;
-    const uint32_t tmem_slot = base + 352, flag = base + 356, bar_recv = base + 360;
+    const uint32_t tmem_slot = base + 352, flag = base + 356, bar_recv = base + 360, bar_ready = base + 368;
     const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const int S = SPLIT ? a.S : 1, rank = SPLIT ? (int)blockIdx.x % S : 0, tile0 = SPLIT ? (int)blockIdx.x / S : (int)blockIdx.x;
     const int tile_step = SPLIT ? (int)gridDim.x / S : (int)gridDim.x;
@@ -147,10 +169,11 @@ prefill_kernel(const PrefillArgs a, const __grid_constant__ CUtensorMap w_map, c
         }
         asm volatile("st.shared.u32 [%0], %1;" ::"r"(flag), "r"(0u) : "memory");
         if (SPLIT) mbar_init(bar_recv, 1);
+        if (SPLIT == kPushParts) mbar_init(bar_ready, 4 * kPrefillSets * S);
         fence_barrier_init();
         if (SPLIT) {
             const int m0 = tile0 / panels * tok, rows = (a.M - m0) < tok ? (a.M - m0) : tok;
-            mbar_arrive_expect_tx(bar_recv, (uint32_t)((S - 1) * rows * (kPanel / S) * 4));
+            mbar_arrive_expect_tx(bar_recv, (uint32_t)((S - 1) * (kPanel / S) * (SPLIT == kPushParts ? (rows + 3) & ~3 : rows) * 4));
         }
         fence_proxy_async();
     }
@@ -162,6 +185,7 @@ prefill_kernel(const PrefillArgs a, const __grid_constant__ CUtensorMap w_map, c
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, lds32(tmem_slot), 0);
+    if (SPLIT == kPushParts) cluster_arrive_release();        // "my barriers are set up"
     pdl_launch_dependents();
 
     const bool is_dq = warp >= kPrefillFirstDq && warp < kPrefillWWarp, is_epi = warp >= kPrefillFirstEpi && warp < kPrefillFirstDq;
@@ -360,79 +384,145 @@ prefill_kernel(const PrefillArgs a, const __grid_constant__ CUtensorMap w_map, c
     }
     if constexpr (SPLIT) {
         // ---------------------------------------------------------------- the cluster's partial tiles
-        // After its main loop a CTA's rings are idle: it parks its partial sums there as [owner][token][own column] floats (a
-        // CTA owns 128 / S neighbouring columns).  Once every CTA has, bulk copies through distributed shared memory bring
-        // each owner its part, [sender][token][own column] behind the parked tile, and the owner adds in rank order.
-        // (st.async of single floats took about 55 clocks per token row: o M = 128 11.6 us.)
+        // A CTA owns 128 / S neighbouring columns; the owner adds the CTAs' parts in rank order.
         const bool layout_ok = ((flags & kFormatGateUp) != 0) == (a.fuse != 0) && ((flags & kFormatBf16) != 0) == BF;
         if (!layout_ok && threadIdx.x == 32 * kPrefillFirstEpi) atomicMax(&g_device_status, (int)kStatusLayoutMismatch);
         const int group = is_epi ? 0 : 1 + ((warp - kPrefillFirstDq) >> 2), n_groups = 1 + kPrefillSets;
         const int mt = tile0 / panels, p = tile0 - mt * panels, m0 = mt * tok, W = kPanel / S;
         const int rows = (a.M - m0) < tok ? (a.M - m0) : tok;
-        const uint32_t part = (uint32_t)(rows * W * 4), park = w_ring, recv = park + (uint32_t)((rows + 31) & ~31) * (kPanel * 4);
-        if (is_dq || is_epi) {
-            const int q = warp & 3, n = 32 * q + lane, owner = n / W, lc = n - owner * W;
-            pdl_wait();
-            decode_wait(bar_dfull, 0, flag);
+        if constexpr (SPLIT == kPushParts) {
             __syncwarp();
-            tc_fence_after_sync();
-            const uint32_t at = park + owner * part + (uint32_t)lc * 4u;
+            cluster_wait_acquire();
+            // Once the dequant warps of all CTAs have read their last weights, the owners' stages and weight rings take the other
+            // CTAs' parts, [sender][own column][token] floats, straight from the registers of the threads that read the accumulator;
+            // the own part waits in the idle x ring.  A CTA that has all parts needs the others no more.  What bounds it is
+            // latency and, for tall tiles, the 16-byte stores.  K = 4096 on 32 panels, bulk copies and two barriers of the cluster
+            // -> this, us: 17 rows 8.4 -> 7.6, 64 rows 9.5 -> 8.8, 100 rows 10.4 -> 10.1, 112 rows 10.6 -> 10.5, 128 rows
+            // 11.1 -> 11.1, 160 rows 12.3 -> 12.5; K = 11008, 64 rows 13.9 -> 13.1; 64 panels, 50 rows 11.3 -> 10.2; 8-bit weights
+            // 17 rows 9.7 -> 9.4, 64 rows 12.3 -> 12.3, 100 rows 13.3 -> 13.6.
+            if (is_dq && lane < S) mbar_arrive_release_cluster(map_to_cluster_rank(bar_ready, (uint32_t)lane));
+            if (is_dq || is_epi) {
+                const int quads = (rows + 3) >> 2, w_shift = S == 4 ? 5 : 6;
+                const uint32_t pitch = (uint32_t)(tok + 4) * 4, part = W * pitch;         // of a column (an odd number of 16-byte pieces), of a sender
+                pdl_wait();
+                decode_wait(bar_dfull, 0, flag);
+                decode_wait_cluster(bar_ready, 0, flag);
+                __syncwarp();
+                tc_fence_after_sync();
+                const bool ok = layout_ok && lds32(flag) == 0;
+                {
+                    const int q = warp & 3, n = 32 * q + lane, owner = n >> w_shift, lc = n & (W - 1);
+                    const uint32_t dst = map_to_cluster_rank(stg0 + (rank < owner ? rank : rank - 1) * part + lc * pitch, (uint32_t)owner);
+                    const uint32_t dbar = map_to_cluster_rank(bar_recv, (uint32_t)owner), own = x_ring + lc * pitch;
 #pragma unroll 1
-            for (int c0 = 32 * group; c0 < rows; c0 += 32 * n_groups) {
-                uint32_t r[32];
-                tmem_ld_32x32(tmem_base + ((uint32_t)(32 * q) << 16) + c0, r);
-                tmem_wait_ld();
+                    for (int c0 = 16 * group; c0 < rows; c0 += 16 * n_groups) {
+                        uint32_t r[16];
+                        tmem_ld_32x16(tmem_base + ((uint32_t)(32 * q) << 16) + c0, r);
+                        tmem_wait_ld();
 #pragma unroll
-                for (int i = 0; i < 32; ++i)
-                    if (c0 + i < rows) sts_f32(at + (uint32_t)((c0 + i) * W) * 4u, __uint_as_float(r[i]));
-            }
-            fence_proxy_async();
-        }
-        __syncwarp();
-        cluster_arrive_release();
-        cluster_wait_acquire();
-        const bool ok = layout_ok && lds32(flag) == 0;
-        if (warp == kPrefillXWarp && ok && elect_one()) {
-            for (int k = 1; k < S; ++k) {
-                const int to = rank + k < S ? rank + k : rank + k - S;
-                const int slot = rank < to ? rank : rank - 1;              // (nobody sends to itself)
-                bulk_s2s_cluster(map_to_cluster_rank(recv + slot * part, (uint32_t)to), park + to * part, part,
-                                 map_to_cluster_rank(bar_recv, (uint32_t)to));
-            }
-        }
-        __syncwarp();
-        if ((is_dq || is_epi) && ok) {
-            decode_wait_cluster(bar_recv, 0, flag);
-            if (lds32(flag) == 0) {
-                const int w4 = W >> 2;
-                for (int idx = threadIdx.x - 32 * kPrefillFirstEpi; idx < rows * w4; idx += 128 * n_groups) {
-                    const int m = idx / w4, c = 4 * (idx - m * w4);
-                    const size_t col = (size_t)p * kPanel + rank * W + c, at = (size_t)(m0 + m) * a.N + col;
-                    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                    for (int k = 0; k < S; ++k) {
-                        const uint32_t from = k == rank ? park + rank * part : recv + (k < rank ? k : k - 1) * part;
-                        const uint4 u = lds128(from + (uint32_t)(m * W + c) * 4u);
-                        v.x += __uint_as_float(u.x);
-                        v.y += __uint_as_float(u.y);
-                        v.z += __uint_as_float(u.z);
-                        v.w += __uint_as_float(u.w);
+                        for (int k = 0; k < 4; ++k) {
+                            if (c0 + 4 * k >= rows || !ok) break;
+                            if (owner == rank) sts128(own + (c0 + 4 * k) * 4, make_uint4(r[4 * k], r[4 * k + 1], r[4 * k + 2], r[4 * k + 3]));
+                            else st_async_b32x4(dst + (c0 + 4 * k) * 4, r[4 * k], r[4 * k + 1], r[4 * k + 2], r[4 * k + 3], dbar);
+                        }
+                        __syncwarp();
                     }
-                    auto add4 = [&](const __half *from) {
-                        const uint2 b = *reinterpret_cast<const uint2 *>(from);
-                        const float2 b0 = __half22float2(*reinterpret_cast<const __half2 *>(&b.x));
-                        const float2 b1 = __half22float2(*reinterpret_cast<const __half2 *>(&b.y));
-                        v.x += b0.x, v.y += b0.y, v.z += b1.x, v.w += b1.y;
-                    };
-                    if (a.bias) add4(a.bias + col);
-                    if (a.residual) add4(a.residual + at);
-                    *reinterpret_cast<uint2 *>(a.y + at) = make_uint2(pack_out16<BF>(make_float2(v.x, v.y)), pack_out16<BF>(make_float2(v.z, v.w)));
+                }
+                named_bar_sync(1, 128 * n_groups);                      // the own part is there
+                if (ok) decode_wait_cluster(bar_recv, 0, flag);
+                if (ok && lds32(flag) == 0) {
+                    // a thread takes a column of four rows
+                    for (int idx = threadIdx.x - 32 * kPrefillFirstEpi; idx < quads * W; idx += 128 * n_groups) {
+                        const int c = idx & (W - 1), m = 4 * (idx >> w_shift);
+                        const size_t col = (size_t)p * kPanel + rank * W + c, at = (size_t)(m0 + m) * a.N + col;
+                        float v[4] = {};
+                        for (int k = 0; k < S; ++k) {
+                            const uint4 u = lds128((k == rank ? x_ring : stg0 + (k < rank ? k : k - 1) * part) + c * pitch + m * 4);
+                            v[0] += __uint_as_float(u.x);
+                            v[1] += __uint_as_float(u.y);
+                            v[2] += __uint_as_float(u.z);
+                            v[3] += __uint_as_float(u.w);
+                        }
+                        const float bias = a.bias ? __half2float(a.bias[col]) : 0.f;
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            if (m + e >= rows) break;
+                            float f = v[e] + bias;
+                            if (a.residual) f += __half2float(a.residual[at + (size_t)e * a.N]);
+                            store_out16<BF>(a.y + at + (size_t)e * a.N, f);
+                        }
+                    }
                 }
             }
+        } else {
+            // After its main loop a CTA's rings are idle: it parks its partial sums there as [owner][token][own column] floats.  Once
+            // every CTA has, bulk copies through distributed shared memory bring each owner its part, [sender][token][own column]
+            // behind the parked tile.
+            const uint32_t part = (uint32_t)(rows * W * 4), park = w_ring, recv = park + (uint32_t)((rows + 31) & ~31) * (kPanel * 4);
+            if (is_dq || is_epi) {
+                const int q = warp & 3, n = 32 * q + lane, owner = n / W, lc = n - owner * W;
+                pdl_wait();
+                decode_wait(bar_dfull, 0, flag);
+                __syncwarp();
+                tc_fence_after_sync();
+                const uint32_t at = park + owner * part + (uint32_t)lc * 4u;
+    #pragma unroll 1
+                for (int c0 = 32 * group; c0 < rows; c0 += 32 * n_groups) {
+                    uint32_t r[32];
+                    tmem_ld_32x32(tmem_base + ((uint32_t)(32 * q) << 16) + c0, r);
+                    tmem_wait_ld();
+    #pragma unroll
+                    for (int i = 0; i < 32; ++i)
+                        if (c0 + i < rows) sts_f32(at + (uint32_t)((c0 + i) * W) * 4u, __uint_as_float(r[i]));
+                }
+                fence_proxy_async();
+            }
+            __syncwarp();
+            cluster_arrive_release();
+            cluster_wait_acquire();
+            const bool ok = layout_ok && lds32(flag) == 0;
+            if (warp == kPrefillXWarp && ok && elect_one()) {
+                for (int k = 1; k < S; ++k) {
+                    const int to = rank + k < S ? rank + k : rank + k - S;
+                    const int slot = rank < to ? rank : rank - 1;              // (nobody sends to itself)
+                    bulk_s2s_cluster(map_to_cluster_rank(recv + slot * part, (uint32_t)to), park + to * part, part,
+                                     map_to_cluster_rank(bar_recv, (uint32_t)to));
+                }
+            }
+            __syncwarp();
+            if ((is_dq || is_epi) && ok) {
+                decode_wait_cluster(bar_recv, 0, flag);
+                if (lds32(flag) == 0) {
+                    const int w4 = W >> 2;
+                    for (int idx = threadIdx.x - 32 * kPrefillFirstEpi; idx < rows * w4; idx += 128 * n_groups) {
+                        const int m = idx / w4, c = 4 * (idx - m * w4);
+                        const size_t col = (size_t)p * kPanel + rank * W + c, at = (size_t)(m0 + m) * a.N + col;
+                        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+                        for (int k = 0; k < S; ++k) {
+                            const uint32_t from = k == rank ? park + rank * part : recv + (k < rank ? k : k - 1) * part;
+                            const uint4 u = lds128(from + (uint32_t)(m * W + c) * 4u);
+                            v.x += __uint_as_float(u.x);
+                            v.y += __uint_as_float(u.y);
+                            v.z += __uint_as_float(u.z);
+                            v.w += __uint_as_float(u.w);
+                        }
+                        auto add4 = [&](const __half *from) {
+                            const uint2 b = *reinterpret_cast<const uint2 *>(from);
+                            const float2 b0 = __half22float2(*reinterpret_cast<const __half2 *>(&b.x));
+                            const float2 b1 = __half22float2(*reinterpret_cast<const __half2 *>(&b.y));
+                            v.x += b0.x, v.y += b0.y, v.z += b1.x, v.w += b1.y;
+                        };
+                        if (a.bias) add4(a.bias + col);
+                        if (a.residual) add4(a.residual + at);
+                        *reinterpret_cast<uint2 *>(a.y + at) = make_uint2(pack_out16<BF>(make_float2(v.x, v.y)), pack_out16<BF>(make_float2(v.z, v.w)));
+                    }
+                }
+            }
+            // no CTA may leave while its parked sums are being read; what it sent has landed once all have received
+            __syncwarp();
+            cluster_arrive_release();
+            cluster_wait_acquire();
         }
-        // no CTA may leave while its parked sums are being read; what it sent has landed once all have received
-        __syncwarp();
-        cluster_arrive_release();
-        cluster_wait_acquire();
     } else if (is_dq || is_epi) {
         // ---------------------------------------------------------------- epilogue
         // A warp reads its 32 lanes (columns of y) x 32 tokens as 8 x 8 fragments, rounds them and transposes them with
@@ -575,6 +665,10 @@ prefill_kernel(const PrefillArgs a, const __grid_constant__ CUtensorMap w_map, c
         const uint64_t start = global_timer_ns();
         while (global_timer_ns() - start < 200000ull) { }
         __syncthreads();
+        if (SPLIT == kPushParts) {        // ... and stay until the other CTAs of the cluster have left or come here too: they may still send
+            cluster_arrive_release();
+            cluster_wait_acquire();
+        }
     }
     if (warp == 1) {
         tc_fence_after_sync();
@@ -647,7 +741,7 @@ inline PrefillPlan plan_prefill(int M, int N, int K, int group_size, int sm_coun
     return pl;
 }
 
-template <int SUB, bool BF, bool W8, bool SPLIT>
+template <int SUB, bool BF, bool W8, int SPLIT>
 static int launch_prefill_split(const PrefillArgs &args, const CUtensorMap &w_map, const CUtensorMap &x_map, const PrefillPlan &plan,
                               cudaStream_t s)
 {
@@ -675,9 +769,11 @@ template <int SUB, bool BF, bool W8>
 static int launch_prefill_sub(const PrefillArgs &args, const CUtensorMap &w_map, const CUtensorMap &x_map, const PrefillPlan &plan,
                               cudaStream_t s)
 {
-    // (a template: with the number of CTAs per tile known only at run time, launches without a split were 7 % slower)
-    return plan.S > 1 ? launch_prefill_split<SUB, BF, W8, true>(args, w_map, x_map, plan, s)
-                      : launch_prefill_split<SUB, BF, W8, false>(args, w_map, x_map, plan, s);
+    // (a template: with the number of CTAs per tile known only at run time, launches without a split were 7 % slower; with both
+    // kinds of exchange in one kernel registers spilled)
+    if (plan.S == 1) return launch_prefill_split<SUB, BF, W8, 0>(args, w_map, x_map, plan, s);
+    return plan.tok <= prefill_push_rows(W8) ? launch_prefill_split<SUB, BF, W8, kPushParts>(args, w_map, x_map, plan, s)
+                                             : launch_prefill_split<SUB, BF, W8, kParkParts>(args, w_map, x_map, plan, s);
 }
 
 int launch_prefill(const __half *x, const void *qweight, const void *qzeros, const void *scales, __half *y, int M, int N, int K,

@@ -245,6 +245,10 @@ splitk_kernel(const SplitKArgs a, const __grid_constant__ CUtensorMap x_map)
         for (int it = 0; it < n_items; ++it) {
             const uint32_t st = ring + s * kStage;
             if (ok) ok = mbar_wait(bar_full + 8 * s, phase);   // on failure: stale data, status word set
+            // The barrier keeps the loads of x behind the wait: without it one launch in a hundred multiplied old rows of x where the
+            // waits are long (activations from host buffers, 3 to 8 rows, 4096 x 22016).  A vote over the wait, after which the
+            // lanes go on together as well, did not help.  It costs 2 to 3 % (8 rows 14.2 -> 14.5 us).
+            __syncwarp();
             if (it == 0 && threadIdx.x == 0) GPTQ_TRACE_MIN(a.trace_slot, first_data);
 
             ItemSums<MT, SUB> sums;

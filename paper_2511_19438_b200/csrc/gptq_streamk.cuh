@@ -250,6 +250,7 @@ streamk_kernel(const StreamKArgs a, const __grid_constant__ CUtensorMap x_map)
     for (int t = t0; t < t1; ++t) {
         const uint32_t st = ring + s * kStage;
         if (ok) ok = mbar_wait(bar_full + 8 * s, phase);   // on failure: stale data, status word set
+        __syncwarp();           // keeps the loads of x behind the wait (see splitk_kernel)
 
         ItemSums<MT, 1> sums;
         consume_item<MT, 1>(st, w_off, s_off, z_off, x_off0, x_off1, z_add, sums);

@@ -1659,3 +1659,33 @@ def test_host_batch_results_for_one_host_buffer(ws):
         assert B.gptq_gemm_host_batch(B.make_host_problems(items))[0] == B.GPTQ_OK
         torch.cuda.synchronize()
         assert torch.equal(big, expect), rnd
+
+
+@pytest.mark.parametrize("M", [3, 4, 8])
+def test_host_batch_repeats_bit_for_bit(M):
+    """A decode step from host buffers, a hundred times over: every result has the bits of the same call on device buffers.
+    (The kernels wait longest here, for activations that have just come up and weights that are not in the L2 cache.)"""
+    gen = torch.Generator(device="cuda").manual_seed(77 + M)
+
+    def words(*shape):
+        return torch.randint(-(1 << 31), 1 << 31, shape, generator=gen, device="cuda", dtype=torch.int64).to(torch.int32)
+
+    ops, items = [], []
+    for _ in range(8):
+        for K, N in wl.SHAPES_7B.values():
+            outs = [torch.empty(B.gptq_repack_bytes(w, N, K, 128, 0), dtype=torch.uint8, device="cuda") for w in range(3)]
+            sc = torch.rand((K // 128, N), generator=gen, device="cuda").mul_(0.02).half()
+            B.check(B.gptq_repack(words(K // 8, N), words(K // 128, N // 8), sc, None, *outs, None, N, K, 128, 0), "gptq_repack")
+            x, y = torch.randn((M, K), generator=gen, device="cuda").half(), torch.empty((M, N), dtype=torch.float16, device="cuda")
+            B.check(B.gptq_gemm(x, *outs, None, y, M, N, K, 128, 0), "gptq_gemm")
+            xh, yh = x.cpu().pin_memory(), torch.empty((M, N), dtype=torch.float16).pin_memory()
+            ops.append((outs, x, y, xh, yh, y.cpu()))
+            items.append((xh, *outs, None, yh, x, y, M, N, K, 128, False))
+    problems = B.make_host_problems(items)
+    torch.cuda.synchronize()
+    for it in range(100):
+        B.check(B.gptq_gemm_host_batch(problems)[0], "gptq_gemm_host_batch")
+        torch.cuda.synchronize()
+        for i, op in enumerate(ops):
+            assert torch.equal(op[4].view(torch.int16), op[5].view(torch.int16)), (it, i)
+    B.check(B.gptq_check_status(), "status")

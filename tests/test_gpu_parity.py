@@ -1573,6 +1573,20 @@ def test_prefill_kernel(K, N, gs, act, zm1, M, ws):
     assert B.gptq_check_status() == B.GPTQ_OK
 
 
+@pytest.mark.parametrize("K,N", [(2048, 1024), (4096, 5120)])      # clusters of four, of two
+@pytest.mark.parametrize("M", [18, 63, 112, 113])                  # rows no multiple of four; the tallest tile that stores its parts; two tiles, or a taller one
+def test_prefill_kernel_exchanges_parts(K, N, M, ws):
+    """A tile's K range shared by a cluster: both ways of exchanging the partial sums, with the plain and bias + residual epilogues."""
+    st, pl = B.gptq_plan_prefill(M, N, K, 128, 0, 0, 148)
+    assert st == B.GPTQ_OK and pl.cluster_size > 1, "the planner no longer splits this shape: choose another"
+    L = wl.make_linear(K, N, seed=wl.seed_for("prefill-parts", K, N))
+    x_np = wl.make_x(M, K, wl.seed_for("prefill-parts-x", M, K))
+    y, _ = run_gemm(L, x_np, ws)
+    assert_close(y, oracle.gemm_f64(x_np, L.qweight, L.qzeros, L.scales, None, 128), K, M)
+    check_bias_residual(L, M, ws, True, True)
+    assert B.gptq_check_status() == B.GPTQ_OK
+
+
 @pytest.mark.parametrize("M", [17, 31, 64, 130, 300])
 def test_prefill_kernel_silu_mul_keeps_fp32_factors(M, ws):
     """With power-of-two scales the weights are exact in fp16, so gate and up are fp32 sums (2e-6 of the sum of magnitudes

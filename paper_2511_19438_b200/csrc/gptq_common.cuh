@@ -218,11 +218,29 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity)
         if (mbar_try_wait(bar, parity)) return true;
     return mbar_wait_slow(bar, parity);
 }
+// For a converged warp that stays one: the lanes leave the wait together, as mma.sync behind it wants them.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity)
+{
+    for (int it = 0; it < 64; ++it)
+        if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    return __all_sync(0xffffffffu, mbar_wait_slow(bar, parity));
+}
 // One inlined try, the rest behind a call: 53 clocks instead of 78 for a barrier that is ready, and less code in the loops
 // that wait.  (In the 256-token tcgen05 kernel the polling form measured 2 % faster, at 64 tokens this one 3 %.)
 __device__ __forceinline__ bool mbar_wait_once(uint32_t bar, uint32_t parity)
 {
     return mbar_try_wait(bar, parity) || mbar_wait_slow(bar, parity);
+}
+// For the thread that refills a ring: the stage has been handed back by warps that read it with ordinary loads, and the next copy
+// into it goes through the async proxy.  The arrivals alone do not keep that copy behind those loads; the fence on the way from
+// them to the copy does.  Without it the last load of x of an item now and then found what the refill had brought (host batches of
+// 3 to 8 rows, 4096 x 22016: in 0.1 to 0.7 % of the launches the last 32 rows of K of an item were multiplied with the x of the
+// item four on).  In the refilling thread it costs nothing that can be measured, in the reading warps up to 2 % (decode kernel).
+__device__ __forceinline__ bool mbar_wait_stage_free(uint32_t bar, uint32_t parity)
+{
+    const bool ok = mbar_wait(bar, parity);
+    fence_proxy_async();
+    return ok;
 }
 // 1-D bulk copy global -> shared with an L2 cache-policy hint, completion counted in bytes on an
 // mbarrier.  dst, src and bytes must be multiples of 16.  Issue it from a dedicated producer thread:

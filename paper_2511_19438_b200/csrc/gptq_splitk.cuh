@@ -117,7 +117,7 @@ struct SplitKPlan {
     int smem_bytes;
 };
 
-// The 8-row, group-128 instantiation compiles to 56 registers, which plan_splitk counts on for four resident CTAs; the
+// The 8-row, group-128 instantiation compiles to 53 registers (plan_splitk counts on at most 56 for four resident CTAs); the
 // timeline build's extra code would push it over, so there the bound is stated (a stated bound of 4 in the normal build
 // made the compiler choose 52 registers and a 1-2 % slower schedule).
 #ifdef GPTQ_TIMELINE
@@ -211,7 +211,7 @@ splitk_kernel(const SplitKArgs a, const __grid_constant__ CUtensorMap x_map)
             for (int it = 0; it < n_items; ++it) {
                 const uint32_t bar = bar_full + 8 * s;
                 if (it >= stages) {
-                    if (!mbar_wait(bar_empty + 8 * s, (uint32_t)((round - 1) & 1))) break;
+                    if (!mbar_wait_stage_free(bar_empty + 8 * s, (uint32_t)((round - 1) & 1))) break;
                     issue_weights(t0 + it, s);
                 }
                 // the group's activations for all token rows: two swizzled K64 tiles, rows >= M read as zero
@@ -244,11 +244,7 @@ splitk_kernel(const SplitKArgs a, const __grid_constant__ CUtensorMap x_map)
         bool ok = true;   // false after a wait gave up: keep taking part in barriers, skip the data
         for (int it = 0; it < n_items; ++it) {
             const uint32_t st = ring + s * kStage;
-            if (ok) ok = mbar_wait(bar_full + 8 * s, phase);   // on failure: stale data, status word set
-            // The barrier keeps the loads of x behind the wait: without it one launch in a hundred multiplied old rows of x where the
-            // waits are long (activations from host buffers, 3 to 8 rows, 4096 x 22016).  A vote over the wait, after which the
-            // lanes go on together as well, did not help.  It costs 2 to 3 % (8 rows 14.2 -> 14.5 us).
-            __syncwarp();
+            if (ok) ok = mbar_wait_warp(bar_full + 8 * s, phase);   // on failure: stale data, status word set
             if (it == 0 && threadIdx.x == 0) GPTQ_TRACE_MIN(a.trace_slot, first_data);
 
             ItemSums<MT, SUB> sums;
@@ -393,7 +389,7 @@ SplitKPlan plan_splitk(int m_rows, int N, int K, int group_size, int sm_count)
     const int G = K / kGroup, panels = N / kPanel;
     pl.sub = kGroup / group_size;
     const int stage = streamk_stage_bytes(MT, pl.sub);
-    // The 8-row, group-128 instantiation needs 56 registers, so four of its CTAs fit an SM, and for it cluster sizes 3
+    // The 8-row, group-128 instantiation needs at most 56 registers, so four of its CTAs fit an SM, and for it cluster sizes 3
     // and 6 are candidates too (5 and 7 measured badly: clusters of that size often find no room): the 7B gate_up
     // (172 panels) takes 13.8 us with 3 x 172 CTAs against 14.9 with 2 x 172, the 13B qkv 12.6 us with S = 4 against 13.9
     // with S = 2.  The other instantiations keep powers of two and three CTAs per SM.

@@ -206,7 +206,7 @@ streamk_kernel(const StreamKArgs a, const __grid_constant__ CUtensorMap x_map)
         for (int it = 0; it < n_items; ++it) {
             const uint32_t bar = bar_full + 8 * s;
             if (it >= stages) {
-                if (!mbar_wait(bar_empty + 8 * s, (uint32_t)((round - 1) & 1))) break;
+                if (!mbar_wait_stage_free(bar_empty + 8 * s, (uint32_t)((round - 1) & 1))) break;
                 issue_weights(t0 + it, s);
             }
             // the group's activations for all token rows: two swizzled K64 tiles, rows >= M read as zero
@@ -249,8 +249,7 @@ streamk_kernel(const StreamKArgs a, const __grid_constant__ CUtensorMap x_map)
     bool ok = true;   // false after a wait gave up: keep taking part in barriers, skip the data
     for (int t = t0; t < t1; ++t) {
         const uint32_t st = ring + s * kStage;
-        if (ok) ok = mbar_wait(bar_full + 8 * s, phase);   // on failure: stale data, status word set
-        __syncwarp();           // keeps the loads of x behind the wait (see splitk_kernel)
+        if (ok) ok = mbar_wait_warp(bar_full + 8 * s, phase);   // on failure: stale data, status word set
 
         ItemSums<MT, 1> sums;
         consume_item<MT, 1>(st, w_off, s_off, z_off, x_off0, x_off1, z_add, sums);

@@ -1675,31 +1675,85 @@ def test_host_batch_results_for_one_host_buffer(ws):
         assert torch.equal(big, expect), rnd
 
 
-@pytest.mark.parametrize("M", [3, 4, 8])
-def test_host_batch_repeats_bit_for_bit(M):
-    """A decode step from host buffers, a hundred times over: every result has the bits of the same call on device buffers.
-    (The kernels wait longest here, for activations that have just come up and weights that are not in the L2 cache.)"""
-    gen = torch.Generator(device="cuda").manual_seed(77 + M)
+def random_layers(kind, gs, layers, seed):
+    """The linears of some 7B decoder layers with random words, repacked on the device: (K, N, outs, perm) each."""
+    gen = torch.Generator(device="cuda").manual_seed(seed)
 
     def words(*shape):
         return torch.randint(-(1 << 31), 1 << 31, shape, generator=gen, device="cuda", dtype=torch.int64).to(torch.int32)
 
-    ops, items = [], []
-    for _ in range(8):
+    made = []
+    for _ in range(layers):
         for K, N in wl.SHAPES_7B.values():
-            outs = [torch.empty(B.gptq_repack_bytes(w, N, K, 128, 0), dtype=torch.uint8, device="cuda") for w in range(3)]
-            sc = torch.rand((K // 128, N), generator=gen, device="cuda").mul_(0.02).half()
-            B.check(B.gptq_repack(words(K // 8, N), words(K // 128, N // 8), sc, None, *outs, None, N, K, 128, 0), "gptq_repack")
-            x, y = torch.randn((M, K), generator=gen, device="cuda").half(), torch.empty((M, N), dtype=torch.float16, device="cuda")
-            B.check(B.gptq_gemm(x, *outs, None, y, M, N, K, 128, 0), "gptq_gemm")
-            xh, yh = x.cpu().pin_memory(), torch.empty((M, N), dtype=torch.float16).pin_memory()
-            ops.append((outs, x, y, xh, yh, y.cpu()))
-            items.append((xh, *outs, None, yh, x, y, M, N, K, 128, False))
+            sc = torch.rand((K // gs, N), generator=gen, device="cuda").mul_(0.02)
+            if kind == "w8":
+                outs = [torch.empty(B.gptq_repack_w8_bytes(w, N, K, gs), dtype=torch.uint8, device="cuda") for w in range(3)]
+                perm, n = torch.empty(2 * K, dtype=torch.int32, device="cuda"), B.gptq_repack_w8_scratch_bytes(N, K, gs)
+                scratch = torch.empty(n, dtype=torch.uint8, device="cuda")
+                B.check(B.gptq_repack_w8(words(K // 4, N), words(K // gs, N // 4), sc.mul_(1 / 16).half(), None, *outs, perm, scratch, n, N, K, gs,
+                                         0, 0), "gptq_repack_w8")
+            else:
+                bf16 = kind == "bf16"
+                outs, perm = [torch.empty(B.gptq_repack_bytes(w, N, K, gs, 0), dtype=torch.uint8, device="cuda") for w in range(3)], None
+                B.check(B.gptq_repack_format(words(K // 8, N), words(K // gs, N // 8), sc.to(torch.bfloat16 if bf16 else torch.float16), None, *outs,
+                                             None, N, K, gs, 0, B.GPTQ_FORMAT_BF16 if bf16 else 0), "gptq_repack_format")
+            made.append((K, N, outs, perm))
+    return made, gen
+
+
+@pytest.mark.parametrize("M,kind,gs,rounds", [
+    (3, "fp16", 128, 400), (4, "fp16", 128, 400), (8, "fp16", 128, 400),
+    (16, "fp16", 128, 100), (12, "fp16", 64, 100), (7, "fp16", 32, 100), (5, "bf16", 128, 100), (13, "bf16", 64, 100), (6, "w8", 128, 100)])
+def test_host_batch_repeats_bit_for_bit(M, kind, gs, rounds, ws):
+    """A decode step from host buffers, again and again: every result has the bits of the same call on device buffers.  Every buffer
+    that the step writes is overwritten before each round.  (Weights that are not in the L2 cache and activations that have just come
+    up: where the kernels' stages are used again at the worst times.)"""
+    made, gen = random_layers(kind, gs, 4 if kind == "w8" else 8, 77 + M)
+    dt = torch.bfloat16 if kind == "bf16" else torch.float16
+    single, batch = {"fp16": (B.gptq_gemm, B.gptq_gemm_host_batch), "bf16": (B.gptq_gemm_bf16, B.gptq_gemm_host_batch_bf16),
+                     "w8": (B.gptq_gemm_w8, B.gptq_gemm_host_batch_w8)}[kind]
+    if kind == "w8":
+        ws.ensure(max(B.gptq_workspace_bytes(M, N, 2 * K, gs, 1) for K, N, _, _ in made))
+    ops, items = [], []
+    for K, N, outs, perm in made:
+        x, y = torch.randn((M, K), generator=gen, device="cuda").to(dt), torch.empty((M, N), dtype=dt, device="cuda")
+        B.check(single(x, *outs, perm, y, M, N, K, gs) if kind == "w8" else single(x, *outs, None, y, M, N, K, gs, 0), "on the device")
+        xh, yh = x.cpu().pin_memory(), torch.empty((M, N), dtype=dt).pin_memory()
+        ops.append((x, y, yh, y.cpu()))
+        items.append((xh, *outs, perm, yh, x, y, M, N, K, gs, False))
     problems = B.make_host_problems(items)
-    torch.cuda.synchronize()
-    for it in range(100):
-        B.check(B.gptq_gemm_host_batch(problems)[0], "gptq_gemm_host_batch")
+    for rnd in range(rounds):
+        for x, y, yh, _ in ops:
+            yh.fill_(7.0)
+            x.zero_()
+            y.fill_(3.0)
+        if rnd & 1:
+            torch.cuda.synchronize()
+        B.check(batch(problems)[0], "host batch")
         torch.cuda.synchronize()
-        for i, op in enumerate(ops):
-            assert torch.equal(op[4].view(torch.int16), op[5].view(torch.int16)), (it, i)
+        for i, (_, _, yh, want) in enumerate(ops):
+            assert torch.equal(yh.view(torch.int16), want.view(torch.int16)), (rnd, i)
+    B.check(B.gptq_check_status(), "status")
+
+
+@pytest.mark.parametrize("M", [3, 8, 16])
+def test_noalloc_repeats_bit_for_bit(M):
+    """gptq_gemm_noalloc, whose kernel has such a ring too, again and again: activations come up in front of each call."""
+    made, gen = random_layers("fp16", 128, 4, 99 + M)
+    ops = []
+    for K, N, outs, _ in made:
+        x, y = torch.randn((M, K), generator=gen, device="cuda").half(), torch.empty((M, N), dtype=torch.float16, device="cuda")
+        B.check(B.gptq_gemm_noalloc(x, *outs, None, y, M, N, K, 128, 0), "gptq_gemm_noalloc")
+        ops.append((outs, x, x.cpu().pin_memory(), y, y.clone(), K, N))
+    for rnd in range(200):
+        for _, x, _, y, _, _, _ in ops:
+            x.zero_()
+            y.fill_(3.0)
+        if rnd & 1:
+            torch.cuda.synchronize()
+        for outs, x, xh, y, _, K, N in ops:
+            x.copy_(xh, non_blocking=True)
+            B.check(B.gptq_gemm_noalloc(x, *outs, None, y, M, N, K, 128, 0), "gptq_gemm_noalloc")
+        for i, (_, _, _, y, want, _, _) in enumerate(ops):
+            assert torch.equal(y.view(torch.int16), want.view(torch.int16)), (rnd, i)
     B.check(B.gptq_check_status(), "status")

@@ -420,6 +420,7 @@ decode_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ CUte
                 for (int i = 0; i < nc; i += P) {
                     if (left-- == kDecodeLead) pdl_launch_dependents();
                     decode_wait(bar_wempty + 8 * s, eph, flag);
+                    fence_proxy_async();        // the copies stay behind the dequant warps' loads, as in mbar_wait_stage_free
                     if (elect_one()) {
                         const bool two = P == 2 && i + 1 < nc;
                         mbar_arrive_expect_tx(bar_wfull + 8 * s, two ? 2 * kItemWBytes : kItemWBytes);
@@ -595,6 +596,7 @@ decode_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ CUte
         const uint32_t dst = map_to_cluster_rank(recv, (uint32_t)owner) + (uint32_t)((rank * wide + pos) * a.M * 4);
         const uint32_t dbar = map_to_cluster_rank(bar_recv, (uint32_t)owner);
         constexpr uint32_t kSumItem = SUB * NX * 4;
+        const uint32_t no_bits = (uint32_t)warp >> 8;       // 0, which the compiler cannot know
         uint32_t mb = 0, mph = 0, sd = 0, dph = 0;
         for (int pi = 0; pi < n_panels; ++pi) {
             uint64_t run = 0;
@@ -647,8 +649,10 @@ decode_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ CUte
                     sum_at += P * kSumItem;
                     if (++sd == ND) { sd = 0; dph ^= 1u; }
                 }
+                // The buffer's next copies must not overtake the loads above.  The arrival's address takes a zero out of the sums, into
+                // which all that was loaded has gone.  (A fence, here or in front of the copies: groups of 32 1 to 2 % slower.)
                 __syncwarp();
-                if (lane == 0) mbar_arrive(bar_mempty + 8 * mb);
+                if (lane == 0) mbar_arrive(bar_mempty + 8 * mb + ((uint32_t)run & no_bits));
                 if (++mb == kDecodeMetaBufs) { mb = 0; mph ^= 1u; }
             }
             // ---- send the panel's sums to the columns' owners

@@ -1702,7 +1702,7 @@ def random_layers(kind, gs, layers, seed):
 
 
 @pytest.mark.parametrize("M,kind,gs,rounds", [
-    (3, "fp16", 128, 400), (4, "fp16", 128, 400), (8, "fp16", 128, 400),
+    (3, "fp16", 128, 400), (4, "fp16", 128, 400), (8, "fp16", 128, 400), (1, "fp16", 128, 400), (2, "fp16", 128, 400), (1, "fp16", 64, 100), (2, "fp16", 32, 100),
     (16, "fp16", 128, 100), (12, "fp16", 64, 100), (7, "fp16", 32, 100), (5, "bf16", 128, 100), (13, "bf16", 64, 100), (6, "w8", 128, 100)])
 def test_host_batch_repeats_bit_for_bit(M, kind, gs, rounds, ws):
     """A decode step from host buffers, again and again: every result has the bits of the same call on device buffers.  Every buffer

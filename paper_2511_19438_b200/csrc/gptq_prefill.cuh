@@ -43,11 +43,21 @@ __host__ __device__ constexpr int prefill_acc_columns(int tok) { return tok <= 1
 // item, one of the CTA's last kPrefillSets, has waited for the MMAs of the item an A ring earlier, and two tiles lie behind.
 constexpr int kPrefillMinItems = 4;
 static_assert(2 * kPrefillMinItems + 1 > kPrefillSets + prefill_a_stages(0), "a dequant warp's wait for the last tile's accumulator would be ambiguous");
-constexpr int kPrefillXSlots = 4;            // of x, at most: more gained nothing at 128 rows and less, up to 16 were tried
+// Slots of x, at most.  4096 x 22016 with three / four / eight, us: 64 rows 22.3 / 21.1 / 21.0, 96 rows 24.6 / 22.2 / 22.0; 112 rows
+// 25.7 / 23.0 / 22.8 (five fit), 128 rows 27.1 / 24.4 (four fit).
+constexpr int kPrefillXSlots = 4;
+static_assert(kPrefillXSlots <= kUmmaDoneRing, "x would be requested onto a barrier whose last item has not been multiplied");
 // Weight slots.  A set's parity wait on a slot needs the slot's previous item to be in: with this many that is known, the
 // set's last pass (four items ago) has waited for the MMAs of the item that had its A stage before.  With 8-bit weights
 // (16 KB per slot) five, and the set asks.
 __host__ __device__ constexpr int prefill_w_slots(int tok, bool w8) { return w8 ? 5 : kPrefillSets + prefill_a_stages(tok); }
+// bytes of the epilogue's stage and the weight ring, and x slots of tok * 256 bytes that fit behind them (2 KB: barriers, alignment)
+__host__ __device__ constexpr int prefill_ring_bytes(int tok, bool w8) { return kPrefillStage + prefill_w_slots(tok, w8) * (w8 ? 2 : 1) * kItemWBytes; }
+__host__ __device__ constexpr int prefill_x_slots(int tok, bool w8)
+{
+    const int fit = (227 * 1024 - 2048 - prefill_ring_bytes(tok, w8)) / (tok * 256);
+    return fit < kPrefillXSlots ? fit : kPrefillXSlots;
+}
 
 // 16 lanes x 32 columns of tensor memory as four 8-column groups: r[4 g], r[4 g + 1] are lane T / 4, columns 8 g + 2 (T % 4) and
 // the next one, r[4 g + 2], r[4 g + 3] the same of lane T / 4 + 8 (T: thread of the warp)
@@ -111,6 +121,18 @@ __device__ __forceinline__ uint32_t pack_out16(float2 v)
 // Tiles of at most this many token rows exchange their parts by stores into the owners' shared memory, taller ones by bulk copies
 // (8-bit weights: see prefill_kernel).
 __host__ __device__ constexpr int prefill_push_rows(bool w8) { return w8 ? 64 : 112; }
+// bytes of a sender's part: 128 / S columns of the tile's rows, a column an odd number of 16-byte pieces
+__host__ __device__ constexpr int prefill_part_bytes(int tok, int S) { return kPanel / S * (tok + 4) * 4; }
+// The others' parts land in the epilogue's stage and the weight ring, the own one in the x ring.
+constexpr bool prefill_parts_fit(bool w8)
+{
+    for (int S = 2; S <= 4; S *= 2)
+        for (int tok = 32; tok <= prefill_push_rows(w8); tok += 16)
+            if ((S - 1) * prefill_part_bytes(tok, S) > prefill_ring_bytes(tok, w8) || prefill_part_bytes(tok, S) > prefill_x_slots(tok, w8) * tok * 256)
+                return false;
+    return true;
+}
+static_assert(prefill_parts_fit(false) && prefill_parts_fit(true), "stored parts would run over what a CTA still uses");
 
 struct PrefillArgs {
     const uint8_t *scales, *qzeros;   // tiled
@@ -403,7 +425,7 @@ prefill_kernel(const PrefillArgs a, const __grid_constant__ CUtensorMap w_map, c
             if (is_dq && lane < S) mbar_arrive_release_cluster(map_to_cluster_rank(bar_ready, (uint32_t)lane));
             if (is_dq || is_epi) {
                 const int quads = (rows + 3) >> 2, w_shift = S == 4 ? 5 : 6;
-                const uint32_t pitch = (uint32_t)(tok + 4) * 4, part = W * pitch;         // of a column (an odd number of 16-byte pieces), of a sender
+                const uint32_t pitch = (uint32_t)(tok + 4) * 4, part = (uint32_t)prefill_part_bytes(tok, S);      // of a column, of a sender
                 pdl_wait();
                 decode_wait(bar_dfull, 0, flag);
                 decode_wait_cluster(bar_ready, 0, flag);
@@ -466,12 +488,12 @@ prefill_kernel(const PrefillArgs a, const __grid_constant__ CUtensorMap w_map, c
                 __syncwarp();
                 tc_fence_after_sync();
                 const uint32_t at = park + owner * part + (uint32_t)lc * 4u;
-    #pragma unroll 1
+#pragma unroll 1
                 for (int c0 = 32 * group; c0 < rows; c0 += 32 * n_groups) {
                     uint32_t r[32];
                     tmem_ld_32x32(tmem_base + ((uint32_t)(32 * q) << 16) + c0, r);
                     tmem_wait_ld();
-    #pragma unroll
+#pragma unroll
                     for (int i = 0; i < 32; ++i)
                         if (c0 + i < rows) sts_f32(at + (uint32_t)((c0 + i) * W) * 4u, __uint_as_float(r[i]));
                 }
@@ -732,10 +754,8 @@ inline PrefillPlan plan_prefill(int M, int N, int K, int group_size, int sm_coun
     }
     pl.use = true;
     pl.ctas = pl.S > 1 ? pl.tiles * pl.S : pl.tiles < sm_count ? pl.tiles : sm_count;
-    const int fixed = 2048 + kPrefillStage + prefill_w_slots(pl.tok, w8) * (w8 ? 2 : 1) * kItemWBytes, x_slot = pl.tok * 256;
-    pl.x_slots = (227 * 1024 - fixed) / x_slot;
-    if (pl.x_slots > kPrefillXSlots) pl.x_slots = kPrefillXSlots;
-    pl.smem_bytes = fixed + pl.x_slots * x_slot;
+    pl.x_slots = prefill_x_slots(pl.tok, w8);
+    pl.smem_bytes = 2048 + prefill_ring_bytes(pl.tok, w8) + pl.x_slots * pl.tok * 256;
     const int floor_one_per_sm = (227 * 1024) / 2 + 512;                 // the CTA owns all tensor memory
     if (pl.smem_bytes < floor_one_per_sm) pl.smem_bytes = floor_one_per_sm;
     return pl;

@@ -1529,14 +1529,10 @@ def test_gather_of_few_rows(K, M, ws):
 
 
 # ------------------------------------------------------------------------------- 8-bit weights joined in the tcgen05 kernel
-@pytest.mark.parametrize("K,N,gs", [(384, 256, 128), (384, 256, 64), (256, 128, 32), (2048, 4864, 128)])
-@pytest.mark.parametrize("M", [17, 33, 64, 65, 129, 257])
-def test_w8_token_tiles(K, N, gs, M, ws):
-    """Every token tile of the 8-bit tcgen05 kernel at its edges, odd numbers of K groups, split-K clusters; each weight is
-    rounded to fp16 once, so per output the error has standard deviation (2^-11 / sqrt 3) sqrt(sum x^2 w^2), of which eight
-    are allowed, plus the output's rounding."""
-    L = wl.make_linear_w8(K, N, seed=wl.seed_for("w8-tiles", K, N, gs), group_size=gs, act_order=True)
-    x = wl.make_x(M, K, wl.seed_for("w8-tiles-x", M, K))
+def check_w8_rounding(L, M, gs, ws):
+    """An 8-bit layer on a tcgen05 kernel: each weight is rounded to fp16 once, so per output the error has standard deviation
+    (2^-11 / sqrt 3) sqrt(sum x^2 w^2), of which eight are allowed, plus the output's rounding."""
+    x = wl.make_x(M, L.K, wl.seed_for("w8-tiles-x", M, L.K))
     D = H.upload_and_repack_w8(L)
     H.ensure_for_w8(ws, M, D)
     y = H.gemm_w8(H.to_device(x), D).cpu().numpy().astype(np.float64)
@@ -1548,6 +1544,13 @@ def test_w8_token_tiles(K, N, gs, M, ws):
     bound = 8 * sigma + 2.0 ** -11 * np.abs(want) + 1e-3
     err = np.abs(y - want)
     assert np.all(err[finite] <= bound[finite]), (err[finite] / bound[finite]).max()
+
+
+@pytest.mark.parametrize("K,N,gs", [(384, 256, 128), (384, 256, 64), (256, 128, 32), (2048, 4864, 128)])
+@pytest.mark.parametrize("M", [17, 33, 64, 65, 129, 257])
+def test_w8_token_tiles(K, N, gs, M, ws):
+    """Every token tile of the 8-bit tcgen05 kernel at its edges, odd numbers of K groups, split-K clusters."""
+    check_w8_rounding(wl.make_linear_w8(K, N, seed=wl.seed_for("w8-tiles", K, N, gs), group_size=gs, act_order=True), M, gs, ws)
 
 
 # ------------------------------------------------------------------------------- persistent tcgen05 kernel
@@ -1573,18 +1576,44 @@ def test_prefill_kernel(K, N, gs, act, zm1, M, ws):
     assert B.gptq_check_status() == B.GPTQ_OK
 
 
-@pytest.mark.parametrize("K,N", [(2048, 1024), (4096, 5120)])      # clusters of four, of two
-@pytest.mark.parametrize("M", [18, 63, 112, 113])                  # rows no multiple of four; the tallest tile that stores its parts; two tiles, or a taller one
-def test_prefill_kernel_exchanges_parts(K, N, M, ws):
+def assert_exchange(M, N, K, gs, eight_bit, cluster, tallest_stored, stored):
+    """A tile's K range is shared by `cluster` CTAs, and their parts are stored into the owners' memory (or else copied)."""
+    st, pl = B.gptq_plan_prefill(M, N, K, gs, 0, eight_bit, 148)
+    assert st == B.GPTQ_OK and pl.cluster_size == cluster, "the planner no longer splits this shape so: choose another"
+    assert (pl.m_tile <= tallest_stored) == stored, "the planner chose another tile: choose another row count"
+
+
+# rows no multiple of four, the tallest tile that stores its parts, two tiles of 64, the lowest tiles that copy them, odd rows there
+@pytest.mark.parametrize("K,N,cluster,M,stored", [(2048, 1024, 4, M, True) for M in (18, 63, 112, 113)] + [(4096, 4096, 4, M, False) for M in (113, 139)] +
+                         [(4096, 5120, 2, M, True) for M in (18, 63, 112)] + [(4096, 5120, 2, M, False) for M in (113, 139)])
+def test_prefill_kernel_exchanges_parts(K, N, cluster, M, stored, ws):
     """A tile's K range shared by a cluster: both ways of exchanging the partial sums, with the plain and bias + residual epilogues."""
-    st, pl = B.gptq_plan_prefill(M, N, K, 128, 0, 0, 148)
-    assert st == B.GPTQ_OK and pl.cluster_size > 1, "the planner no longer splits this shape: choose another"
+    assert_exchange(M, N, K, 128, 0, cluster, 112, stored)
     L = wl.make_linear(K, N, seed=wl.seed_for("prefill-parts", K, N))
     x_np = wl.make_x(M, K, wl.seed_for("prefill-parts-x", M, K))
     y, _ = run_gemm(L, x_np, ws)
     assert_close(y, oracle.gemm_f64(x_np, L.qweight, L.qzeros, L.scales, None, 128), K, M)
     check_bias_residual(L, M, ws, True, True)
     assert B.gptq_check_status() == B.GPTQ_OK
+
+
+@pytest.mark.parametrize("K,N,cluster", [(4096, 4096, 4), (4096, 5120, 2)])
+@pytest.mark.parametrize("M,gs,stored", [(17, 128, True), (41, 64, True), (63, 32, True), (64, 128, True), (65, 64, False), (127, 32, False)])
+def test_w8_exchanges_parts(K, N, cluster, M, gs, stored, ws):
+    """The same with 8-bit weights, whose tiles store their parts up to 64 rows.  The bound is that of test_w8_token_tiles."""
+    assert_exchange(M, N, K, gs, 1, cluster, 64, stored)
+    check_w8_rounding(wl.make_linear_w8(K, N, seed=wl.seed_for("w8-parts", K, N, gs), group_size=gs), M, gs, ws)
+
+
+@pytest.mark.parametrize("K,N,cluster,M,gs", [(4096, 4096, 4, 23, 64), (4096, 5120, 2, 50, 32), (4096, 4096, 4, 139, 32)])
+def test_bf16_exchanges_parts(K, N, cluster, M, gs, ws):
+    """... and in bfloat16, with groups of 64 and 32."""
+    assert_exchange(M, N, K, gs, 0, cluster, 112, M < 113)
+    L = wl.make_linear(K, N, seed=wl.seed_for("bf16-parts", K, N, gs), group_size=gs)
+    s_bits = wl.make_scales_bf16(K // gs, N, wl.seed_for("bf16-parts-s", K, N, gs))
+    x_bits = wl.make_x_bf16(M, K, wl.seed_for("bf16-parts-x", M))
+    y, _ = run_gemm_bf16(L, s_bits, x_bits, ws)
+    assert_close_bf16(y, oracle.gemm_f64_bf16(x_bits, L.qweight, L.qzeros, s_bits, None, gs), K, M)
 
 
 @pytest.mark.parametrize("M", [17, 31, 64, 130, 300])
@@ -1703,7 +1732,8 @@ def random_layers(kind, gs, layers, seed):
 
 @pytest.mark.parametrize("M,kind,gs,rounds", [
     (3, "fp16", 128, 400), (4, "fp16", 128, 400), (8, "fp16", 128, 400), (1, "fp16", 128, 400), (2, "fp16", 128, 400), (1, "fp16", 64, 100), (2, "fp16", 32, 100),
-    (16, "fp16", 128, 100), (12, "fp16", 64, 100), (7, "fp16", 32, 100), (5, "bf16", 128, 100), (13, "bf16", 64, 100), (6, "w8", 128, 100)])
+    (16, "fp16", 128, 100), (12, "fp16", 64, 100), (7, "fp16", 32, 100), (5, "bf16", 128, 100), (13, "bf16", 64, 100), (6, "w8", 128, 100),
+    (17, "fp16", 128, 50), (64, "fp16", 128, 30), (100, "fp16", 64, 30), (23, "bf16", 32, 30), (40, "w8", 64, 30)])
 def test_host_batch_repeats_bit_for_bit(M, kind, gs, rounds, ws):
     """A decode step from host buffers, again and again: every result has the bits of the same call on device buffers.  Every buffer
     that the step writes is overwritten before each round.  (Weights that are not in the L2 cache and activations that have just come

@@ -233,10 +233,10 @@ __device__ __forceinline__ bool mbar_wait_once(uint32_t bar, uint32_t parity)
 }
 // For the thread that refills a ring: the stage has been handed back by warps that read it with ordinary loads, and the next copy
 // into it goes through the async proxy.  The arrivals alone do not keep that copy behind those loads; the fence on the way from
-// them to the copy does.  Without it the last load of x of an item now and then found what the refill had brought (host batches of
-// 3 to 8 rows, 4096 x 22016: in 0.1 to 0.7 % of the launches the last 32 rows of K of an item were multiplied with the x of the
-// item four on).  In the refilling thread it costs nothing that can be measured, in the reading warps up to 2 % (decode kernel).
-// Where a refill waits for MMAs whose operand was made of what had been loaded, the loads are over anyway.
+// them to the copy does.  Without it the last load of x of an item now and then found what the refill had brought (host batches,
+// 4096 x 22016: in 0.6 % of the launches at 3 and 4 rows, 2.6 % at 8, the last 32 rows of K of an item were multiplied with the x of
+// the item four on; none of 72000 with it).  In the refilling thread it costs nothing that can be measured, in the reading warps up
+// to 2 % (decode kernel).  Where a refill waits for MMAs whose operand was made of what had been loaded, the loads are over anyway.
 __device__ __forceinline__ bool mbar_wait_stage_free(uint32_t bar, uint32_t parity)
 {
     const bool ok = mbar_wait(bar, parity);

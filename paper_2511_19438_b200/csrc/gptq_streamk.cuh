@@ -49,7 +49,8 @@ __host__ __device__ constexpr int token_row_of_slot(int n) { return ((n & 1) << 
 // (128 / group_size: the whole item, a K64 block, or half of one) it reads the scale pair and the zero byte of its
 // columns, turns nibbles into exact fp16 integers q - z (z_add = 1 when the stored zero points are one too small),
 // multiplies them with the stage's x tiles and folds the fp32 group sums into `acc` with the group's scales.
-// The stage may be released once `consume_item` has returned; `fold_item` needs registers only.
+// The stage may be released once `consume_item` has returned (mbar_wait_stage_free keeps its refill behind the loads); `fold_item`
+// needs registers only.
 template <int MT, int SUB>
 struct ItemSums {
     float g[SUB][MT][4];

@@ -119,7 +119,9 @@ __device__ __forceinline__ uint32_t pack_out16(float2 v)
 }
 
 // Tiles of at most this many token rows exchange their parts by stores into the owners' shared memory, taller ones by bulk copies
-// (8-bit weights: see prefill_kernel).
+// (what both take with 4-bit weights: see prefill_kernel).  8-bit weights, copies / stores, us: clusters of four, 4096 x 4096, 17 rows
+// 9.7 / 9.4, 64 rows 12.4 / 12.3, 80 rows 12.8 / 12.7, 96 rows 13.1 / 13.5; 11008 x 4096, 17 to 64 rows the same, 112 rows 22.4 / 23.1;
+// 2048 x 2048, 64 rows 8.1 / 8.0, 112 rows 9.4 / 9.6; clusters of two, 4096 x 5120, 17 rows 12.5 / 11.7, 64 rows 14.9 / 14.7, 112 rows 16.3 / 16.3.
 __host__ __device__ constexpr int prefill_push_rows(bool w8) { return w8 ? 64 : 112; }
 // bytes of a sender's part: 128 / S columns of the tile's rows, a column an odd number of 16-byte pieces
 __host__ __device__ constexpr int prefill_part_bytes(int tok, int S) { return kPanel / S * (tok + 4) * 4; }
